@@ -11,11 +11,15 @@
 // 2 plaquette staples (weight 2 c0) and 6 rectangle staples (weight c1) per direction nu != mu.
 // Output kind 1: G; kind 0: F = TA(U G^dag) (dS/deps = tr(X F) along U -> exp(eps X) U).
 //
-// One thread per link (force) or per site (action), canonical complex128 [4][V][3][3], FP64
-// (the staples are 84 complex 3x3 products per link: GB300's FP64 rate bounds this, not HBM).
+// Canonical complex128 [4][V][3][3]; FP64 forces share their staples between links, FP32 ones are
+// one thread per link over its loops (84 complex 3x3 products).
+#include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 
+#include "dslash.cuh"
+#include "plaq.cuh"
 #include "stg_common.h"
 #include "su3.cuh"
 
@@ -137,6 +141,100 @@ __global__ void __launch_bounds__(kGaugeBlock, 1) k_gauge_force(const __grid_con
     st(a.out, g, mu, x, G);
 }
 
+// ------------------------------------------------------------------ force by shared staples
+// The 2x1 rectangle across link (y, nu) is tr[Sup(nu, mu)(y) Slo(nu, mu)(y-mu)^dag], the product of
+// the link's upper and lower staples (plaq.cuh).  So the rectangle part of the force is the plaquette
+// part with one link of the plaquette replaced by its staple on the outer side:
+//   P'(mu, nu)(x) = Slo(nu, mu)(x-mu) U_mu(x+nu) + U_nu(x) Sup(mu, nu)(x+nu)
+//   G_mu(x) = sum_nu  wp Sup(mu, nu)(x) + wr [ P'(mu, nu)(x) U_nu(x+mu)^dag + P(mu, nu)(x) Sup(nu, mu)(x+mu)^dag ]
+//                   + wp Slo(mu, nu)(y) + wr [ U_nu(y)^dag P'(nu, mu)(y) + Slo(nu, mu)(y-mu)^dag P(nu, mu)(y) ]
+// with y = x - nu.  Three products per ordered pair for P, Sup, Slo (k_gauge_staples), two for P'
+// (k_gauge_bent), four per link and nu for G (k_gauge_gather): 27 products per link where the loops
+// one by one take 84 (k_gauge_force), for 4 matrices of workspace per pair and site.
+// Bound by the FP64 pipe: 18x22x14x26 8.73 -> 3.02 ms (2970 multiply-adds per link at 0.57e12/s),
+// 24^4 20.0 -> 6.93 ms, 4^4 317 -> 77 us.  One warp per block: the pipe is per quarter SM and one warp
+// keeps it busy, so small lattices spread best in single warps (6^4: 98 us against 123 us with four).
+constexpr int kPlaqBlock = 32;
+
+template <typename T>
+struct GaugePlaqArgs {
+    using C = typename C2<T>::type;
+    plaq::PlaqGeo g;
+    const C *U;
+    C *P, *Sup, *Slo, *Pb;  // one field per ordered pair of the planes [p0, p1)
+    C *out;
+    T wp, wr;
+    int p0, p1;  // planes of this pass
+    int first, last, kind;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kPlaqBlock) k_gauge_staples(const __grid_constant__ GaugePlaqArgs<T> a)
+{
+    using namespace plaq;
+    pdl_enter();
+    const int x = blockIdx.x * kPlaqBlock + threadIdx.x;
+    if (x >= a.g.V) return;
+    int mu, nu;
+    plane_dirs(a.p0 + (blockIdx.y >> 1), mu, nu);
+    if (blockIdx.y & 1) { const int t = mu; mu = nu; nu = t; }
+    const int f = blockIdx.y;
+    const M3T<T> p = mul<false, false>(link_at<T>(a.U, a.g, nu, x), link_at<T>(a.U, a.g, mu, up(a.g, x, nu)));
+    ws_st(a.P, a.g.V, f, x, p);
+    ws_st(a.Sup, a.g.V, f, x, mul<false, true>(p, link_at<T>(a.U, a.g, nu, up(a.g, x, mu))));
+    ws_st(a.Slo, a.g.V, f ^ 1, x, mul<true, false>(link_at<T>(a.U, a.g, mu, x), p));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kPlaqBlock) k_gauge_bent(const __grid_constant__ GaugePlaqArgs<T> a)
+{
+    using namespace plaq;
+    pdl_enter();
+    const int x = blockIdx.x * kPlaqBlock + threadIdx.x;
+    if (x >= a.g.V) return;
+    int mu, nu;
+    plane_dirs(a.p0 + (blockIdx.y >> 1), mu, nu);
+    if (blockIdx.y & 1) { const int t = mu; mu = nu; nu = t; }
+    const int f = blockIdx.y, xn = up(a.g, x, nu);
+    M3T<T> p = mul<false, false>(ws_ld<T>(a.Slo, a.g.V, f ^ 1, down(a.g, x, mu)), link_at<T>(a.U, a.g, mu, xn));
+    mul_acc<false, false>(p, link_at<T>(a.U, a.g, nu, x), ws_ld<T>(a.Sup, a.g.V, f, xn));
+    ws_st(a.Pb, a.g.V, f, x, p);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kPlaqBlock) k_gauge_gather(const __grid_constant__ GaugePlaqArgs<T> a)
+{
+    using namespace plaq;
+    pdl_enter();
+    const int mu = blockIdx.y, x = blockIdx.x * kPlaqBlock + threadIdx.x;
+    if (x >= a.g.V) return;
+    const int V = a.g.V, xm = up(a.g, x, mu);
+    M3T<T> G = zero3<T>(), R = zero3<T>();
+    if (!a.first) G = link_at<T>(a.out, a.g, mu, x);
+#pragma unroll 1
+    for (int nu = 0; nu < 4; ++nu) {
+        if (nu == mu) continue;
+        const int p = plane_of(mu, nu);
+        if (p < a.p0 || p >= a.p1) continue;
+        const int f = slot_of(mu, nu) - 2 * a.p0;  // pair (mu, nu); (nu, mu) is f ^ 1
+        const int y = down(a.g, x, nu), ym = down(a.g, y, mu);
+        axpy3(G, a.wp, ws_ld<T>(a.Sup, V, f, x));
+        axpy3(G, a.wp, ws_ld<T>(a.Slo, V, f, y));
+        mul_acc<false, true>(R, ws_ld<T>(a.Pb, V, f, x), link_at<T>(a.U, a.g, nu, xm));
+        mul_acc<false, true>(R, ws_ld<T>(a.P, V, f, x), ws_ld<T>(a.Sup, V, f ^ 1, xm));
+        mul_acc<true, false>(R, link_at<T>(a.U, a.g, nu, y), ws_ld<T>(a.Pb, V, f ^ 1, y));
+        mul_acc<true, false>(R, ws_ld<T>(a.Slo, V, f ^ 1, ym), ws_ld<T>(a.P, V, f ^ 1, y));
+    }
+    axpy3(G, a.wr, R);
+    if (a.last && a.kind == 0) G = expand_anti_traceless(anti_mul<false, true>(link_at<T>(a.U, a.g, mu, x), G));
+    typename C2<T>::type *o = a.out + ((long long)mu * V + x) * 9;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        o[k].x = G.m[k / 3][k % 3].re;
+        o[k].y = G.m[k / 3][k % 3].im;
+    }
+}
+
 __global__ void __launch_bounds__(kGaugeBlock, 1) k_gauge_action(const __grid_constant__ GaugeArgs<double> a)
 {
     __shared__ double sh[33];
@@ -206,10 +304,64 @@ bool misaligned(const void *p) { return p == nullptr || (reinterpret_cast<uintpt
 
 using namespace stg;
 
+// Workspace of the shared-staple force: as many planes per pass as fit kGaugeWorkspace (all 6 up to
+// 24^4 in FP64), at least one.  Returns false (nothing launched) when the pool has no room for even
+// one plane.
+constexpr size_t kGaugeWorkspace = (size_t)4 << 30;
+
+template <typename T>
+static bool gauge_force_plaq(const stg_lattice *lat, double beta, const void *links, void *out, int kind,
+                             cudaStream_t st, cudaError_t &err)
+{
+    using C = typename C2<T>::type;
+    if (lat->V > INT_MAX) return false;
+    GaugePlaqArgs<T> a;
+    memset(&a, 0, sizeof(a));
+    a.g = plaq::plaq_geo(lat->g);
+    a.U = static_cast<const C *>(links);
+    a.out = static_cast<C *>(out);
+    a.wp = T(-beta / 3.0 * 2.0 * kC0);
+    a.wr = T(-beta / 3.0 * kC1);
+    a.kind = kind;
+    const size_t field = (size_t)9 * a.g.V, per_plane = 8 * field * sizeof(C);
+    int np = (int)std::min<size_t>(6, std::max<size_t>(1, kGaugeWorkspace / per_plane));
+    C *ws = nullptr;
+    keep_pool_mapped(st);
+    err = cudaMallocAsync((void **)&ws, np * per_plane, st);
+    if (err != cudaSuccess && np > 1) {
+        cudaGetLastError();
+        np = 1;
+        err = cudaMallocAsync((void **)&ws, per_plane, st);
+    }
+    if (err != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    a.P = ws;
+    a.Sup = ws + 2 * np * field;
+    a.Slo = ws + 4 * np * field;
+    a.Pb = ws + 6 * np * field;
+    const unsigned nb = (unsigned)((a.g.V + kPlaqBlock - 1) / kPlaqBlock);
+    for (int p = 0; p < 6 && err == cudaSuccess; p += np) {
+        a.p0 = p;
+        a.p1 = std::min(6, p + np);
+        a.first = p == 0;
+        a.last = a.p1 == 6;
+        const dim3 pairs(nb, 2 * (a.p1 - a.p0));
+        err = launch_pdl(k_gauge_staples<T>, pairs, dim3(kPlaqBlock), st, a);
+        if (err == cudaSuccess) err = launch_pdl(k_gauge_bent<T>, pairs, dim3(kPlaqBlock), st, a);
+        if (err == cudaSuccess) err = launch_pdl(k_gauge_gather<T>, dim3(nb, 4), dim3(kPlaqBlock), st, a);
+    }
+    const cudaError_t f = cudaFreeAsync(ws, st);
+    if (err == cudaSuccess) err = f;
+    return true;
+}
+
 template <typename T>
 static cudaError_t gauge_force_t(const stg_lattice *lat, double beta, const void *links, void *out, int kind,
                                  cudaStream_t st)
 {
+    cudaError_t err = cudaSuccess;
     GaugeArgs<T> a;
     memset(&a, 0, sizeof(a));
     a.g = link_geo(lat->g);
@@ -217,6 +369,9 @@ static cudaError_t gauge_force_t(const stg_lattice *lat, double beta, const void
     a.U = static_cast<const typename C2<T>::type *>(links);
     a.out = static_cast<typename C2<T>::type *>(out);
     a.kind = kind;
+    // FP64: the shared staples wherever they fit (figures at the kernels).
+    // FP32: the loops one by one, which need no workspace traffic (32^4: 2.79 ms against 2.77 ms shared)
+    if (sizeof(T) == 8 && gauge_force_plaq<T>(lat, beta, links, out, kind, st, err)) return err;
     const dim3 grid((unsigned)((a.g.V + kGaugeBlock - 1) / kGaugeBlock), 4);
     k_gauge_force<T><<<grid, kGaugeBlock, 0, st>>>(a);
     return cudaGetLastError();

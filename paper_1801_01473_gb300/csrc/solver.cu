@@ -982,18 +982,7 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
         }
     const int vb = Field<R>::kBytesPerSite;
 
-    // The workspace comes from the device's default stream-ordered memory pool.  Keep up to
-    // 64 GiB of freed pool memory mapped between solves (the default threshold of 0 returns it at
-    // every synchronisation and the next solve pays for mapping it again).
-    {
-        int dev = 0;
-        cudaMemPool_t pool;
-        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
-            uint64_t thr = 64ull << 30;
-            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
-        }
-        cudaGetLastError();
-    }
+    keep_pool_mapped(user_st);  // the workspace comes from the default stream-ordered pool
     const bool verbose = getenv("STG_VERBOSE") && getenv("STG_VERBOSE")[0] == '1';
     auto t_start = std::chrono::steady_clock::now();
     auto stamp = [&](const char *what) {

@@ -60,6 +60,11 @@ stg_status f32_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge 
 // gauge): the operator of the mixed solver's FP64-accurate residuals, run on the FP32 pipes.
 stg_status ds_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge **out);
 
+// Sets the release threshold of the device's default stream-ordered memory pool to 64 GiB, so that
+// freed workspaces stay mapped between calls (the default threshold of 0 returns them at every
+// synchronisation and the next call pays for mapping them again).  Does nothing while `st` captures.
+void keep_pool_mapped(cudaStream_t st);
+
 // Error reporting (thread-local message read by stg_last_error).
 stg_status set_error(stg_status s, const std::string &msg);
 stg_status cuda_error(cudaError_t e, const char *where);

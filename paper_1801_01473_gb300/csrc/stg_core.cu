@@ -64,6 +64,19 @@ cudaError_t launch_dslash_bs(int kind, const DArgs &a, int mode, int bs, cudaStr
     return cudaErrorInvalidValue;
 }
 
+void keep_pool_mapped(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    int dev = 0;
+    cudaMemPool_t pool;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+        cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
+        uint64_t thr = 64ull << 30;
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
+    }
+    cudaGetLastError();
+}
+
 bool pdl_enabled()
 {
     static const bool on = [] {
