@@ -186,5 +186,235 @@ __device__ __forceinline__ M3T<T> expand_anti_traceless(const H9<T> &z)
     return y;
 }
 
+// Workspace of 9-number matrices: field f holds [9][V] reals (diagonal, then re, im of the triangle).
+template <typename T>
+__device__ __forceinline__ H9<T> ws_ld9(const T *__restrict__ base, int V, int f, int i)
+{
+    const T *p = base + (long long)f * 9 * V + i;
+    T v[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) v[k] = p[(long long)k * V];
+    H9<T> z;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        z.d[k] = v[k];
+        z.o[k] = cx<T>{v[3 + 2 * k], v[4 + 2 * k]};
+    }
+    return z;
+}
+template <typename T>
+__device__ __forceinline__ void ws_st9(T *__restrict__ base, int V, int f, int i, const H9<T> &z)
+{
+    T *p = base + (long long)f * 9 * V + i;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        p[(long long)k * V] = z.d[k];
+        p[(long long)(3 + 2 * k) * V] = z.o[k].re;
+        p[(long long)(4 + 2 * k) * V] = z.o[k].im;
+    }
+}
+
+// z += w a
+template <typename T>
+__device__ __forceinline__ void axpy9(H9<T> &z, T w, const H9<T> &a)
+{
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        z.d[k] = fma(w, a.d[k], z.d[k]);
+        z.o[k].re = fma(w, a.o[k].re, z.o[k].re);
+        z.o[k].im = fma(w, a.o[k].im, z.o[k].im);
+    }
+}
+
+// acc += w b for an anti-Hermitian w (90 multiply-adds)
+template <typename T>
+__device__ __forceinline__ void anti_mul_acc(M3T<T> &acc, const H9<T> &w, const M3T<T> &b)
+{
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            acc.m[r][c].re = fma(-w.d[r], b.m[r][c].im, acc.m[r][c].re);
+            acc.m[r][c].im = fma(w.d[r], b.m[r][c].re, acc.m[r][c].im);
+        }
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            const int r = e == 2 ? 1 : 0, k = e == 0 ? 1 : 2;
+            cmac(acc.m[r][c], w.o[e], b.m[k][c]);
+            cmac_conj(acc.m[k][c], cx<T>{-w.o[e].re, -w.o[e].im}, b.m[r][c]);
+        }
+    }
+}
+
+// square of a Hermitian matrix
+template <typename T>
+__device__ __forceinline__ H9<T> square9(const H9<T> &q)
+{
+    const T n01 = q.o[0].re * q.o[0].re + q.o[0].im * q.o[0].im, n02 = q.o[1].re * q.o[1].re + q.o[1].im * q.o[1].im,
+            n12 = q.o[2].re * q.o[2].re + q.o[2].im * q.o[2].im;
+    H9<T> s;
+    s.d[0] = fma(q.d[0], q.d[0], n01 + n02);
+    s.d[1] = fma(q.d[1], q.d[1], n01 + n12);
+    s.d[2] = fma(q.d[2], q.d[2], n02 + n12);
+    const T t01 = q.d[0] + q.d[1], t02 = q.d[0] + q.d[2], t12 = q.d[1] + q.d[2];
+    s.o[0] = cx<T>{t01 * q.o[0].re, t01 * q.o[0].im};
+    cmac_conj(s.o[0], q.o[2], q.o[1]);  // q02 conj(q12)
+    s.o[1] = cx<T>{t02 * q.o[1].re, t02 * q.o[1].im};
+    cmac(s.o[1], q.o[0], q.o[2]);
+    s.o[2] = cx<T>{t12 * q.o[2].re, t12 * q.o[2].im};
+    cmac_conj(s.o[2], q.o[0], q.o[1]);  // conj(q01) q02
+    return s;
+}
+
+// q n + n q of two Hermitian matrices
+template <typename T>
+__device__ __forceinline__ H9<T> anticommutator9(const H9<T> &q, const H9<T> &n)
+{
+    T p[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) p[k] = fma(q.o[k].re, n.o[k].re, q.o[k].im * n.o[k].im);
+    H9<T> s;
+    s.d[0] = T(2) * fma(q.d[0], n.d[0], p[0] + p[1]);
+    s.d[1] = T(2) * fma(q.d[1], n.d[1], p[0] + p[2]);
+    s.d[2] = T(2) * fma(q.d[2], n.d[2], p[1] + p[2]);
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        const int r = e == 2 ? 1 : 0, c = e == 0 ? 1 : 2;
+        const T tq = q.d[r] + q.d[c], tn = n.d[r] + n.d[c];
+        s.o[e].re = fma(tq, n.o[e].re, tn * q.o[e].re);
+        s.o[e].im = fma(tq, n.o[e].im, tn * q.o[e].im);
+    }
+    cmac_conj(s.o[0], n.o[2], q.o[1]);  // q02 conj(n12)
+    cmac_conj(s.o[0], q.o[2], n.o[1]);  // n02 conj(q12)
+    cmac(s.o[1], q.o[0], n.o[2]);
+    cmac(s.o[1], n.o[0], q.o[2]);
+    cmac_conj(s.o[2], q.o[0], n.o[1]);
+    cmac_conj(s.o[2], n.o[0], q.o[1]);
+    return s;
+}
+
+// c0 = det q and c1 = tr q^2 / 2 of a Hermitian q with square q2
+template <typename T>
+__device__ __forceinline__ void char_coefs9(const H9<T> &q, const H9<T> &q2, T &c0, T &c1)
+{
+    c1 = T(0.5) * (q2.d[0] + q2.d[1] + q2.d[2]);
+    // det q = Re of the expansion along the first row, q10 = conj(q01) and so on
+    const T n01 = q.o[0].re * q.o[0].re + q.o[0].im * q.o[0].im, n02 = q.o[1].re * q.o[1].re + q.o[1].im * q.o[1].im,
+            n12 = q.o[2].re * q.o[2].re + q.o[2].im * q.o[2].im;
+    const cx<T> t = cmul(q.o[0], q.o[2]);  // q01 q12, to be taken with q20 = conj(q02)
+    const T re = fma(t.re, q.o[1].re, t.im * q.o[1].im);
+    c0 = fma(q.d[0], fma(q.d[1], q.d[2], -n12), fma(T(2), re, -fma(q.d[1], n02, q.d[2] * n01)));
+}
+
+// 1/n!, n = 0..131
+template <typename T>
+struct InvFactorial {
+    T v[132];
+    constexpr InvFactorial() : v{}
+    {
+        double f = 1.0;
+        for (int n = 0; n < 132; ++n) {
+            v[n] = f < (sizeof(T) == 4 ? 1e-37 : 0.0) ? T(0) : (T)f;
+            f /= n + 1;
+        }
+    }
+};
+__constant__ constexpr InvFactorial<double> kInvFactorial64{};
+__constant__ constexpr InvFactorial<float> kInvFactorial32{};
+template <typename T>
+__device__ __forceinline__ T inv_factorial(int n)
+{
+    return sizeof(T) == 8 ? (T)kInvFactorial64.v[n] : (T)kInvFactorial32.v[n];
+}
+
+// exp(iQ) = f0 + f1 Q + f2 Q^2 with the derivatives of the f_j, as exp_coef, from one sequence.
+// Q^3 = c1 Q + c0 gives Q^n = c0 h_{n-1} + h_{n+1} Q + h_n Q^2 (n >= 1) with
+//   h_0 = h_1 = 0, h_2 = 1, h_{n+1} = c1 h_{n-1} + c0 h_{n-2},
+// and g_n = dh_n/dc0 satisfies dh_n/dc1 = g_{n+1} (both from the generating function
+// t^2 / (1 - c1 t^2 - c0 t^3)), g_{n+1} = c1 g_{n-1} + c0 g_{n-2} + h_{n-2}.  So with s_n = i^n / n!
+//   f2 = sum s_n h_n, f1 = sum s_n h_{n+1}, f0 = 1 + c0 sum s_n h_{n-1},
+//   df2/dc0 = sum s_n g_n,  df2/dc1 = df1/dc0 = sum s_n g_{n+1},  df1/dc1 = sum s_n g_{n+2},
+//   df0/dc0 = sum s_n h_{n-1} + c0 sum s_n g_{n-1},  df0/dc1 = c0 df2/dc0:
+// 5 (12 with derivatives) multiply-adds per term, no divisions; the number of terms is settled
+// beforehand in FP32 by exp_coef's bound.
+template <bool DERIV, typename T>
+__device__ __forceinline__ ExpCoefT<T> exp_sums(T c0, T c1)
+{
+    int nmax = 6;
+    {
+        const float stop = sizeof(T) == 4 ? 1e-9f : 1e-18f;
+        float r = sqrtf(fmaxf(2.f * (float)c1, 0.f));
+        if (!(r >= 1.f)) r = 1.f;
+        float bound = 1.f;  // r^n / n!
+        for (int n = 1; n < 128; ++n) {
+            bound *= __fdividef(r, (float)n);
+            const float m = (float)(n + 1);
+            nmax = n;
+            if (n >= 6 && bound * m * m * m < stop) break;
+        }
+    }
+    T hm = T(0), h = T(0), hp = T(1);               // h_{n-1}, h_n, h_{n+1} at n = 1
+    T gm = T(0), g = T(0), gp = T(0), gpp = T(0);               // g_{n-1}, g_n, g_{n+1}, g_{n+2}
+    T s0[2] = {T(0), T(0)}, s1[2] = {T(0), T(0)}, s2[2] = {T(0), T(0)};  // sums of h_{n-1}, h_n, h_{n+1}; [1] odd n
+    T d0[2] = {T(0), T(0)}, d1[2] = {T(0), T(0)}, d2[2] = {T(0), T(0)}, d3[2] = {T(0), T(0)};  // g_{n-1} .. g_{n+2}
+#pragma unroll 1
+    for (int n0 = 1; n0 <= nmax; n0 += 4) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {  // n = n0 + u = 1 + u mod 4: i^n = i, -1, -i, 1
+            T s = inv_factorial<T>(n0 + u);
+            if (u == 1 || u == 2) s = -s;
+            const int o = (u & 1) ? 0 : 1;
+            s0[o] = fma(s, hm, s0[o]);
+            s1[o] = fma(s, h, s1[o]);
+            s2[o] = fma(s, hp, s2[o]);
+            if (DERIV) {
+                d0[o] = fma(s, gm, d0[o]);
+                d1[o] = fma(s, g, d1[o]);
+                d2[o] = fma(s, gp, d2[o]);
+                d3[o] = fma(s, gpp, d3[o]);
+                const T gn = fma(c1, gp, fma(c0, g, h));  // g_{n+3}
+                gm = g; g = gp; gp = gpp; gpp = gn;
+            }
+            const T hn = fma(c1, h, c0 * hm);  // h_{n+2}
+            hm = h; h = hp; hp = hn;
+        }
+    }
+    ExpCoefT<T> e;
+    e.f[0] = cx<T>{fma(c0, s0[0], T(1)), c0 * s0[1]};
+    e.f[1] = cx<T>{s2[0], s2[1]};
+    e.f[2] = cx<T>{s1[0], s1[1]};
+    if (DERIV) {
+        e.d0[0] = cx<T>{fma(c0, d0[0], s0[0]), fma(c0, d0[1], s0[1])};
+        e.d0[1] = cx<T>{d2[0], d2[1]};
+        e.d0[2] = cx<T>{d1[0], d1[1]};
+        e.d1[0] = cx<T>{c0 * d1[0], c0 * d1[1]};
+        e.d1[1] = cx<T>{d3[0], d3[1]};
+        e.d1[2] = cx<T>{d2[0], d2[1]};
+    }
+    return e;
+}
+
+// f0 + f1 q + f2 q2 of Hermitian q, q2
+template <typename T>
+__device__ __forceinline__ M3T<T> poly9(const cx<T> f[3], const H9<T> &q, const H9<T> &q2)
+{
+    M3T<T> e;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+        e.m[r][r] = cx<T>{fma(f[1].re, q.d[r], fma(f[2].re, q2.d[r], f[0].re)),
+                          fma(f[1].im, q.d[r], fma(f[2].im, q2.d[r], f[0].im))};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int r = k == 2 ? 1 : 0, c = k == 0 ? 1 : 2;
+        cx<T> v = cmul(f[1], q.o[k]);
+        cmac(v, f[2], q2.o[k]);
+        e.m[r][c] = v;
+        v = cmul(f[1], cconj(q.o[k]));
+        cmac(v, f[2], cconj(q2.o[k]));
+        e.m[c][r] = v;
+    }
+    return e;
+}
+
 }  // namespace plaq
 }  // namespace stg

@@ -16,12 +16,16 @@
 // and k_stout_back_staples (per link: adds the product-rule terms of every staple of the other
 // links' C that contains this link, gathered from Y -- each output is written by one thread).
 //
-// Layout: canonical complex128 [4][V][3][3] (site index x + Lx (y + Ly (z + Lz t))); one thread
-// per link.  All arithmetic FP64 (GB300's FP64 rate bounds these kernels, not HBM).
+// Layout: canonical complex128 or complex64 [4][V][3][3] (site index x + Lx (y + Ly (z + Lz t))); one
+// thread per link.  FP64 steps mostly go by shared plaquettes (further down).
+#include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <string>
 
+#include "dslash.cuh"
+#include "plaq.cuh"
 #include "stg_common.h"
 #include "su3.cuh"
 
@@ -229,6 +233,242 @@ __global__ void __launch_bounds__(kStoutBlock) k_lie_force(const __grid_constant
     st(a.out, a.g, mu, i, ta(mul<false, true>(u, gr)));
 }
 
+// ------------------------------------------------------------------ by shared plaquettes
+// The same step with every corner path made once per plaquette (plaq.cuh).  C U^dag is a sum over
+// the plaquettes of the link of closed loops at its start: for the upper plaquette of (x, mu)
+// P(mu, nu) P(nu, mu)^dag, whose anti-Hermitian part serves link (x, nu) with the opposite sign; for
+// the lower one Slo(mu, nu)(x-nu) U_mu(x)^dag.  Only the anti-Hermitian parts are needed (9 numbers).
+//
+// Chain rule: with W = rho G_Omega of every link fixed, dS is the change of Re tr of the plaquettes
+// when each link moves by Y = W U, so the gradient has the form of the rectangle force, with
+//   P'(mu, nu)(x) = (W_nu - W_mu)(x) P(mu, nu)(x) + U_nu(x) Y_mu(x+nu)
+//   G_mu(x) = E^dag G' + sum_nu [ P'(mu, nu)(x) U_nu(x+mu)^dag + P(mu, nu)(x) Y_nu(x+mu)^dag
+//                               + U_nu(y)^dag P'(nu, mu)(y) ] - W_mu(x) sum_nu Slo(mu, nu)(y),  y = x - nu.
+//
+// ~1450 FP64 multiply-adds per link and smearing step (k_stout_fwd ~2300) and ~3700 per step of the
+// chain rule (k_stout_back_* ~6850), both at the FP64 pipe's rate (0.58e12/s): two steps of 16^3x32
+// 4.59 -> 2.65 ms, of the chain rule on 20x12x28x16 10.7 -> 5.7 ms.
+template <typename T>
+struct StoutPlaqArgs {
+    using C = typename C2<T>::type;
+    plaq::PlaqGeo g;
+    T rho;
+    const C *U;    // links of this step
+    const C *G;    // gradient of the step's output (backward)
+    C *out;        // smeared links / gradient of U
+    T *K, *Lo;     // anti-Hermitian loops: upper per plane [6], lower per ordered pair [12] (based at x)
+    C *P, *Slo, *Pb;  // per ordered pair [12] (backward)
+    T *W;          // [4] rho G_Omega, anti-Hermitian
+    C *Y;          // [4] W U
+    const C *proj;  // last step of kind 0: the links for F = TA(U G^dag); null otherwise
+};
+
+template <bool BWD, typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_loops(const __grid_constant__ StoutPlaqArgs<T> a)
+{
+    using namespace plaq;
+    pdl_enter();
+    const int x = blockIdx.x * kStoutBlock + threadIdx.x, V = a.g.V;
+    if (x >= V) return;
+    const int p = blockIdx.y;
+    int m, n;
+    plane_dirs(p, m, n);
+    const int xm = up(a.g, x, m), xn = up(a.g, x, n);
+    const M3T<T> pmn = mul<false, false>(link_at<T>(a.U, a.g, n, x), link_at<T>(a.U, a.g, m, xn));
+    const M3T<T> pnm = mul<false, false>(link_at<T>(a.U, a.g, m, x), link_at<T>(a.U, a.g, n, xm));
+    if (BWD) {
+        ws_st(a.P, V, 2 * p, x, pmn);
+        ws_st(a.P, V, 2 * p + 1, x, pnm);
+    }
+    ws_st9(a.K, V, p, x, anti_mul<false, true>(pmn, pnm));
+    M3T<T> s = mul<true, false>(link_at<T>(a.U, a.g, n, x), pnm);  // Slo(m, n): of link (x+n, m)
+    if (BWD) ws_st(a.Slo, V, 2 * p, x, s);
+    ws_st9(a.Lo, V, 2 * p, x, anti_mul<false, true>(s, link_at<T>(a.U, a.g, m, xn)));
+    s = mul<true, false>(link_at<T>(a.U, a.g, m, x), pmn);  // Slo(n, m): of link (x+m, n)
+    if (BWD) ws_st(a.Slo, V, 2 * p + 1, x, s);
+    ws_st9(a.Lo, V, 2 * p + 1, x, anti_mul<false, true>(s, link_at<T>(a.U, a.g, n, xm)));
+}
+
+// Q = -i TA(C U^dag) of link (x, mu) from its loops
+template <typename T>
+__device__ __forceinline__ plaq::H9<T> loops_q(const StoutPlaqArgs<T> &a, int mu, int x)
+{
+    using namespace plaq;
+    H9<T> z;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        z.d[k] = T(0);
+        z.o[k] = cx<T>{T(0), T(0)};
+    }
+#pragma unroll 1
+    for (int nu = 0; nu < 4; ++nu) {
+        if (nu == mu) continue;
+        axpy9(z, mu < nu ? T(1) : T(-1), ws_ld9(a.K, a.g.V, plane_of(mu, nu), x));
+        axpy9(z, T(1), ws_ld9(a.Lo, a.g.V, slot_of(mu, nu), down(a.g, x, nu)));
+    }
+    const T tr = (z.d[0] + z.d[1] + z.d[2]) / T(3);
+    H9<T> q;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        q.d[k] = a.rho * (z.d[k] - tr);
+        q.o[k] = cx<T>{a.rho * z.o[k].im, -a.rho * z.o[k].re};
+    }
+    return q;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_apply(const __grid_constant__ StoutPlaqArgs<T> a)
+{
+    using namespace plaq;
+    pdl_enter();
+    const int mu = blockIdx.y, x = blockIdx.x * kStoutBlock + threadIdx.x;
+    if (x >= a.g.V) return;
+    const H9<T> q = loops_q(a, mu, x), q2 = square9(q);
+    T c0, c1;
+    char_coefs9(q, q2, c0, c1);
+    const ExpCoefT<T> e = exp_sums<false>(c0, c1);
+    const M3T<T> u = mul<false, false>(poly9(e.f, q, q2), link_at<T>(a.U, a.g, mu, x));
+    typename C2<T>::type *o = a.out + ((long long)mu * a.g.V + x) * 9;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        o[k].x = u.m[k / 3][k % 3].re;
+        o[k].y = u.m[k / 3][k % 3].im;
+    }
+}
+
+// per link: E^dag G' into out, W and Y
+template <typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_grad_exp(const __grid_constant__ StoutPlaqArgs<T> a)
+{
+    using namespace plaq;
+    pdl_enter();
+    const int mu = blockIdx.y, x = blockIdx.x * kStoutBlock + threadIdx.x, V = a.g.V;
+    if (x >= V) return;
+    const H9<T> q = loops_q(a, mu, x), q2 = square9(q);
+    T c0, c1;
+    char_coefs9(q, q2, c0, c1);
+    const ExpCoefT<T> e = exp_sums<true>(c0, c1);
+    const M3T<T> gp = link_at<T>(a.G, a.g, mu, x);
+    {
+        const M3T<T> gu = mul<true, false>(poly9(e.f, q, q2), gp);
+        typename C2<T>::type *o = a.out + ((long long)mu * V + x) * 9;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            o[k].x = gu.m[k / 3][k % 3].re;
+            o[k].y = gu.m[k / 3][k % 3].im;
+        }
+    }
+    const M3T<T> u = link_at<T>(a.U, a.g, mu, x);
+    const M3T<T> M = mul<false, true>(gp, u);  // gradient of E
+    // t_j = tr(M^dag Q^j);  K0, K1 = sum_j Re(t_j df_j/dc0,1)
+    cx<T> t[3];
+    t[0] = cx<T>{M.m[0][0].re + M.m[1][1].re + M.m[2][2].re, -(M.m[0][0].im + M.m[1][1].im + M.m[2][2].im)};
+#pragma unroll
+    for (int j = 1; j < 3; ++j) {
+        const H9<T> &h = j == 1 ? q : q2;
+        cx<T> s = cx<T>{T(0), T(0)};
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            s.re = fma(M.m[r][r].re, h.d[r], s.re);
+            s.im = fma(-M.m[r][r].im, h.d[r], s.im);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int r = k == 2 ? 1 : 0, c = k == 0 ? 1 : 2;
+            cmac_conj(s, M.m[r][c], h.o[k]);
+            cmac_conj(s, M.m[c][r], cconj(h.o[k]));
+        }
+        t[j] = s;
+    }
+    T K0 = T(0), K1 = T(0);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        K0 += t[j].re * e.d0[j].re - t[j].im * e.d0[j].im;
+        K1 += t[j].re * e.d1[j].re - t[j].im * e.d1[j].im;
+    }
+    // Hermitian part of G_Q = K1 Q + K0 Q^2 + conj(f1) M + conj(f2) (M Q + Q M): the last term's is
+    // the anticommutator of Q with the Hermitian part of conj(f2) M
+    H9<T> n1, n2;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        n1.d[r] = fma(e.f[1].re, M.m[r][r].re, e.f[1].im * M.m[r][r].im);
+        n2.d[r] = fma(e.f[2].re, M.m[r][r].re, e.f[2].im * M.m[r][r].im);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int r = k == 2 ? 1 : 0, c = k == 0 ? 1 : 2;
+        const cx<T> s = M.m[r][c], z = cconj(M.m[c][r]);
+        cx<T> v = cmul(cconj(e.f[1]), s);
+        cmac(v, e.f[1], z);
+        n1.o[k] = cx<T>{T(0.5) * v.re, T(0.5) * v.im};
+        v = cmul(cconj(e.f[2]), s);
+        cmac(v, e.f[2], z);
+        n2.o[k] = cx<T>{T(0.5) * v.re, T(0.5) * v.im};
+    }
+    axpy9(n1, T(1), anticommutator9(q, n2));
+    axpy9(n1, K1, q);
+    axpy9(n1, K0, q2);
+    // W = rho TA(i G_Q)
+    const T tr = (n1.d[0] + n1.d[1] + n1.d[2]) / T(3);
+    H9<T> w;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        w.d[k] = a.rho * (n1.d[k] - tr);
+        w.o[k] = cx<T>{-a.rho * n1.o[k].im, a.rho * n1.o[k].re};
+    }
+    ws_st9(a.W, V, mu, x, w);
+    M3T<T> y = zero3<T>();
+    anti_mul_acc(y, w, u);
+    ws_st(a.Y, V, mu, x, y);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_bent(const __grid_constant__ StoutPlaqArgs<T> a)
+{
+    using namespace plaq;
+    pdl_enter();
+    const int x = blockIdx.x * kStoutBlock + threadIdx.x, V = a.g.V;
+    if (x >= V) return;
+    const int f = blockIdx.y;  // ordered pair (mu, nu)
+    int mu, nu;
+    plane_dirs(f >> 1, mu, nu);
+    if (f & 1) { const int t = mu; mu = nu; nu = t; }
+    H9<T> d = ws_ld9(a.W, V, nu, x);
+    axpy9(d, T(-1), ws_ld9(a.W, V, mu, x));
+    M3T<T> p = zero3<T>();
+    anti_mul_acc(p, d, ws_ld<T>(a.P, V, f, x));
+    mul_acc<false, false>(p, link_at<T>(a.U, a.g, nu, x), ws_ld<T>(a.Y, V, mu, up(a.g, x, nu)));
+    ws_st(a.Pb, V, f, x, p);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_gather(const __grid_constant__ StoutPlaqArgs<T> a)
+{
+    using namespace plaq;
+    pdl_enter();
+    const int mu = blockIdx.y, x = blockIdx.x * kStoutBlock + threadIdx.x, V = a.g.V;
+    if (x >= V) return;
+    const int xm = up(a.g, x, mu);
+    M3T<T> G = link_at<T>(a.out, a.g, mu, x), S = zero3<T>();
+#pragma unroll 1
+    for (int nu = 0; nu < 4; ++nu) {
+        if (nu == mu) continue;
+        const int f = slot_of(mu, nu), y = down(a.g, x, nu);
+        axpy3(S, T(-1), ws_ld<T>(a.Slo, V, f, y));
+        mul_acc<false, true>(G, ws_ld<T>(a.Pb, V, f, x), link_at<T>(a.U, a.g, nu, xm));
+        mul_acc<false, true>(G, ws_ld<T>(a.P, V, f, x), ws_ld<T>(a.Y, V, nu, xm));
+        mul_acc<true, false>(G, link_at<T>(a.U, a.g, nu, y), ws_ld<T>(a.Pb, V, f ^ 1, y));
+    }
+    anti_mul_acc(G, ws_ld9(a.W, V, mu, x), S);
+    if (a.proj) G = expand_anti_traceless(anti_mul<false, true>(link_at<T>(a.proj, a.g, mu, x), G));
+    typename C2<T>::type *o = a.out + ((long long)mu * V + x) * 9;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        o[k].x = G.m[k / 3][k % 3].re;
+        o[k].y = G.m[k / 3][k % 3].im;
+    }
+}
+
 stg_status check_common(const stg_lattice *lat, int nstep, double rho, const char *fn)
 {
     const std::string f(fn);
@@ -239,6 +479,119 @@ stg_status check_common(const stg_lattice *lat, int nstep, double rho, const cha
 }
 
 bool misaligned(const void *p) { return p == nullptr || (reinterpret_cast<uintptr_t>(p) & 15) != 0; }
+
+// Workspaces of the shared-plaquette steps: 1.3 kB (smearing) and 7.3 kB (chain rule) per site in
+// FP64.  Up to kStoutWorkspace they are taken from the pool; beyond, or when the pool has no room,
+// the per-link kernels above do the step.
+constexpr size_t kStoutWorkspace = (size_t)8 << 30;
+
+// Bump allocation of [count] fields of 9 V entries
+template <typename E>
+E *take(char *&p, int V, int count)
+{
+    E *r = reinterpret_cast<E *>(p);
+    p += ((size_t)count * 9 * V * sizeof(E) + 255) & ~(size_t)255;
+    return r;
+}
+
+// Whether the steps go by shared plaquettes.  FP32 stays with the per-link kernels, which are not
+// bound by their products (32^4 chain rule: 4.1 ms against 5.1 ms shared).  In FP64 every warp has a
+// quarter SM's pipe to itself while a launch has no more warps than quarters; the one window where
+// the per-link kernels fit that once and the 6 planes of a site do not (3243 to 4864 sites on 152
+// SMs) is theirs: 8^4 smears in 191 us against 220 us, 6^4 (191 against 94) and 5120 sites (351
+// against 250) do not.
+template <typename T>
+bool use_plaq(long long V, size_t bytes)
+{
+    if (sizeof(T) != 8 || V > INT_MAX || bytes > kStoutWorkspace) return false;
+    int dev = 0, nsm = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const long long warps = (V + 31) / 32;
+    return 6 * warps <= 4 * nsm || 4 * warps > 4 * nsm;
+}
+
+template <typename T>
+bool smear_plaq(const stg_lattice *lat, int nstep, double rho, const void *links, void *levels, cudaStream_t st,
+                cudaError_t &err)
+{
+    using C = typename C2<T>::type;
+    const size_t bytes = (size_t)18 * 9 * lat->V * sizeof(T) + 4096;
+    if (!use_plaq<T>(lat->V, bytes)) return false;
+    keep_pool_mapped(st);
+    char *ws = nullptr, *w;
+    if (cudaMallocAsync((void **)&ws, bytes, st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    StoutPlaqArgs<T> a;
+    memset(&a, 0, sizeof(a));
+    a.g = plaq::plaq_geo(lat->g);
+    a.rho = (T)rho;
+    w = ws;
+    a.K = take<T>(w, a.g.V, 6);
+    a.Lo = take<T>(w, a.g.V, 12);
+    const size_t level = (size_t)4 * a.g.V * 9;
+    const unsigned nb = (unsigned)((a.g.V + kStoutBlock - 1) / kStoutBlock);
+    err = cudaSuccess;
+    for (int k = 0; k < nstep && err == cudaSuccess; ++k) {
+        a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
+        a.out = static_cast<C *>(levels) + (size_t)k * level;
+        err = launch_pdl(k_stout_loops<false, T>, dim3(nb, 6), dim3(kStoutBlock), st, a);
+        if (err == cudaSuccess) err = launch_pdl(k_stout_apply<T>, dim3(nb, 4), dim3(kStoutBlock), st, a);
+    }
+    const cudaError_t f = cudaFreeAsync(ws, st);
+    if (err == cudaSuccess) err = f;
+    return true;
+}
+
+template <typename T>
+bool force_plaq(const stg_lattice *lat, int nstep, double rho, const void *links, const void *levels, const void *grad,
+                void *out_v, int kind, cudaStream_t st, cudaError_t &err)
+{
+    using C = typename C2<T>::type;
+    const size_t level = (size_t)4 * lat->V * 9;
+    const size_t bytes = (size_t)(22 * 9 + (36 + 4) * 18) * lat->V * sizeof(T) +
+                         (nstep > 1 ? level * sizeof(C) : 0) + 4096;
+    if (!use_plaq<T>(lat->V, bytes)) return false;
+    keep_pool_mapped(st);
+    char *ws = nullptr, *w;
+    if (cudaMallocAsync((void **)&ws, bytes, st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    StoutPlaqArgs<T> a;
+    memset(&a, 0, sizeof(a));
+    a.g = plaq::plaq_geo(lat->g);
+    a.rho = (T)rho;
+    w = ws;
+    a.K = take<T>(w, a.g.V, 6);
+    a.Lo = take<T>(w, a.g.V, 12);
+    a.W = take<T>(w, a.g.V, 4);
+    a.P = take<C>(w, a.g.V, 12);
+    a.Slo = take<C>(w, a.g.V, 12);
+    a.Pb = take<C>(w, a.g.V, 12);
+    a.Y = take<C>(w, a.g.V, 4);
+    C *tmp = nstep > 1 ? take<C>(w, a.g.V, 4) : nullptr;
+    C *out = static_cast<C *>(out_v);
+    const unsigned nb = (unsigned)((a.g.V + kStoutBlock - 1) / kStoutBlock);
+    const dim3 links4(nb, 4);
+    a.G = static_cast<const C *>(grad);
+    err = cudaSuccess;
+    for (int k = nstep - 1; k >= 0 && err == cudaSuccess; --k) {
+        // the last step (k = 0) lands in out; earlier ones alternate so that it does
+        a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
+        a.out = (k % 2 == 0) ? out : tmp;
+        a.proj = k == 0 && kind == 0 ? static_cast<const C *>(links) : nullptr;
+        err = launch_pdl(k_stout_loops<true, T>, dim3(nb, 6), dim3(kStoutBlock), st, a);
+        if (err == cudaSuccess) err = launch_pdl(k_stout_grad_exp<T>, links4, dim3(kStoutBlock), st, a);
+        if (err == cudaSuccess) err = launch_pdl(k_stout_bent<T>, dim3(nb, 12), dim3(kStoutBlock), st, a);
+        if (err == cudaSuccess) err = launch_pdl(k_stout_gather<T>, links4, dim3(kStoutBlock), st, a);
+        a.G = a.out;
+    }
+    const cudaError_t f = cudaFreeAsync(ws, st);
+    if (err == cudaSuccess) err = f;
+    return true;
+}
 
 template <typename T>
 cudaError_t smear_t(const LinkGeo &g, int nstep, double rho, const void *links, void *levels, cudaStream_t st)
@@ -315,6 +668,11 @@ extern "C" stg_status stg_stout_smear(const stg_lattice *lat, stg_prec prec, int
         return set_error(STG_ERR_ARG, "stg_stout_smear: buffers must be non-null and 16-byte aligned");
     const LinkGeo g = link_geo(lat->g);
     cudaStream_t st = (cudaStream_t)stream;
+    cudaError_t err = cudaSuccess;
+    if (prec == STG_F64 && smear_plaq<double>(lat, nstep, rho, links_dev, levels_dev, st, err)) {
+        STG_CUDA_TRY(err);
+        return STG_OK;
+    }
     STG_CUDA_TRY(prec == STG_F64 ? smear_t<double>(g, nstep, rho, links_dev, levels_dev, st)
                                  : smear_t<float>(g, nstep, rho, links_dev, levels_dev, st));
     return STG_OK;
@@ -336,6 +694,12 @@ extern "C" stg_status stg_stout_force(const stg_lattice *lat, stg_prec prec, int
         return set_error(STG_ERR_ARG, "stg_stout_force: out must not alias the inputs");
     const LinkGeo g = link_geo(lat->g);
     cudaStream_t st = (cudaStream_t)stream;
+    cudaError_t err = cudaSuccess;
+    if (prec == STG_F64 &&
+        force_plaq<double>(lat, nstep, rho, links_dev, levels_dev, grad_dev, out_dev, kind, st, err)) {
+        STG_CUDA_TRY(err);
+        return STG_OK;
+    }
     STG_CUDA_TRY(prec == STG_F64 ? force_t<double>(g, nstep, rho, links_dev, levels_dev, grad_dev, out_dev, kind, st)
                                  : force_t<float>(g, nstep, rho, links_dev, levels_dev, grad_dev, out_dev, kind, st));
     return STG_OK;
