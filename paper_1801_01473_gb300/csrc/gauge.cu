@@ -45,27 +45,11 @@ struct GaugeArgs {
 
 template <typename T>
 __device__ __forceinline__ M3T<T> lk(const typename C2<T>::type *__restrict__ U, const LinkGeo &g, int d,
-                                     long long site)
+                                     int site)
 {
     M3T<T> m;
     ld(U, g, d, site, m);
     return m;
-}
-
-// acc += w * op(a) op(b)
-template <bool DA, bool DB, typename T>
-__device__ __forceinline__ void mul_acc_w(M3T<T> &acc, T w, const M3T<T> &a, const M3T<T> &b)
-{
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            cx<T> z = cx<T>{T(0), T(0)};
-#pragma unroll
-            for (int k = 0; k < 3; ++k) cmac(z, el<DA>(a, r, k), el<DB>(b, k, c));
-            acc.m[r][c].re = fma(w, z.re, acc.m[r][c].re);
-            acc.m[r][c].im = fma(w, z.im, acc.m[r][c].im);
-        }
 }
 
 // Re tr(a b)
@@ -79,65 +63,70 @@ __device__ __forceinline__ double retr_mul(const M3 &a, const M3 &b)
     return s;
 }
 
-// One block per SM as the bound keeps ptxas from a low register target and heavy spills (FP32 with
-// three blocks per SM spilled and ran 18.5 ms instead of 15.2 ms at 48^4)
+// G = wr [sum of rectangle staples + kPlaq * sum of plaquette staples], kPlaq = 2 c0 / c1.  Each side
+// (upper, lower) of a plane is one plaquette staple U_nu U_mu U_nu^dag (lower: U_nu^dag U_mu U_nu) and
+// its three forms with one factor replaced by that link's outer staple: 11 products a side (each summed
+// before it is added to the larger total, which keeps the rounding of the loop-by-loop form), 66 per
+// link (84 when every loop is multiplied out).  Bound by latency at two blocks of 250 registers per SM;
+// three blocks of 168 ran 3 % slower at 32^4, four spill.  FP32, 32^4: 2.79 -> 1.75 ms with 32-bit site
+// arithmetic (neighbours by multiplication instead of 64-bit division), 16^4: 182 -> 118 us.
 template <typename T>
-__global__ void __launch_bounds__(kGaugeBlock, 1) k_gauge_force(const __grid_constant__ GaugeArgs<T> a)
+__global__ void __launch_bounds__(kGaugeBlock, 2) k_gauge_force(const __grid_constant__ GaugeArgs<T> a)
 {
     const int mu = blockIdx.y;
-    const long long x = (long long)blockIdx.x * kGaugeBlock + threadIdx.x;
+    const int x = blockIdx.x * kGaugeBlock + threadIdx.x;
     if (x >= a.g.V) return;
-    const LinkGeo g = a.g;
+    const LinkGeo &g = a.g;
     const typename C2<T>::type *__restrict__ Ub = a.U;
-    // G = -(beta/3) (2 c0 sum of plaquette staples + c1 sum of rectangle staples)
-    const T wp = T(-a.beta / 3.0 * 2.0 * kC0), wr = T(-a.beta / 3.0 * kC1);
+    const T wr = T(-a.beta / 3.0 * kC1), kPlaq = T(2.0 * kC0 / kC1);
     M3T<T> G = zero3<T>();
-    const long long xpm = nb(g, x, mu, 1), xmm = nb(g, x, mu, -1), xp2m = nb(g, xpm, mu, 1);
+    const int xpm = up(g, x, mu), xmm = down(g, x, mu), xp2m = up(g, xpm, mu);
 #pragma unroll 1
     for (int nu = 0; nu < 4; ++nu) {
         if (nu == mu) continue;
-        const long long xpn = nb(g, x, nu, 1), xmn = nb(g, x, nu, -1);
-        const long long xpm_pn = nb(g, xpm, nu, 1), xpm_mn = nb(g, xpm, nu, -1);
-        M3T<T> t;
-        // plaquette staples: U_nu(x) U_mu(x+nu) U_nu(x+mu)^dag and U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)
-        t = mul<false, false>(lk<T>(Ub, g, nu, x), lk<T>(Ub, g, mu, xpn));
-        mul_acc_w<false, true>(G, wp, t, lk<T>(Ub, g, nu, xpm));
-        t = mul<true, false>(lk<T>(Ub, g, nu, xmn), lk<T>(Ub, g, mu, xmn));
-        mul_acc_w<false, false>(G, wp, t, lk<T>(Ub, g, nu, xpm_mn));
-        // r1: U_nu(x) U_mu(x+nu) U_mu(x+mu+nu) U_nu(x+2mu)^dag U_mu(x+mu)^dag
-        t = mul<false, false>(lk<T>(Ub, g, nu, x), lk<T>(Ub, g, mu, xpn));
-        t = mul<false, false>(t, lk<T>(Ub, g, mu, xpm_pn));
-        t = mul<false, true>(t, lk<T>(Ub, g, nu, xp2m));
-        mul_acc_w<false, true>(G, wr, t, lk<T>(Ub, g, mu, xpm));
-        // r2: U_mu(x-mu)^dag U_nu(x-mu) U_mu(x-mu+nu) U_mu(x+nu) U_nu(x+mu)^dag
-        const long long xmm_pn = nb(g, xmm, nu, 1), xmm_mn = nb(g, xmm, nu, -1);
-        t = mul<true, false>(lk<T>(Ub, g, mu, xmm), lk<T>(Ub, g, nu, xmm));
-        t = mul<false, false>(t, lk<T>(Ub, g, mu, xmm_pn));
-        t = mul<false, false>(t, lk<T>(Ub, g, mu, xpn));
-        mul_acc_w<false, true>(G, wr, t, lk<T>(Ub, g, nu, xpm));
-        // r3: U_nu(x-nu)^dag U_mu(x-nu) U_mu(x+mu-nu) U_nu(x+2mu-nu) U_mu(x+mu)^dag
-        t = mul<true, false>(lk<T>(Ub, g, nu, xmn), lk<T>(Ub, g, mu, xmn));
-        t = mul<false, false>(t, lk<T>(Ub, g, mu, xpm_mn));
-        t = mul<false, false>(t, lk<T>(Ub, g, nu, nb(g, xp2m, nu, -1)));
-        mul_acc_w<false, true>(G, wr, t, lk<T>(Ub, g, mu, xpm));
-        // r4: U_mu(x-mu)^dag U_nu(x-mu-nu)^dag U_mu(x-mu-nu) U_mu(x-nu) U_nu(x+mu-nu)
-        t = mul<true, true>(lk<T>(Ub, g, mu, xmm), lk<T>(Ub, g, nu, xmm_mn));
-        t = mul<false, false>(t, lk<T>(Ub, g, mu, xmm_mn));
-        t = mul<false, false>(t, lk<T>(Ub, g, mu, xmn));
-        mul_acc_w<false, false>(G, wr, t, lk<T>(Ub, g, nu, xpm_mn));
-        // r5: U_nu(x) U_nu(x+nu) U_mu(x+2nu) U_nu(x+mu+nu)^dag U_nu(x+mu)^dag
-        t = mul<false, false>(lk<T>(Ub, g, nu, x), lk<T>(Ub, g, nu, xpn));
-        t = mul<false, false>(t, lk<T>(Ub, g, mu, nb(g, xpn, nu, 1)));
-        t = mul<false, true>(t, lk<T>(Ub, g, nu, xpm_pn));
-        mul_acc_w<false, true>(G, wr, t, lk<T>(Ub, g, nu, xpm));
-        // r6: U_nu(x-nu)^dag U_nu(x-2nu)^dag U_mu(x-2nu) U_nu(x+mu-2nu) U_nu(x+mu-nu)
-        const long long xm2n = nb(g, xmn, nu, -1);
-        t = mul<true, true>(lk<T>(Ub, g, nu, xmn), lk<T>(Ub, g, nu, xm2n));
-        t = mul<false, false>(t, lk<T>(Ub, g, mu, xm2n));
-        t = mul<false, false>(t, lk<T>(Ub, g, nu, nb(g, xpm_mn, nu, -1)));
-        mul_acc_w<false, false>(G, wr, t, lk<T>(Ub, g, nu, xpm_mn));
+        M3T<T> t, s, X;
+        {
+            const int xpn = up(g, x, nu), xpm_pn = up(g, xpm, nu);
+            // U_nu(x) U_mu(x+nu), with the outer staple of the last factor U_nu(x+mu)^dag
+            t = mul<false, false>(lk<T>(Ub, g, nu, x), lk<T>(Ub, g, mu, xpn));
+            s = mul<false, true>(lk<T>(Ub, g, mu, xpm_pn), lk<T>(Ub, g, nu, xp2m));
+            s = mul<false, true>(s, lk<T>(Ub, g, mu, xpm));
+            plaq::axpy3(G, T(1), mul<false, false>(t, s));
+            // outer staple of the middle factor U_mu(x+nu)
+            s = mul<false, false>(lk<T>(Ub, g, nu, xpn), lk<T>(Ub, g, mu, up(g, xpn, nu)));
+            s = mul<false, true>(s, lk<T>(Ub, g, nu, xpm_pn));
+            X = mul<false, false>(lk<T>(Ub, g, nu, x), s);
+            // outer staple of the first factor U_nu(x)
+            s = mul<true, false>(lk<T>(Ub, g, mu, xmm), lk<T>(Ub, g, nu, xmm));
+            s = mul<false, false>(s, lk<T>(Ub, g, mu, up(g, xmm, nu)));
+            mul_acc<false, false>(X, s, lk<T>(Ub, g, mu, xpn));
+            plaq::axpy3(X, kPlaq, t);
+            plaq::axpy3(G, T(1), mul<false, true>(X, lk<T>(Ub, g, nu, xpm)));
+        }
+        {
+            const int xmn = down(g, x, nu), xpm_mn = down(g, xpm, nu), xm2n = down(g, xmn, nu), xmm_mn = down(g, xmm, nu);
+            // U_nu(x-nu)^dag U_mu(x-nu), with the outer staple of the last factor U_nu(x+mu-nu)
+            t = mul<true, false>(lk<T>(Ub, g, nu, xmn), lk<T>(Ub, g, mu, xmn));
+            s = mul<false, false>(lk<T>(Ub, g, mu, xpm_mn), lk<T>(Ub, g, nu, down(g, xp2m, nu)));
+            s = mul<false, true>(s, lk<T>(Ub, g, mu, xpm));
+            plaq::axpy3(G, T(1), mul<false, false>(t, s));
+            // outer staple of the middle factor U_mu(x-nu)
+            s = mul<true, false>(lk<T>(Ub, g, nu, xm2n), lk<T>(Ub, g, mu, xm2n));
+            s = mul<false, false>(s, lk<T>(Ub, g, nu, down(g, xpm_mn, nu)));
+            X = mul<true, false>(lk<T>(Ub, g, nu, xmn), s);
+            // outer staple of the first factor U_nu(x-nu)^dag
+            s = mul<true, true>(lk<T>(Ub, g, mu, xmm), lk<T>(Ub, g, nu, xmm_mn));
+            s = mul<false, false>(s, lk<T>(Ub, g, mu, xmm_mn));
+            mul_acc<false, false>(X, s, lk<T>(Ub, g, mu, xmn));
+            plaq::axpy3(X, kPlaq, t);
+            plaq::axpy3(G, T(1), mul<false, false>(X, lk<T>(Ub, g, nu, xpm_mn)));
+        }
     }
-    if (a.kind == 0) G = ta(mul<false, true>(lk<T>(Ub, g, mu, x), G));
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) G.m[r][c] = cx<T>{wr * G.m[r][c].re, wr * G.m[r][c].im};
+    if (a.kind == 0) G = plaq::expand_anti_traceless(plaq::anti_mul<false, true>(lk<T>(Ub, g, mu, x), G));
     st(a.out, g, mu, x, G);
 }
 
@@ -159,7 +148,7 @@ constexpr int kPlaqBlock = 32;
 template <typename T>
 struct GaugePlaqArgs {
     using C = typename C2<T>::type;
-    plaq::PlaqGeo g;
+    LinkGeo g;
     const C *U;
     C *P, *Sup, *Slo, *Pb;  // one field per ordered pair of the planes [p0, p1)
     C *out;
@@ -227,42 +216,37 @@ __global__ void __launch_bounds__(kPlaqBlock) k_gauge_gather(const __grid_consta
     }
     axpy3(G, a.wr, R);
     if (a.last && a.kind == 0) G = expand_anti_traceless(anti_mul<false, true>(link_at<T>(a.U, a.g, mu, x), G));
-    typename C2<T>::type *o = a.out + ((long long)mu * V + x) * 9;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        o[k].x = G.m[k / 3][k % 3].re;
-        o[k].y = G.m[k / 3][k % 3].im;
-    }
+    st(a.out, a.g, mu, x, G);
 }
 
 __global__ void __launch_bounds__(kGaugeBlock, 1) k_gauge_action(const __grid_constant__ GaugeArgs<double> a)
 {
     __shared__ double sh[33];
-    const long long x = (long long)blockIdx.x * kGaugeBlock + threadIdx.x;
+    const int x = blockIdx.x * kGaugeBlock + threadIdx.x;
     const LinkGeo g = a.g;
     const double2 *__restrict__ Ub = a.U;
     double ps = 0.0, rs = 0.0;
     if (x < g.V) {
 #pragma unroll 1
         for (int mu = 0; mu < 4; ++mu) {
-            const long long xpm = nb(g, x, mu, 1);
+            const int xpm = up(g, x, mu);
 #pragma unroll 1
             for (int nu = mu + 1; nu < 4; ++nu) {
-                const long long xpn = nb(g, x, nu, 1);
+                const int xpn = up(g, x, nu);
                 // P = U_mu(x) U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
                 M3 t = mul<false, false>(lk<double>(Ub, g, mu, x), lk<double>(Ub, g, nu, xpm));
                 M3 w = mul<true, true>(lk<double>(Ub, g, mu, xpn), lk<double>(Ub, g, nu, x));
                 ps += retr_mul(t, w);
                 // R_{mu nu} = U_mu(x) U_mu(x+mu) U_nu(x+2mu) U_mu(x+mu+nu)^dag U_mu(x+nu)^dag U_nu(x)^dag
                 t = mul<false, false>(lk<double>(Ub, g, mu, x), lk<double>(Ub, g, mu, xpm));
-                t = mul<false, false>(t, lk<double>(Ub, g, nu, nb(g, xpm, mu, 1)));
-                w = mul<true, true>(lk<double>(Ub, g, mu, nb(g, xpm, nu, 1)), lk<double>(Ub, g, mu, xpn));
+                t = mul<false, false>(t, lk<double>(Ub, g, nu, up(g, xpm, mu)));
+                w = mul<true, true>(lk<double>(Ub, g, mu, up(g, xpm, nu)), lk<double>(Ub, g, mu, xpn));
                 w = mul<false, true>(w, lk<double>(Ub, g, nu, x));
                 rs += retr_mul(t, w);
                 // R_{nu mu} = U_nu(x) U_nu(x+nu) U_mu(x+2nu) U_nu(x+nu+mu)^dag U_nu(x+mu)^dag U_mu(x)^dag
                 t = mul<false, false>(lk<double>(Ub, g, nu, x), lk<double>(Ub, g, nu, xpn));
-                t = mul<false, false>(t, lk<double>(Ub, g, mu, nb(g, xpn, nu, 1)));
-                w = mul<true, true>(lk<double>(Ub, g, nu, nb(g, xpn, mu, 1)), lk<double>(Ub, g, nu, xpm));
+                t = mul<false, false>(t, lk<double>(Ub, g, mu, up(g, xpn, nu)));
+                w = mul<true, true>(lk<double>(Ub, g, nu, up(g, xpn, mu)), lk<double>(Ub, g, nu, xpm));
                 w = mul<false, true>(w, lk<double>(Ub, g, mu, x));
                 rs += retr_mul(t, w);
             }
@@ -317,7 +301,7 @@ static bool gauge_force_plaq(const stg_lattice *lat, double beta, const void *li
     if (lat->V > INT_MAX) return false;
     GaugePlaqArgs<T> a;
     memset(&a, 0, sizeof(a));
-    a.g = plaq::plaq_geo(lat->g);
+    a.g = link_geo(lat->g);
     a.U = static_cast<const C *>(links);
     a.out = static_cast<C *>(out);
     a.wp = T(-beta / 3.0 * 2.0 * kC0);
@@ -370,8 +354,10 @@ static cudaError_t gauge_force_t(const stg_lattice *lat, double beta, const void
     a.out = static_cast<typename C2<T>::type *>(out);
     a.kind = kind;
     // FP64: the shared staples wherever they fit (figures at the kernels).
-    // FP32: the loops one by one, which need no workspace traffic (32^4: 2.79 ms against 2.77 ms shared)
-    if (sizeof(T) == 8 && gauge_force_plaq<T>(lat, beta, links, out, kind, st, err)) return err;
+    // FP32: the loops one by one, which need no workspace traffic (32^4: 1.75 ms against 2.77 ms shared)
+    if constexpr (sizeof(T) == 8) {
+        if (gauge_force_plaq<T>(lat, beta, links, out, kind, st, err)) return err;
+    }
     const dim3 grid((unsigned)((a.g.V + kGaugeBlock - 1) / kGaugeBlock), 4);
     k_gauge_force<T><<<grid, kGaugeBlock, 0, st>>>(a);
     return cudaGetLastError();

@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kMdBlock) k_md_update_links(const __grid_const
     const M3 q2 = mul<false, false>(q, q);
     double c0, c1;
     char_coefs(q, q2, c0, c1);
-    const ExpCoef e = exp_coef<false>(c0, c1);
+    const ExpCoef e = exp_sums<false>(c0, c1);
     ldl(a.U, l, u);
     stl(a.U, l, mul<false, false>(poly3(e.f, q, q2), u));
 }

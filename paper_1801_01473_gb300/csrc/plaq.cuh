@@ -1,6 +1,6 @@
-// plaq.cuh -- what the plaquette-sharing link kernels have in common: the geometry of a site's
-// plaquettes, matrices held as structure-of-arrays workspaces, anti-Hermitian and Hermitian 3x3
-// matrices by their 9 real numbers, and exp(iQ) of a Hermitian Q in that form.
+// plaq.cuh -- what the plaquette-sharing link kernels have in common: the planes of a site, matrices
+// held as structure-of-arrays workspaces, anti-Hermitian and Hermitian 3x3 matrices by their 9 real
+// numbers.
 //
 // For an ordered pair of directions (mu, nu) and a site x,
 //   P(mu, nu)(x)   = U_nu(x) U_mu(x+nu)             the corner path x -> x+nu -> x+nu+mu
@@ -16,43 +16,6 @@
 namespace stg {
 namespace plaq {
 using namespace su3;
-
-struct PlaqGeo {
-    int L[4], stride[4];
-    int V;
-    FastDiv by_stride[4], by_L[4];
-};
-
-inline PlaqGeo plaq_geo(const Geom &geo)
-{
-    PlaqGeo g;
-    long long s = 1;
-    for (int mu = 0; mu < 4; ++mu) {
-        g.L[mu] = geo.L[mu];
-        g.stride[mu] = (int)s;
-        g.by_stride[mu] = make_fast_div((unsigned)s);
-        g.by_L[mu] = make_fast_div((unsigned)geo.L[mu]);
-        s *= geo.L[mu];
-    }
-    g.V = (int)s;
-    return g;
-}
-
-__device__ __forceinline__ int coord(const PlaqGeo &g, int i, int mu)
-{
-    const int q = fast_div(i, g.by_stride[mu]);
-    return q - fast_div(q, g.by_L[mu]) * g.L[mu];
-}
-
-// neighbours of site i along mu (periodic)
-__device__ __forceinline__ int up(const PlaqGeo &g, int i, int mu)
-{
-    return coord(g, i, mu) == g.L[mu] - 1 ? i - (g.L[mu] - 1) * g.stride[mu] : i + g.stride[mu];
-}
-__device__ __forceinline__ int down(const PlaqGeo &g, int i, int mu)
-{
-    return coord(g, i, mu) == 0 ? i + (g.L[mu] - 1) * g.stride[mu] : i - g.stride[mu];
-}
 
 // The 6 planes (m < n) in the order 01 02 03 12 13 23; an ordered pair (mu, nu) is slot 2 p of its
 // plane p when mu < nu and slot 2 p + 1 otherwise.
@@ -70,15 +33,10 @@ __device__ __forceinline__ void plane_dirs(int p, int &m, int &n)
 
 // matrix of canonical links [4][V][3][3]
 template <typename T>
-__device__ __forceinline__ M3T<T> link_at(const typename C2<T>::type *__restrict__ U, const PlaqGeo &g, int mu, int i)
+__device__ __forceinline__ M3T<T> link_at(const typename C2<T>::type *__restrict__ U, const LinkGeo &g, int mu, int i)
 {
     M3T<T> a;
-    const typename C2<T>::type *p = U + ((long long)mu * g.V + i) * 9;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const typename C2<T>::type v = p[k];
-        a.m[k / 3][k % 3] = cx<T>{v.x, v.y};
-    }
+    ld(U, g, mu, i, a);
     return a;
 }
 
@@ -304,94 +262,6 @@ __device__ __forceinline__ void char_coefs9(const H9<T> &q, const H9<T> &q2, T &
     const cx<T> t = cmul(q.o[0], q.o[2]);  // q01 q12, to be taken with q20 = conj(q02)
     const T re = fma(t.re, q.o[1].re, t.im * q.o[1].im);
     c0 = fma(q.d[0], fma(q.d[1], q.d[2], -n12), fma(T(2), re, -fma(q.d[1], n02, q.d[2] * n01)));
-}
-
-// 1/n!, n = 0..131
-template <typename T>
-struct InvFactorial {
-    T v[132];
-    constexpr InvFactorial() : v{}
-    {
-        double f = 1.0;
-        for (int n = 0; n < 132; ++n) {
-            v[n] = f < (sizeof(T) == 4 ? 1e-37 : 0.0) ? T(0) : (T)f;
-            f /= n + 1;
-        }
-    }
-};
-__constant__ constexpr InvFactorial<double> kInvFactorial64{};
-__constant__ constexpr InvFactorial<float> kInvFactorial32{};
-template <typename T>
-__device__ __forceinline__ T inv_factorial(int n)
-{
-    return sizeof(T) == 8 ? (T)kInvFactorial64.v[n] : (T)kInvFactorial32.v[n];
-}
-
-// exp(iQ) = f0 + f1 Q + f2 Q^2 with the derivatives of the f_j, as exp_coef, from one sequence.
-// Q^3 = c1 Q + c0 gives Q^n = c0 h_{n-1} + h_{n+1} Q + h_n Q^2 (n >= 1) with
-//   h_0 = h_1 = 0, h_2 = 1, h_{n+1} = c1 h_{n-1} + c0 h_{n-2},
-// and g_n = dh_n/dc0 satisfies dh_n/dc1 = g_{n+1} (both from the generating function
-// t^2 / (1 - c1 t^2 - c0 t^3)), g_{n+1} = c1 g_{n-1} + c0 g_{n-2} + h_{n-2}.  So with s_n = i^n / n!
-//   f2 = sum s_n h_n, f1 = sum s_n h_{n+1}, f0 = 1 + c0 sum s_n h_{n-1},
-//   df2/dc0 = sum s_n g_n,  df2/dc1 = df1/dc0 = sum s_n g_{n+1},  df1/dc1 = sum s_n g_{n+2},
-//   df0/dc0 = sum s_n h_{n-1} + c0 sum s_n g_{n-1},  df0/dc1 = c0 df2/dc0:
-// 5 (12 with derivatives) multiply-adds per term, no divisions; the number of terms is settled
-// beforehand in FP32 by exp_coef's bound.
-template <bool DERIV, typename T>
-__device__ __forceinline__ ExpCoefT<T> exp_sums(T c0, T c1)
-{
-    int nmax = 6;
-    {
-        const float stop = sizeof(T) == 4 ? 1e-9f : 1e-18f;
-        float r = sqrtf(fmaxf(2.f * (float)c1, 0.f));
-        if (!(r >= 1.f)) r = 1.f;
-        float bound = 1.f;  // r^n / n!
-        for (int n = 1; n < 128; ++n) {
-            bound *= __fdividef(r, (float)n);
-            const float m = (float)(n + 1);
-            nmax = n;
-            if (n >= 6 && bound * m * m * m < stop) break;
-        }
-    }
-    T hm = T(0), h = T(0), hp = T(1);               // h_{n-1}, h_n, h_{n+1} at n = 1
-    T gm = T(0), g = T(0), gp = T(0), gpp = T(0);               // g_{n-1}, g_n, g_{n+1}, g_{n+2}
-    T s0[2] = {T(0), T(0)}, s1[2] = {T(0), T(0)}, s2[2] = {T(0), T(0)};  // sums of h_{n-1}, h_n, h_{n+1}; [1] odd n
-    T d0[2] = {T(0), T(0)}, d1[2] = {T(0), T(0)}, d2[2] = {T(0), T(0)}, d3[2] = {T(0), T(0)};  // g_{n-1} .. g_{n+2}
-#pragma unroll 1
-    for (int n0 = 1; n0 <= nmax; n0 += 4) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {  // n = n0 + u = 1 + u mod 4: i^n = i, -1, -i, 1
-            T s = inv_factorial<T>(n0 + u);
-            if (u == 1 || u == 2) s = -s;
-            const int o = (u & 1) ? 0 : 1;
-            s0[o] = fma(s, hm, s0[o]);
-            s1[o] = fma(s, h, s1[o]);
-            s2[o] = fma(s, hp, s2[o]);
-            if (DERIV) {
-                d0[o] = fma(s, gm, d0[o]);
-                d1[o] = fma(s, g, d1[o]);
-                d2[o] = fma(s, gp, d2[o]);
-                d3[o] = fma(s, gpp, d3[o]);
-                const T gn = fma(c1, gp, fma(c0, g, h));  // g_{n+3}
-                gm = g; g = gp; gp = gpp; gpp = gn;
-            }
-            const T hn = fma(c1, h, c0 * hm);  // h_{n+2}
-            hm = h; h = hp; hp = hn;
-        }
-    }
-    ExpCoefT<T> e;
-    e.f[0] = cx<T>{fma(c0, s0[0], T(1)), c0 * s0[1]};
-    e.f[1] = cx<T>{s2[0], s2[1]};
-    e.f[2] = cx<T>{s1[0], s1[1]};
-    if (DERIV) {
-        e.d0[0] = cx<T>{fma(c0, d0[0], s0[0]), fma(c0, d0[1], s0[1])};
-        e.d0[1] = cx<T>{d2[0], d2[1]};
-        e.d0[2] = cx<T>{d1[0], d1[1]};
-        e.d1[0] = cx<T>{c0 * d1[0], c0 * d1[1]};
-        e.d1[1] = cx<T>{d3[0], d3[1]};
-        e.d1[2] = cx<T>{d2[0], d2[1]};
-    }
-    return e;
 }
 
 // f0 + f1 q + f2 q2 of Hermitian q, q2

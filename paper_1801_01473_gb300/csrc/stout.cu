@@ -31,11 +31,11 @@
 
 namespace stg {
 namespace {
-using namespace su3;
+using namespace plaq;
 
 // Weighted staple sum C_mu(x) = rho * sum_{nu != mu} (upper + lower staple).
 template <typename T>
-__device__ M3T<T> staple_sum(const typename C2<T>::type *__restrict__ U, const LinkGeo &g, int mu, long long i,
+__device__ M3T<T> staple_sum(const typename C2<T>::type *__restrict__ U, const LinkGeo &g, int mu, int i,
                              T rho)
 {
     M3T<T> c = zero3<T>();
@@ -45,16 +45,16 @@ __device__ M3T<T> staple_sum(const typename C2<T>::type *__restrict__ U, const L
         M3T<T> a, b, t;
         // U_nu(x) U_mu(x+nu) U_nu(x+mu)^dag
         ld(U, g, nu, i, a);
-        ld(U, g, mu, nb(g, i, nu, 1), b);
+        ld(U, g, mu, up(g, i, nu), b);
         t = mul<false, false>(a, b);
-        ld(U, g, nu, nb(g, i, mu, 1), a);
+        ld(U, g, nu, up(g, i, mu), a);
         mul_acc<false, true>(c, t, a);
         // U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)
-        const long long xm = nb(g, i, nu, -1);
+        const int xm = down(g, i, nu);
         ld(U, g, nu, xm, a);
         ld(U, g, mu, xm, b);
         t = mul<true, false>(a, b);
-        ld(U, g, nu, nb(g, xm, mu, 1), a);
+        ld(U, g, nu, up(g, xm, mu), a);
         mul_acc<false, false>(c, t, a);
     }
 #pragma unroll
@@ -64,301 +64,31 @@ __device__ M3T<T> staple_sum(const typename C2<T>::type *__restrict__ U, const L
     return c;
 }
 
-// Q = -i TA(C U^dag) and its square; returns nothing else
+// Q = -i rho TA(Z) from the anti-Hermitian part of Z
 template <typename T>
-__device__ __forceinline__ void make_q(const M3T<T> &C, const M3T<T> &u, M3T<T> &q, M3T<T> &q2)
+__device__ __forceinline__ H9<T> q_of(const H9<T> &z, T rho)
 {
-    const M3T<T> a = ta(mul<false, true>(C, u));  // = i Q
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) q.m[r][c] = cx<T>{a.m[r][c].im, -a.m[r][c].re};
-    q2 = mul<false, false>(q, q);
-}
-
-template <typename T>
-struct StoutArgs {
-    using C = typename C2<T>::type;
-    LinkGeo g;
-    T rho;
-    const C *U;  // links of this step
-    const C *G;  // gradient of the step's output (backward)
-    C *out;      // smeared links (forward) / gradient of U (backward)
-    C *Y;        // rho G_Omega U (backward)
-};
-
-constexpr int kStoutBlock = 128;
-
-template <typename T>
-__global__ void __launch_bounds__(kStoutBlock) k_stout_fwd(const __grid_constant__ StoutArgs<T> a)
-{
-    const int mu = blockIdx.y;
-    const long long i = (long long)blockIdx.x * kStoutBlock + threadIdx.x;
-    if (i >= a.g.V) return;
-    M3T<T> q, q2, u;
-    {
-        const M3T<T> C = staple_sum(a.U, a.g, mu, i, a.rho);
-        ld(a.U, a.g, mu, i, u);
-        make_q(C, u, q, q2);
-    }
-    T c0, c1;
-    char_coefs(q, q2, c0, c1);
-    const ExpCoefT<T> e = exp_coef<false>(c0, c1);
-    const M3T<T> E = poly3(e.f, q, q2);
-    st(a.out, a.g, mu, i, mul<false, false>(E, u));
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kStoutBlock) k_stout_back_link(const __grid_constant__ StoutArgs<T> a)
-{
-    const int mu = blockIdx.y;
-    const long long i = (long long)blockIdx.x * kStoutBlock + threadIdx.x;
-    if (i >= a.g.V) return;
-    M3T<T> u, q, q2, gp;
-    const M3T<T> C = staple_sum(a.U, a.g, mu, i, a.rho);
-    ld(a.U, a.g, mu, i, u);
-    make_q(C, u, q, q2);
-    T c0, c1;
-    char_coefs(q, q2, c0, c1);
-    const ExpCoefT<T> e = exp_coef<true>(c0, c1);
-    ld(a.G, a.g, mu, i, gp);
-    // the link's own terms: E^dag G' (later + G_Omega^dag C)
-    M3T<T> gu = mul<true, false>(poly3(e.f, q, q2), gp);
-    const M3T<T> M = mul<false, true>(gp, u);  // gradient of E
-    // Tr_j = tr(M^dag Q^j);  K = sum_j Re(T_j df_j/dc)
-    cx<T> Tr[3] = {cx<T>{T(0), T(0)}, cx<T>{T(0), T(0)}, cx<T>{T(0), T(0)}};
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        Tr[0] = cx<T>{Tr[0].re + M.m[r][r].re, Tr[0].im - M.m[r][r].im};
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            cmac_conj(Tr[1], M.m[k][r], q.m[k][r]);
-            cmac_conj(Tr[2], M.m[k][r], q2.m[k][r]);
-        }
-    }
-    T K0 = T(0), K1 = T(0);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        K0 += Tr[j].re * e.d0[j].re - Tr[j].im * e.d0[j].im;
-        K1 += Tr[j].re * e.d1[j].re - Tr[j].im * e.d1[j].im;
-    }
-    // G_Q = K1 Q + K0 Q^2 + conj(f1) M + conj(f2) (M Q + Q M)
-    M3T<T> gq = mul<false, false>(M, q);
-    mul_acc<false, false>(gq, q, M);
-    const cx<T> f1c = cconj(e.f[1]), f2c = cconj(e.f[2]);
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            cx<T> v = cmul(f2c, gq.m[r][c]);
-            cmac(v, f1c, M.m[r][c]);
-            v.re += K1 * q.m[r][c].re + K0 * q2.m[r][c].re;
-            v.im += K1 * q.m[r][c].im + K0 * q2.m[r][c].im;
-            gq.m[r][c] = cx<T>{-v.im, v.re};  // i G_Q
-        }
-    const M3T<T> go = ta(gq);  // G_Omega
-    mul_acc<true, false>(gu, go, C);
-    st(a.out, a.g, mu, i, gu);
-    M3T<T> y = mul<false, false>(go, u);
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) y.m[r][c] = cx<T>{a.rho * y.m[r][c].re, a.rho * y.m[r][c].im};
-    st(a.Y, a.g, mu, i, y);
-}
-
-// Adds to the gradient of link (y, nu) the staple terms: for every mu != nu, the link sits in
-//   C_mu(y)       as the first factor of the upper staple      -> Y_mu(y) U_nu(y+mu) U_mu(y+nu)^dag
-//   C_mu(y+nu)    as the first factor of the lower staple      -> U_mu(y) U_nu(y+mu) Y_mu(y+nu)^dag
-//   C_nu(y+mu)    as the middle factor of the lower staple     -> U_mu(y) Y_nu(y+mu) U_mu(y+nu)^dag
-//   C_mu(y-mu)    as the last factor of the upper staple       -> Y_mu(y-mu)^dag U_nu(y-mu) U_mu(y-mu+nu)
-//   C_mu(y-mu+nu) as the last factor of the lower staple       -> U_mu(y-mu)^dag U_nu(y-mu) Y_mu(y-mu+nu)
-//   C_nu(y-mu)    as the middle factor of the upper staple     -> U_mu(y-mu)^dag Y_nu(y-mu) U_mu(y-mu+nu)
-// with Y the gradient of the unweighted staple sums.
-template <typename T>
-__global__ void __launch_bounds__(kStoutBlock) k_stout_back_staples(const __grid_constant__ StoutArgs<T> a)
-{
-    const int nu = blockIdx.y;
-    const long long i = (long long)blockIdx.x * kStoutBlock + threadIdx.x;
-    if (i >= a.g.V) return;
-    M3T<T> acc;
-    ld(a.out, a.g, nu, i, acc);
-#pragma unroll 1
-    for (int mu = 0; mu < 4; ++mu) {
-        if (mu == nu) continue;
-        const long long yp = nb(a.g, i, mu, 1), yn = nb(a.g, i, nu, 1);
-        const long long ym = nb(a.g, i, mu, -1), ymn = nb(a.g, ym, nu, 1);
-        M3T<T> p, q, t;
-        // forward side: U_nu(y+mu) shared by the first two terms
-        ld(a.U, a.g, nu, yp, p);   // U_nu(y+mu)
-        ld(a.U, a.g, mu, yn, q);   // U_mu(y+nu)
-        t = mul<false, true>(p, q);
-        ld(a.Y, a.g, mu, i, q);    // Y_mu(y)
-        mul_acc<false, false>(acc, q, t);
-        ld(a.U, a.g, mu, i, q);    // U_mu(y)
-        t = mul<false, false>(q, p);
-        ld(a.Y, a.g, mu, yn, p);   // Y_mu(y+nu)
-        mul_acc<false, true>(acc, t, p);
-        ld(a.Y, a.g, nu, yp, p);   // Y_nu(y+mu)
-        t = mul<false, false>(q, p);
-        ld(a.U, a.g, mu, yn, q);   // U_mu(y+nu)
-        mul_acc<false, true>(acc, t, q);
-        // backward side: U_mu(y-mu)^dag leads the last two terms
-        ld(a.U, a.g, nu, ym, p);   // U_nu(y-mu)
-        ld(a.U, a.g, mu, ymn, q);  // U_mu(y-mu+nu)
-        t = mul<false, false>(p, q);
-        ld(a.Y, a.g, mu, ym, q);   // Y_mu(y-mu)
-        mul_acc<true, false>(acc, q, t);
-        ld(a.Y, a.g, mu, ymn, q);  // Y_mu(y-mu+nu)
-        t = mul<false, false>(p, q);
-        ld(a.Y, a.g, nu, ym, p);   // Y_nu(y-mu)
-        ld(a.U, a.g, mu, ymn, q);  // U_mu(y-mu+nu)
-        mul_acc<false, false>(t, p, q);
-        ld(a.U, a.g, mu, ym, p);   // U_mu(y-mu)
-        mul_acc<true, false>(acc, p, t);
-    }
-    st(a.out, a.g, nu, i, acc);
-}
-
-// F = TA(U G^dag) in place over G
-template <typename T>
-__global__ void __launch_bounds__(kStoutBlock) k_lie_force(const __grid_constant__ StoutArgs<T> a)
-{
-    const int mu = blockIdx.y;
-    const long long i = (long long)blockIdx.x * kStoutBlock + threadIdx.x;
-    if (i >= a.g.V) return;
-    M3T<T> u, gr;
-    ld(a.U, a.g, mu, i, u);
-    ld(a.out, a.g, mu, i, gr);
-    st(a.out, a.g, mu, i, ta(mul<false, true>(u, gr)));
-}
-
-// ------------------------------------------------------------------ by shared plaquettes
-// The same step with every corner path made once per plaquette (plaq.cuh).  C U^dag is a sum over
-// the plaquettes of the link of closed loops at its start: for the upper plaquette of (x, mu)
-// P(mu, nu) P(nu, mu)^dag, whose anti-Hermitian part serves link (x, nu) with the opposite sign; for
-// the lower one Slo(mu, nu)(x-nu) U_mu(x)^dag.  Only the anti-Hermitian parts are needed (9 numbers).
-//
-// Chain rule: with W = rho G_Omega of every link fixed, dS is the change of Re tr of the plaquettes
-// when each link moves by Y = W U, so the gradient has the form of the rectangle force, with
-//   P'(mu, nu)(x) = (W_nu - W_mu)(x) P(mu, nu)(x) + U_nu(x) Y_mu(x+nu)
-//   G_mu(x) = E^dag G' + sum_nu [ P'(mu, nu)(x) U_nu(x+mu)^dag + P(mu, nu)(x) Y_nu(x+mu)^dag
-//                               + U_nu(y)^dag P'(nu, mu)(y) ] - W_mu(x) sum_nu Slo(mu, nu)(y),  y = x - nu.
-//
-// ~1450 FP64 multiply-adds per link and smearing step (k_stout_fwd ~2300) and ~3700 per step of the
-// chain rule (k_stout_back_* ~6850), both at the FP64 pipe's rate (0.58e12/s): two steps of 16^3x32
-// 4.59 -> 2.65 ms, of the chain rule on 20x12x28x16 10.7 -> 5.7 ms.
-template <typename T>
-struct StoutPlaqArgs {
-    using C = typename C2<T>::type;
-    plaq::PlaqGeo g;
-    T rho;
-    const C *U;    // links of this step
-    const C *G;    // gradient of the step's output (backward)
-    C *out;        // smeared links / gradient of U
-    T *K, *Lo;     // anti-Hermitian loops: upper per plane [6], lower per ordered pair [12] (based at x)
-    C *P, *Slo, *Pb;  // per ordered pair [12] (backward)
-    T *W;          // [4] rho G_Omega, anti-Hermitian
-    C *Y;          // [4] W U
-    const C *proj;  // last step of kind 0: the links for F = TA(U G^dag); null otherwise
-};
-
-template <bool BWD, typename T>
-__global__ void __launch_bounds__(kStoutBlock) k_stout_loops(const __grid_constant__ StoutPlaqArgs<T> a)
-{
-    using namespace plaq;
-    pdl_enter();
-    const int x = blockIdx.x * kStoutBlock + threadIdx.x, V = a.g.V;
-    if (x >= V) return;
-    const int p = blockIdx.y;
-    int m, n;
-    plane_dirs(p, m, n);
-    const int xm = up(a.g, x, m), xn = up(a.g, x, n);
-    const M3T<T> pmn = mul<false, false>(link_at<T>(a.U, a.g, n, x), link_at<T>(a.U, a.g, m, xn));
-    const M3T<T> pnm = mul<false, false>(link_at<T>(a.U, a.g, m, x), link_at<T>(a.U, a.g, n, xm));
-    if (BWD) {
-        ws_st(a.P, V, 2 * p, x, pmn);
-        ws_st(a.P, V, 2 * p + 1, x, pnm);
-    }
-    ws_st9(a.K, V, p, x, anti_mul<false, true>(pmn, pnm));
-    M3T<T> s = mul<true, false>(link_at<T>(a.U, a.g, n, x), pnm);  // Slo(m, n): of link (x+n, m)
-    if (BWD) ws_st(a.Slo, V, 2 * p, x, s);
-    ws_st9(a.Lo, V, 2 * p, x, anti_mul<false, true>(s, link_at<T>(a.U, a.g, m, xn)));
-    s = mul<true, false>(link_at<T>(a.U, a.g, m, x), pmn);  // Slo(n, m): of link (x+m, n)
-    if (BWD) ws_st(a.Slo, V, 2 * p + 1, x, s);
-    ws_st9(a.Lo, V, 2 * p + 1, x, anti_mul<false, true>(s, link_at<T>(a.U, a.g, n, xm)));
-}
-
-// Q = -i TA(C U^dag) of link (x, mu) from its loops
-template <typename T>
-__device__ __forceinline__ plaq::H9<T> loops_q(const StoutPlaqArgs<T> &a, int mu, int x)
-{
-    using namespace plaq;
-    H9<T> z;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        z.d[k] = T(0);
-        z.o[k] = cx<T>{T(0), T(0)};
-    }
-#pragma unroll 1
-    for (int nu = 0; nu < 4; ++nu) {
-        if (nu == mu) continue;
-        axpy9(z, mu < nu ? T(1) : T(-1), ws_ld9(a.K, a.g.V, plane_of(mu, nu), x));
-        axpy9(z, T(1), ws_ld9(a.Lo, a.g.V, slot_of(mu, nu), down(a.g, x, nu)));
-    }
     const T tr = (z.d[0] + z.d[1] + z.d[2]) / T(3);
     H9<T> q;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        q.d[k] = a.rho * (z.d[k] - tr);
-        q.o[k] = cx<T>{a.rho * z.o[k].im, -a.rho * z.o[k].re};
+        q.d[k] = rho * (z.d[k] - tr);
+        q.o[k] = cx<T>{rho * z.o[k].im, -rho * z.o[k].re};
     }
     return q;
 }
 
+// One link of the chain rule: with G' = gp the gradient of the smeared link E U, E = exp(iQ), sets
+// gu = E^dag G' and w = rho G_Omega, G_Omega = TA(i G_Q) the gradient of the algebra element.
 template <typename T>
-__global__ void __launch_bounds__(kStoutBlock) k_stout_apply(const __grid_constant__ StoutPlaqArgs<T> a)
+__device__ __forceinline__ void exp_gradient(const H9<T> &q, const M3T<T> &u, const M3T<T> &gp, T rho, M3T<T> &gu,
+                                             H9<T> &w)
 {
-    using namespace plaq;
-    pdl_enter();
-    const int mu = blockIdx.y, x = blockIdx.x * kStoutBlock + threadIdx.x;
-    if (x >= a.g.V) return;
-    const H9<T> q = loops_q(a, mu, x), q2 = square9(q);
-    T c0, c1;
-    char_coefs9(q, q2, c0, c1);
-    const ExpCoefT<T> e = exp_sums<false>(c0, c1);
-    const M3T<T> u = mul<false, false>(poly9(e.f, q, q2), link_at<T>(a.U, a.g, mu, x));
-    typename C2<T>::type *o = a.out + ((long long)mu * a.g.V + x) * 9;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        o[k].x = u.m[k / 3][k % 3].re;
-        o[k].y = u.m[k / 3][k % 3].im;
-    }
-}
-
-// per link: E^dag G' into out, W and Y
-template <typename T>
-__global__ void __launch_bounds__(kStoutBlock) k_stout_grad_exp(const __grid_constant__ StoutPlaqArgs<T> a)
-{
-    using namespace plaq;
-    pdl_enter();
-    const int mu = blockIdx.y, x = blockIdx.x * kStoutBlock + threadIdx.x, V = a.g.V;
-    if (x >= V) return;
-    const H9<T> q = loops_q(a, mu, x), q2 = square9(q);
+    const H9<T> q2 = square9(q);
     T c0, c1;
     char_coefs9(q, q2, c0, c1);
     const ExpCoefT<T> e = exp_sums<true>(c0, c1);
-    const M3T<T> gp = link_at<T>(a.G, a.g, mu, x);
-    {
-        const M3T<T> gu = mul<true, false>(poly9(e.f, q, q2), gp);
-        typename C2<T>::type *o = a.out + ((long long)mu * V + x) * 9;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            o[k].x = gu.m[k / 3][k % 3].re;
-            o[k].y = gu.m[k / 3][k % 3].im;
-        }
-    }
-    const M3T<T> u = link_at<T>(a.U, a.g, mu, x);
+    gu = mul<true, false>(poly9(e.f, q, q2), gp);
     const M3T<T> M = mul<false, true>(gp, u);  // gradient of E
     // t_j = tr(M^dag Q^j);  K0, K1 = sum_j Re(t_j df_j/dc0,1)
     cx<T> t[3];
@@ -410,12 +140,234 @@ __global__ void __launch_bounds__(kStoutBlock) k_stout_grad_exp(const __grid_con
     axpy9(n1, K0, q2);
     // W = rho TA(i G_Q)
     const T tr = (n1.d[0] + n1.d[1] + n1.d[2]) / T(3);
-    H9<T> w;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        w.d[k] = a.rho * (n1.d[k] - tr);
-        w.o[k] = cx<T>{-a.rho * n1.o[k].im, a.rho * n1.o[k].re};
+        w.d[k] = rho * (n1.d[k] - tr);
+        w.o[k] = cx<T>{-rho * n1.o[k].im, rho * n1.o[k].re};
     }
+}
+
+template <typename T>
+struct StoutArgs {
+    using C = typename C2<T>::type;
+    LinkGeo g;
+    T rho;
+    const C *U;  // links of this step
+    const C *G;  // gradient of the step's output (backward)
+    C *out;      // smeared links (forward) / gradient of U (backward)
+    C *Y;        // rho G_Omega U (backward)
+};
+
+constexpr int kStoutBlock = 128;
+
+template <typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_fwd(const __grid_constant__ StoutArgs<T> a)
+{
+    const int mu = blockIdx.y;
+    const int i = blockIdx.x * kStoutBlock + threadIdx.x;
+    if (i >= a.g.V) return;
+    const M3T<T> u = link_at<T>(a.U, a.g, mu, i);
+    const H9<T> q = q_of(anti_mul<false, true>(staple_sum(a.U, a.g, mu, i, a.rho), u), T(1)), q2 = square9(q);
+    T c0, c1;
+    char_coefs9(q, q2, c0, c1);
+    const ExpCoefT<T> e = exp_sums<false>(c0, c1);
+    st(a.out, a.g, mu, i, mul<false, false>(poly9(e.f, q, q2), u));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_back_link(const __grid_constant__ StoutArgs<T> a)
+{
+    const int mu = blockIdx.y;
+    const int i = blockIdx.x * kStoutBlock + threadIdx.x;
+    if (i >= a.g.V) return;
+    const M3T<T> C = staple_sum(a.U, a.g, mu, i, a.rho);
+    const M3T<T> u = link_at<T>(a.U, a.g, mu, i);
+    M3T<T> gu;
+    H9<T> go;
+    exp_gradient(q_of(anti_mul<false, true>(C, u), T(1)), u, link_at<T>(a.G, a.g, mu, i), T(1), gu, go);
+    M3T<T> y = zero3<T>();
+    anti_mul_acc(y, go, u);
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) y.m[r][c] = cx<T>{a.rho * y.m[r][c].re, a.rho * y.m[r][c].im};
+    st(a.Y, a.g, mu, i, y);
+    // the link's own terms: E^dag G' + G_Omega^dag C
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        go.d[k] = -go.d[k];
+        go.o[k] = cx<T>{-go.o[k].re, -go.o[k].im};
+    }
+    anti_mul_acc(gu, go, C);
+    st(a.out, a.g, mu, i, gu);
+}
+
+// Adds to the gradient of link (y, nu) the staple terms: for every mu != nu, the link sits in
+//   C_mu(y)       as the first factor of the upper staple      -> Y_mu(y) U_nu(y+mu) U_mu(y+nu)^dag
+//   C_mu(y+nu)    as the first factor of the lower staple      -> U_mu(y) U_nu(y+mu) Y_mu(y+nu)^dag
+//   C_nu(y+mu)    as the middle factor of the lower staple     -> U_mu(y) Y_nu(y+mu) U_mu(y+nu)^dag
+//   C_mu(y-mu)    as the last factor of the upper staple       -> Y_mu(y-mu)^dag U_nu(y-mu) U_mu(y-mu+nu)
+//   C_mu(y-mu+nu) as the last factor of the lower staple       -> U_mu(y-mu)^dag U_nu(y-mu) Y_mu(y-mu+nu)
+//   C_nu(y-mu)    as the middle factor of the upper staple     -> U_mu(y-mu)^dag Y_nu(y-mu) U_mu(y-mu+nu)
+// with Y the gradient of the unweighted staple sums.
+template <typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_back_staples(const __grid_constant__ StoutArgs<T> a)
+{
+    const int nu = blockIdx.y;
+    const int i = blockIdx.x * kStoutBlock + threadIdx.x;
+    if (i >= a.g.V) return;
+    M3T<T> acc;
+    ld(a.out, a.g, nu, i, acc);
+#pragma unroll 1
+    for (int mu = 0; mu < 4; ++mu) {
+        if (mu == nu) continue;
+        const int yp = up(a.g, i, mu), yn = up(a.g, i, nu);
+        const int ym = down(a.g, i, mu), ymn = up(a.g, ym, nu);
+        M3T<T> p, q, t;
+        // forward side: U_nu(y+mu) shared by the first two terms
+        ld(a.U, a.g, nu, yp, p);   // U_nu(y+mu)
+        ld(a.U, a.g, mu, yn, q);   // U_mu(y+nu)
+        t = mul<false, true>(p, q);
+        ld(a.Y, a.g, mu, i, q);    // Y_mu(y)
+        mul_acc<false, false>(acc, q, t);
+        ld(a.U, a.g, mu, i, q);    // U_mu(y)
+        t = mul<false, false>(q, p);
+        ld(a.Y, a.g, mu, yn, p);   // Y_mu(y+nu)
+        mul_acc<false, true>(acc, t, p);
+        ld(a.Y, a.g, nu, yp, p);   // Y_nu(y+mu)
+        t = mul<false, false>(q, p);
+        ld(a.U, a.g, mu, yn, q);   // U_mu(y+nu)
+        mul_acc<false, true>(acc, t, q);
+        // backward side: U_mu(y-mu)^dag leads the last two terms
+        ld(a.U, a.g, nu, ym, p);   // U_nu(y-mu)
+        ld(a.U, a.g, mu, ymn, q);  // U_mu(y-mu+nu)
+        t = mul<false, false>(p, q);
+        ld(a.Y, a.g, mu, ym, q);   // Y_mu(y-mu)
+        mul_acc<true, false>(acc, q, t);
+        ld(a.Y, a.g, mu, ymn, q);  // Y_mu(y-mu+nu)
+        t = mul<false, false>(p, q);
+        ld(a.Y, a.g, nu, ym, p);   // Y_nu(y-mu)
+        ld(a.U, a.g, mu, ymn, q);  // U_mu(y-mu+nu)
+        mul_acc<false, false>(t, p, q);
+        ld(a.U, a.g, mu, ym, p);   // U_mu(y-mu)
+        mul_acc<true, false>(acc, p, t);
+    }
+    st(a.out, a.g, nu, i, acc);
+}
+
+// F = TA(U G^dag) in place over G
+template <typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_lie_force(const __grid_constant__ StoutArgs<T> a)
+{
+    const int mu = blockIdx.y;
+    const int i = blockIdx.x * kStoutBlock + threadIdx.x;
+    if (i >= a.g.V) return;
+    M3T<T> u, gr;
+    ld(a.U, a.g, mu, i, u);
+    ld(a.out, a.g, mu, i, gr);
+    st(a.out, a.g, mu, i, ta(mul<false, true>(u, gr)));
+}
+
+// ------------------------------------------------------------------ by shared plaquettes
+// The same step with every corner path made once per plaquette (plaq.cuh).  C U^dag is a sum over
+// the plaquettes of the link of closed loops at its start: for the upper plaquette of (x, mu)
+// P(mu, nu) P(nu, mu)^dag, whose anti-Hermitian part serves link (x, nu) with the opposite sign; for
+// the lower one Slo(mu, nu)(x-nu) U_mu(x)^dag.  Only the anti-Hermitian parts are needed (9 numbers).
+//
+// Chain rule: with W = rho G_Omega of every link fixed, dS is the change of Re tr of the plaquettes
+// when each link moves by Y = W U, so the gradient has the form of the rectangle force, with
+//   P'(mu, nu)(x) = (W_nu - W_mu)(x) P(mu, nu)(x) + U_nu(x) Y_mu(x+nu)
+//   G_mu(x) = E^dag G' + sum_nu [ P'(mu, nu)(x) U_nu(x+mu)^dag + P(mu, nu)(x) Y_nu(x+mu)^dag
+//                               + U_nu(y)^dag P'(nu, mu)(y) ] - W_mu(x) sum_nu Slo(mu, nu)(y),  y = x - nu.
+//
+// ~1450 FP64 multiply-adds per link and smearing step (k_stout_fwd ~2300) and ~3700 per step of the
+// chain rule (k_stout_back_* ~6850), both at the FP64 pipe's rate (0.58e12/s): two steps of 16^3x32
+// 4.59 -> 2.65 ms, of the chain rule on 20x12x28x16 10.7 -> 5.7 ms.
+template <typename T>
+struct StoutPlaqArgs {
+    using C = typename C2<T>::type;
+    LinkGeo g;
+    T rho;
+    const C *U;    // links of this step
+    const C *G;    // gradient of the step's output (backward)
+    C *out;        // smeared links / gradient of U
+    T *K, *Lo;     // anti-Hermitian loops: upper per plane [6], lower per ordered pair [12] (based at x)
+    C *P, *Slo, *Pb;  // per ordered pair [12] (backward)
+    T *W;          // [4] rho G_Omega, anti-Hermitian
+    C *Y;          // [4] W U
+    const C *proj;  // last step of kind 0: the links for F = TA(U G^dag); null otherwise
+};
+
+template <bool BWD, typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_loops(const __grid_constant__ StoutPlaqArgs<T> a)
+{
+    pdl_enter();
+    const int x = blockIdx.x * kStoutBlock + threadIdx.x, V = a.g.V;
+    if (x >= V) return;
+    const int p = blockIdx.y;
+    int m, n;
+    plane_dirs(p, m, n);
+    const int xm = up(a.g, x, m), xn = up(a.g, x, n);
+    const M3T<T> pmn = mul<false, false>(link_at<T>(a.U, a.g, n, x), link_at<T>(a.U, a.g, m, xn));
+    const M3T<T> pnm = mul<false, false>(link_at<T>(a.U, a.g, m, x), link_at<T>(a.U, a.g, n, xm));
+    if (BWD) {
+        ws_st(a.P, V, 2 * p, x, pmn);
+        ws_st(a.P, V, 2 * p + 1, x, pnm);
+    }
+    ws_st9(a.K, V, p, x, anti_mul<false, true>(pmn, pnm));
+    M3T<T> s = mul<true, false>(link_at<T>(a.U, a.g, n, x), pnm);  // Slo(m, n): of link (x+n, m)
+    if (BWD) ws_st(a.Slo, V, 2 * p, x, s);
+    ws_st9(a.Lo, V, 2 * p, x, anti_mul<false, true>(s, link_at<T>(a.U, a.g, m, xn)));
+    s = mul<true, false>(link_at<T>(a.U, a.g, m, x), pmn);  // Slo(n, m): of link (x+m, n)
+    if (BWD) ws_st(a.Slo, V, 2 * p + 1, x, s);
+    ws_st9(a.Lo, V, 2 * p + 1, x, anti_mul<false, true>(s, link_at<T>(a.U, a.g, n, xm)));
+}
+
+// Q = -i TA(C U^dag) of link (x, mu) from its loops
+template <typename T>
+__device__ __forceinline__ plaq::H9<T> loops_q(const StoutPlaqArgs<T> &a, int mu, int x)
+{
+    H9<T> z;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        z.d[k] = T(0);
+        z.o[k] = cx<T>{T(0), T(0)};
+    }
+#pragma unroll 1
+    for (int nu = 0; nu < 4; ++nu) {
+        if (nu == mu) continue;
+        axpy9(z, mu < nu ? T(1) : T(-1), ws_ld9(a.K, a.g.V, plane_of(mu, nu), x));
+        axpy9(z, T(1), ws_ld9(a.Lo, a.g.V, slot_of(mu, nu), down(a.g, x, nu)));
+    }
+    return q_of(z, a.rho);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_apply(const __grid_constant__ StoutPlaqArgs<T> a)
+{
+    pdl_enter();
+    const int mu = blockIdx.y, x = blockIdx.x * kStoutBlock + threadIdx.x;
+    if (x >= a.g.V) return;
+    const H9<T> q = loops_q(a, mu, x), q2 = square9(q);
+    T c0, c1;
+    char_coefs9(q, q2, c0, c1);
+    const ExpCoefT<T> e = exp_sums<false>(c0, c1);
+    const M3T<T> u = mul<false, false>(poly9(e.f, q, q2), link_at<T>(a.U, a.g, mu, x));
+    st(a.out, a.g, mu, x, u);
+}
+
+// per link: E^dag G' into out, W and Y
+template <typename T>
+__global__ void __launch_bounds__(kStoutBlock) k_stout_grad_exp(const __grid_constant__ StoutPlaqArgs<T> a)
+{
+    pdl_enter();
+    const int mu = blockIdx.y, x = blockIdx.x * kStoutBlock + threadIdx.x, V = a.g.V;
+    if (x >= V) return;
+    M3T<T> gu;
+    H9<T> w;
+    const M3T<T> u = link_at<T>(a.U, a.g, mu, x);
+    exp_gradient(loops_q(a, mu, x), u, link_at<T>(a.G, a.g, mu, x), a.rho, gu, w);
+    st(a.out, a.g, mu, x, gu);
     ws_st9(a.W, V, mu, x, w);
     M3T<T> y = zero3<T>();
     anti_mul_acc(y, w, u);
@@ -425,7 +377,6 @@ __global__ void __launch_bounds__(kStoutBlock) k_stout_grad_exp(const __grid_con
 template <typename T>
 __global__ void __launch_bounds__(kStoutBlock) k_stout_bent(const __grid_constant__ StoutPlaqArgs<T> a)
 {
-    using namespace plaq;
     pdl_enter();
     const int x = blockIdx.x * kStoutBlock + threadIdx.x, V = a.g.V;
     if (x >= V) return;
@@ -444,7 +395,6 @@ __global__ void __launch_bounds__(kStoutBlock) k_stout_bent(const __grid_constan
 template <typename T>
 __global__ void __launch_bounds__(kStoutBlock) k_stout_gather(const __grid_constant__ StoutPlaqArgs<T> a)
 {
-    using namespace plaq;
     pdl_enter();
     const int mu = blockIdx.y, x = blockIdx.x * kStoutBlock + threadIdx.x, V = a.g.V;
     if (x >= V) return;
@@ -461,12 +411,7 @@ __global__ void __launch_bounds__(kStoutBlock) k_stout_gather(const __grid_const
     }
     anti_mul_acc(G, ws_ld9(a.W, V, mu, x), S);
     if (a.proj) G = expand_anti_traceless(anti_mul<false, true>(link_at<T>(a.proj, a.g, mu, x), G));
-    typename C2<T>::type *o = a.out + ((long long)mu * V + x) * 9;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        o[k].x = G.m[k / 3][k % 3].re;
-        o[k].y = G.m[k / 3][k % 3].im;
-    }
+    st(a.out, a.g, mu, x, G);
 }
 
 stg_status check_common(const stg_lattice *lat, int nstep, double rho, const char *fn)
@@ -495,7 +440,7 @@ E *take(char *&p, int V, int count)
 }
 
 // Whether the steps go by shared plaquettes.  FP32 stays with the per-link kernels, which are not
-// bound by their products (32^4 chain rule: 4.1 ms against 5.1 ms shared).  In FP64 every warp has a
+// bound by their products (32^4 chain rule: 3.5 ms against 5.1 ms shared).  In FP64 every warp has a
 // quarter SM's pipe to itself while a launch has no more warps than quarters; the one window where
 // the per-link kernels fit that once and the 6 planes of a site do not (3243 to 4864 sites on 152
 // SMs) is theirs: 8^4 smears in 191 us against 220 us, 6^4 (191 against 94) and 5120 sites (351
@@ -525,7 +470,7 @@ bool smear_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
     }
     StoutPlaqArgs<T> a;
     memset(&a, 0, sizeof(a));
-    a.g = plaq::plaq_geo(lat->g);
+    a.g = link_geo(lat->g);
     a.rho = (T)rho;
     w = ws;
     a.K = take<T>(w, a.g.V, 6);
@@ -561,7 +506,7 @@ bool force_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
     }
     StoutPlaqArgs<T> a;
     memset(&a, 0, sizeof(a));
-    a.g = plaq::plaq_geo(lat->g);
+    a.g = link_geo(lat->g);
     a.rho = (T)rho;
     w = ws;
     a.K = take<T>(w, a.g.V, 6);

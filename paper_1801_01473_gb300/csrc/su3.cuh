@@ -29,9 +29,9 @@ struct C2<float> {
 };
 
 struct LinkGeo {
-    int L[4];
-    long long stride[4];
-    long long V;
+    int L[4], stride[4];
+    int V;
+    FastDiv by_stride[4], by_L[4];
 };
 
 inline LinkGeo link_geo(const Geom &geo)
@@ -40,25 +40,34 @@ inline LinkGeo link_geo(const Geom &geo)
     long long s = 1;
     for (int mu = 0; mu < 4; ++mu) {
         g.L[mu] = geo.L[mu];
-        g.stride[mu] = s;
-        s *= g.L[mu];
+        g.stride[mu] = (int)s;
+        g.by_stride[mu] = make_fast_div((unsigned)s);
+        g.by_L[mu] = make_fast_div((unsigned)geo.L[mu]);
+        s *= geo.L[mu];
     }
-    g.V = s;
+    g.V = (int)s;
     return g;
 }
 
-// lexicographic index of x + step * mu (periodic; |step| <= L_mu)
-__device__ __forceinline__ long long nb(const LinkGeo &g, long long i, int mu, int step)
+// coordinate mu of site i
+__device__ __forceinline__ int coord(const LinkGeo &g, int i, int mu)
 {
-    const int xm = (int)((i / g.stride[mu]) % g.L[mu]);
-    long long j = i + step * g.stride[mu];
-    if (xm + step >= g.L[mu]) j -= g.L[mu] * g.stride[mu];
-    if (xm + step < 0) j += g.L[mu] * g.stride[mu];
-    return j;
+    const int q = fast_div(i, g.by_stride[mu]);
+    return q - fast_div(q, g.by_L[mu]) * g.L[mu];
+}
+
+// neighbours of site i along mu (periodic)
+__device__ __forceinline__ int up(const LinkGeo &g, int i, int mu)
+{
+    return coord(g, i, mu) == g.L[mu] - 1 ? i - (g.L[mu] - 1) * g.stride[mu] : i + g.stride[mu];
+}
+__device__ __forceinline__ int down(const LinkGeo &g, int i, int mu)
+{
+    return coord(g, i, mu) == 0 ? i + (g.L[mu] - 1) * g.stride[mu] : i - g.stride[mu];
 }
 
 template <typename T>
-__device__ __forceinline__ void ld(const typename C2<T>::type *__restrict__ base, const LinkGeo &g, int mu, long long i,
+__device__ __forceinline__ void ld(const typename C2<T>::type *__restrict__ base, const LinkGeo &g, int mu, int i,
                                    M3T<T> &a)
 {
     const typename C2<T>::type *p = base + ((long long)mu * g.V + i) * 9;
@@ -70,7 +79,7 @@ __device__ __forceinline__ void ld(const typename C2<T>::type *__restrict__ base
 }
 
 template <typename T>
-__device__ __forceinline__ void st(typename C2<T>::type *__restrict__ base, const LinkGeo &g, int mu, long long i,
+__device__ __forceinline__ void st(typename C2<T>::type *__restrict__ base, const LinkGeo &g, int mu, int i,
                                    const M3T<T> &a)
 {
     typename C2<T>::type *p = base + ((long long)mu * g.V + i) * 9;
@@ -142,49 +151,91 @@ struct ExpCoefT {
 };
 using ExpCoef = ExpCoefT<double>;
 
-template <bool DERIV, typename T>
-__device__ ExpCoefT<T> exp_coef(T c0, T c1)
+// 1/n!, n = 0..131
+template <typename T>
+struct InvFactorial {
+    T v[132];
+    constexpr InvFactorial() : v{}
+    {
+        double f = 1.0;
+        for (int n = 0; n < 132; ++n) {
+            v[n] = f < (sizeof(T) == 4 ? 1e-37 : 0.0) ? T(0) : (T)f;
+            f /= n + 1;
+        }
+    }
+};
+__constant__ constexpr InvFactorial<double> kInvFactorial64{};
+__constant__ constexpr InvFactorial<float> kInvFactorial32{};
+template <typename T>
+__device__ __forceinline__ T inv_factorial(int n)
 {
-    ExpCoefT<T> e;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) e.f[j] = e.d0[j] = e.d1[j] = cx<T>{T(0), T(0)};
-    e.f[0].re = T(1);  // n = 0
-    T a = T(1), b = T(0), c = T(0);                                     // Q^n = a + b Q + c Q^2
-    T a0 = T(0), b0 = T(0), cc0 = T(0), a1 = T(0), b1 = T(0), cc1 = T(0);  // d/dc0, d/dc1
-    T r = sqrt(fmax(T(2) * c1, T(0)));                                  // >= spectral radius of Q
-    if (r < T(1)) r = T(1);
-    // remaining terms of the coefficients (and of their c-derivatives, polynomial in n times
-    // r^n/n!) below the precision's resolution
-    const T stop = sizeof(T) == 4 ? T(1e-9) : T(1e-18);
-    T w = T(1), bound = T(1);                                            // 1/n!, r^n/n!
+    return sizeof(T) == 8 ? (T)kInvFactorial64.v[n] : (T)kInvFactorial32.v[n];
+}
+
+// exp(iQ) = f0 + f1 Q + f2 Q^2 with (DERIV) the derivatives of the f_j, from one sequence.
+// Q^3 = c1 Q + c0 gives Q^n = c0 h_{n-1} + h_{n+1} Q + h_n Q^2 (n >= 1) with
+//   h_0 = h_1 = 0, h_2 = 1, h_{n+1} = c1 h_{n-1} + c0 h_{n-2},
+// and g_n = dh_n/dc0 satisfies dh_n/dc1 = g_{n+1} (both from the generating function
+// t^2 / (1 - c1 t^2 - c0 t^3)), g_{n+1} = c1 g_{n-1} + c0 g_{n-2} + h_{n-2}.  So with s_n = i^n / n!
+//   f2 = sum s_n h_n, f1 = sum s_n h_{n+1}, f0 = 1 + c0 sum s_n h_{n-1},
+//   df2/dc0 = sum s_n g_n,  df2/dc1 = df1/dc0 = sum s_n g_{n+1},  df1/dc1 = sum s_n g_{n+2},
+//   df0/dc0 = sum s_n h_{n-1} + c0 sum s_n g_{n-1},  df0/dc1 = c0 df2/dc0:
+// 5 (12 with derivatives) multiply-adds per term, no divisions.  The number of terms is settled
+// beforehand in FP32: the rest of the coefficients, and of their derivatives (polynomial in n times
+// r^n/n!, r >= the spectral radius of Q), lies below the precision's resolution.
+template <bool DERIV, typename T>
+__device__ __forceinline__ ExpCoefT<T> exp_sums(T c0, T c1)
+{
+    int nmax = 6;
+    {
+        const float stop = sizeof(T) == 4 ? 1e-9f : 1e-18f;
+        float r = sqrtf(fmaxf(2.f * (float)c1, 0.f));
+        if (!(r >= 1.f)) r = 1.f;
+        float bound = 1.f;  // r^n / n!
+        for (int n = 1; n < 128; ++n) {
+            bound *= __fdividef(r, (float)n);
+            const float m = (float)(n + 1);
+            nmax = n;
+            if (n >= 6 && bound * m * m * m < stop) break;
+        }
+    }
+    T hm = T(0), h = T(0), hp = T(1);               // h_{n-1}, h_n, h_{n+1} at n = 1
+    T gm = T(0), g = T(0), gp = T(0), gpp = T(0);               // g_{n-1}, g_n, g_{n+1}, g_{n+2}
+    T s0[2] = {T(0), T(0)}, s1[2] = {T(0), T(0)}, s2[2] = {T(0), T(0)};  // sums of h_{n-1}, h_n, h_{n+1}; [1] odd n
+    T d0[2] = {T(0), T(0)}, d1[2] = {T(0), T(0)}, d2[2] = {T(0), T(0)}, d3[2] = {T(0), T(0)};  // g_{n-1} .. g_{n+2}
 #pragma unroll 1
-    for (int n = 1; n < 128; ++n) {
-        if (DERIV) {
-            const T na0 = c + c0 * cc0, nb0 = a0 + c1 * cc0, nc0 = b0;
-            const T na1 = c0 * cc1, nb1 = a1 + c + c1 * cc1, nc1 = b1;
-            a0 = na0; b0 = nb0; cc0 = nc0; a1 = na1; b1 = nb1; cc1 = nc1;
-        }
-        const T na = c0 * c, nb = a + c1 * c, nc = b;
-        a = na; b = nb; c = nc;
-        w /= T(n);
-        bound *= r / T(n);
-        // i^n / n!
-        const T s = (n & 2) ? -w : w;
-        if (n & 1) {
-            e.f[0].im += s * a; e.f[1].im += s * b; e.f[2].im += s * c;
+    for (int n0 = 1; n0 <= nmax; n0 += 4) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {  // n = n0 + u = 1 + u mod 4: i^n = i, -1, -i, 1
+            T s = inv_factorial<T>(n0 + u);
+            if (u == 1 || u == 2) s = -s;
+            const int o = (u & 1) ? 0 : 1;
+            s0[o] = fma(s, hm, s0[o]);
+            s1[o] = fma(s, h, s1[o]);
+            s2[o] = fma(s, hp, s2[o]);
             if (DERIV) {
-                e.d0[0].im += s * a0; e.d0[1].im += s * b0; e.d0[2].im += s * cc0;
-                e.d1[0].im += s * a1; e.d1[1].im += s * b1; e.d1[2].im += s * cc1;
+                d0[o] = fma(s, gm, d0[o]);
+                d1[o] = fma(s, g, d1[o]);
+                d2[o] = fma(s, gp, d2[o]);
+                d3[o] = fma(s, gpp, d3[o]);
+                const T gn = fma(c1, gp, fma(c0, g, h));  // g_{n+3}
+                gm = g; g = gp; gp = gpp; gpp = gn;
             }
-        } else {
-            e.f[0].re += s * a; e.f[1].re += s * b; e.f[2].re += s * c;
-            if (DERIV) {
-                e.d0[0].re += s * a0; e.d0[1].re += s * b0; e.d0[2].re += s * cc0;
-                e.d1[0].re += s * a1; e.d1[1].re += s * b1; e.d1[2].re += s * cc1;
-            }
+            const T hn = fma(c1, h, c0 * hm);  // h_{n+2}
+            hm = h; h = hp; hp = hn;
         }
-        const T m = T(n + 1);
-        if (n >= 6 && bound * m * m * m < stop) break;
+    }
+    ExpCoefT<T> e;
+    e.f[0] = cx<T>{fma(c0, s0[0], T(1)), c0 * s0[1]};
+    e.f[1] = cx<T>{s2[0], s2[1]};
+    e.f[2] = cx<T>{s1[0], s1[1]};
+    if (DERIV) {
+        e.d0[0] = cx<T>{fma(c0, d0[0], s0[0]), fma(c0, d0[1], s0[1])};
+        e.d0[1] = cx<T>{d2[0], d2[1]};
+        e.d0[2] = cx<T>{d1[0], d1[1]};
+        e.d1[0] = cx<T>{c0 * d1[0], c0 * d1[1]};
+        e.d1[1] = cx<T>{d3[0], d3[1]};
+        e.d1[2] = cx<T>{d2[0], d2[1]};
     }
     return e;
 }

@@ -55,3 +55,14 @@ def test_several_passes():
     tr = torch.diagonal(want, dim1=-2, dim2=-1).sum(-1)[..., None, None] / 3
     want = want - tr * torch.eye(3, device="cuda")
     assert float((force - want).abs().max()) <= 1e-13 * float(z.abs().max())
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 10, 4, 14)])
+@pytest.mark.parametrize("kind", [0, 1])
+def test_single_precision_matches_loops(dims, kind):
+    """The per-link kernel (FP32), whose factors are grouped too: 2^-24 in place of 2^-53 above."""
+    import paper_1801_01473_gb300 as p
+    u = S.gauge_links(dims, "haar", 154).astype(np.complex64)
+    want = og.gradient(dims, u, BETA) if kind == 1 else og.force(dims, u, BETA)
+    got = p.gauge_force(p.Lattice(dims), _gpu(u), BETA, kind=kind).cpu().numpy()
+    assert np.abs(got - want).max() <= 24 * 5 * 8 * 2.0**-24 * np.abs(want).max()
