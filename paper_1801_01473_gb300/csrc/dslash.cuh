@@ -33,6 +33,8 @@ __host__ __device__ inline int dslash_partials(int Vh) { return (Vh + kPartialSi
 struct DGroup {
     Geom g;
     const void *links;
+    const void *fx_links;  // fixed-point copy of F64 18-real links (set_fx), or null
+    const int *fx_bad;     // device flag beside it: nonzero when some link has no fixed-point form
     int nrhs;
     const void *in[kMaxRhs];
     void *out[kMaxRhs];

@@ -1145,6 +1145,7 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
             memset(&Goe, 0, sizeof(Goe));
             Goe.g = ii[k].gi->g;
             Goe.links = ii[k].gi->links;
+            set_fx(Goe, ii[k].gi, ws);
             Goe.nrhs = std::min(kMaxRhs, ii[k].nrhs - r0);
             Geo = Goe;
             for (int j = 0; j < Goe.nrhs; ++j) {
@@ -1176,10 +1177,13 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
             memset(&Goe, 0, sizeof(Goe));
             Goe.g = ii[k].gr->g;
             Goe.links = ii[k].gr->links;
+            set_fx(Goe, ii[k].gr, ws);
             Goe.nrhs = std::min(rg, cnt - q0);
             Geo = Goe;
             Hoe = Goe;
             Hoe.links = ii[k].gh->links;
+            Hoe.fx_links = nullptr;
+            set_fx(Hoe, ii[k].gh, ws);
             Heo = Hoe;
             for (int j = 0; j < Goe.nrhs; ++j) {
                 const int pidx = first + q0 + j;
@@ -1221,6 +1225,8 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
                 add_group(pinc.eo, Ieo, 0);
             }
             Hoe.links = Heo.links = ii[k].g64->links;
+            set_fx(Hoe, ii[k].g64, ws);
+            set_fx(Heo, ii[k].g64, ws);
             add_group(p64f.oe, Hoe, 1);
             add_group(p64f.eo, Heo, 0);
         }

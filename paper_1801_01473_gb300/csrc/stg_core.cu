@@ -104,12 +104,15 @@ static cudaError_t launch_dslash_tuned(int kind, const DArgs &a, int mode, cudaS
 // Double-single D is bound by the FP32 pipes, not by link traffic: several right-hand sides per
 // thread only cost registers and occupancy (measured: 4 rhs per thread run at half the per-rhs
 // speed of 1).  Its multi-rhs launches are therefore split into one-rhs groups, and so are those
-// of links with a U(1) phase field (instantiated for one rhs only).
+// of fixed-point FP64 links (bound by the integer pipes: 32^4, 4 rhs per thread 209 us a rhs against
+// 152 us) and of links with a U(1) phase field (instantiated for one rhs only).
 cudaError_t launch_dslash(int kind, const DArgs &a, int mode, cudaStream_t st)
 {
     int maxv, maxr;
     dslash_extent(a, maxv, maxr);
-    if ((!kind_is_ds(kind) && !kind_has_u1(kind)) || maxr <= 1) return launch_dslash_tuned(kind, a, mode, st);
+    bool fx = kind == kF64R18;
+    for (int k = 0; k < a.ngroups; ++k) fx = fx && a.grp[k].fx_links;
+    if ((!kind_is_ds(kind) && !kind_has_u1(kind) && !fx) || maxr <= 1) return launch_dslash_tuned(kind, a, mode, st);
     DArgs b;
     memset(&b, 0, sizeof(b));
     b.out_par = a.out_par;
@@ -428,6 +431,7 @@ stg_status ds_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge *
         g->links = nullptr;
         g->f32_copy = nullptr;
         g->ds_copy = nullptr;
+        g->fx_links = nullptr;
         cudaError_t e = cudaMalloc(&g->links, g->bytes);
         if (e == cudaSuccess) e = cudaMalloc(&g->scratch, g->scratch_count * sizeof(double));
         if (e == cudaSuccess) e = fill_ds_companion(g64, g, st);
@@ -441,6 +445,36 @@ stg_status ds_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge *
     }
     *out = g64->ds_copy;
     return STG_OK;
+}
+
+static int *fx_flag(const stg_gauge *g) { return reinterpret_cast<int *>(static_cast<char *>(g->fx_links) + g->bytes); }
+
+void set_fx(DGroup &G, const stg_gauge *g, cudaStream_t st)
+{
+    // a lattice below 2048 sites is bound by the launch (4^4 15 us against 11 us in fixed point): not
+    // worth the copy
+    if (g->kind != kF64R18 || g->lat->V < 2048) return;
+    std::lock_guard<std::mutex> lk(g_companion_mu);
+    if (!g->fx_links) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return;
+        }
+        // same bytes per link as the FP64 layout, the flag behind them
+        cudaError_t e = cudaMalloc(&g->fx_links, g->bytes + 256);
+        if (e == cudaSuccess) e = launch_links_to_fx(g->g.Vh, g->links, g->fx_links, fx_flag(g), st);
+        // other streams may use the copy from now on
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(g->fx_links);
+            g->fx_links = nullptr;
+            return;
+        }
+    }
+    G.fx_links = g->fx_links;
+    G.fx_bad = fx_flag(g);
 }
 
 stg_status f32_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge **out)
@@ -458,6 +492,7 @@ stg_status f32_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge 
         g->links = nullptr;
         g->f32_copy = nullptr;
         g->ds_copy = nullptr;
+        g->fx_links = nullptr;
         cudaError_t e = cudaMalloc(&g->links, g->bytes);
         if (e == cudaSuccess) e = cudaMalloc(&g->scratch, g->scratch_count * sizeof(double));
         if (e == cudaSuccess) e = fill_f32_companion(g64, g, st);
@@ -679,6 +714,7 @@ static stg_status gauge_create(const stg_lattice *lat, const void *links_c128_de
     g->scratch = nullptr;
     g->f32_copy = nullptr;
     g->ds_copy = nullptr;
+    g->fx_links = nullptr;
     g->scratch_count = (size_t)dslash_partials(lat->g.Vh);
     cudaError_t e = cudaMalloc(&g->links, g->bytes);
     if (e == cudaSuccess) e = cudaMalloc(&g->scratch, g->scratch_count * sizeof(double));
@@ -717,6 +753,7 @@ stg_status stg_gauge_update(stg_gauge *g, const void *links_c128_dev, const doub
     std::lock_guard<std::mutex> lk(g_companion_mu);
     if (g->ds_copy) STG_CUDA_TRY(fill_ds_companion(g, g->ds_copy, st));
     if (g->f32_copy) STG_CUDA_TRY(fill_f32_companion(g, g->f32_copy, st));
+    if (g->fx_links) STG_CUDA_TRY(launch_links_to_fx(g->g.Vh, g->links, g->fx_links, fx_flag(g), st));
     return STG_OK;
 }
 
@@ -734,6 +771,7 @@ void stg_gauge_destroy(stg_gauge *g)
     if (g->f32_copy) stg_gauge_destroy(g->f32_copy);
     if (g->ds_copy) stg_gauge_destroy(g->ds_copy);
     cudaFree(g->links);
+    cudaFree(g->fx_links);
     cudaFree(g->scratch);
     delete g;
 }
@@ -816,6 +854,7 @@ stg_status stg_dslash_multi(const stg_gauge *g, int32_t out_parity, int32_t nrhs
             DGroup &G = a.grp[ng++];
             G.g = g->g;
             G.links = g->links;
+            set_fx(G, g, (cudaStream_t)stream);
             G.nrhs = (nrhs - base) < kMaxRhs ? (nrhs - base) : kMaxRhs;
             for (int j = 0; j < G.nrhs; ++j) {
                 G.in[j] = ib + (size_t)(base + j) * stride_bytes;
@@ -862,6 +901,7 @@ stg_status stg_normal_op(const stg_gauge *g, double mass, double shift, void *ou
     DGroup &G = a.grp[0];
     G.g = g->g;
     G.links = g->links;
+    set_fx(G, g, st);
     G.nrhs = 1;
     // D_oe: even -> odd
     a.out_par = 1;
