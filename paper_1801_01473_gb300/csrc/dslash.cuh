@@ -22,14 +22,14 @@
 namespace stg {
 
 constexpr int kMaxRhs = 8;
-constexpr int kMaxGroups = 16;  // groups per launch (blockIdx.y): a DArgs of 16 groups is ~8.5 KB of kernel parameters
+constexpr int kMaxGroups = 16;  // groups per launch (gridDim.y): a DArgs of 16 groups is ~8.5 KB of kernel parameters
 constexpr int kDslashBlock = 128;   // default block; the autotuner may pick 64, 128 or 256
 constexpr int kPartialSites = 64;   // one FP64 partial per 64 output sites, whatever the block size
 
 // Number of FP64 partial sums an epilogue launch writes for a lattice of Vh sites per parity.
 __host__ __device__ inline int dslash_partials(int Vh) { return (Vh + kPartialSites - 1) / kPartialSites; }
 
-// A set of right-hand sides on one lattice and gauge.  blockIdx.y selects the group.
+// A set of right-hand sides on one lattice and gauge; a launch has gridDim.y of them.
 struct DGroup {
     Geom g;
     const void *links;
@@ -65,6 +65,21 @@ __device__ __forceinline__ void lazy_mac(float &hi, float &lo, const dsf &a, con
     lo = __fadd_rn(lo, __fadd_rn(err, e));
 }
 
+// Block index bx along the output sites and group of this thread block.  The groups of a launch are
+// dealt out in turn, so that blocks of all groups on the same sites run together: groups on one
+// gauge then read each link from DRAM once and from L2 for the others.
+// 12 double-single D on 24^3x32 493 -> 405 us (one group after the other re-read 255 MB of links for each).
+struct BlockPos {
+    int bx, group;
+};
+__device__ __forceinline__ BlockPos block_pos()
+{
+    const unsigned ng = gridDim.y;
+    if (ng == 1) return BlockPos{(int)blockIdx.x, 0};
+    const unsigned id = blockIdx.y * gridDim.x + blockIdx.x;
+    return BlockPos{(int)(id / ng), (int)(id % ng)};
+}
+
 template <typename R>
 __device__ __forceinline__ void neg3(cx<R> v[3])
 {
@@ -76,7 +91,7 @@ __device__ __forceinline__ void neg3(cx<R> v[3])
 // partial sums (MODE 1, 2), store, and write one partial per 64 output sites.  `sh` holds >= 32
 // doubles of shared memory; `act` is uniform over the block.
 template <typename R, int NRHS, int MODE, int BS>
-__device__ __forceinline__ void dslash_epilogue(const DGroup &G, const bool act[NRHS], bool live, int h,
+__device__ __forceinline__ void dslash_epilogue(const DGroup &G, int bx, const bool act[NRHS], bool live, int h,
                                                 const cx<R> acc[NRHS][3], double *sh,
                                                 const cx<R> (*pre_p)[3] = nullptr)
 {
@@ -128,7 +143,7 @@ __device__ __forceinline__ void dslash_epilogue(const DGroup &G, const bool act[
             if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = pv;
             __syncthreads();
             constexpr int kChunks = BS / kPartialSites;
-            const int c = blockIdx.x * kChunks + threadIdx.x;
+            const int c = bx * kChunks + threadIdx.x;
             if (threadIdx.x < kChunks && c < dslash_partials(G.g.h_end - G.g.h_begin))
                 G.partial[j][c] = sh[2 * threadIdx.x] + sh[2 * threadIdx.x + 1];
         }
@@ -238,10 +253,12 @@ __global__ void __launch_bounds__(BS) k_dslash(const __grid_constant__ DArgs a)
 {
     using R = typename LinkT::R;
     pdl_enter();
-    const DGroup &G = a.grp[blockIdx.y];
+    const BlockPos pos = block_pos();
+    const int bx = pos.bx;
+    const DGroup &G = a.grp[pos.group];
     const int Vh = G.g.Vh;
     const int nout = G.g.h_end - G.g.h_begin;
-    if ((int)(blockIdx.x * BS) >= nout) return;  // block-uniform
+    if (bx * BS >= nout) return;  // block-uniform
 
     bool act[NRHS];
     bool any = false;
@@ -252,7 +269,7 @@ __global__ void __launch_bounds__(BS) k_dslash(const __grid_constant__ DArgs a)
     }
     if (!any) return;  // block-uniform
 
-    const int h = G.g.h_begin + blockIdx.x * BS + threadIdx.x;
+    const int h = G.g.h_begin + bx * BS + threadIdx.x;
     const bool live = h < G.g.h_end;
     const int op = a.out_par;
 
@@ -327,7 +344,7 @@ __global__ void __launch_bounds__(BS) k_dslash(const __grid_constant__ DArgs a)
             cx<float> pre_p[NRHS][3];
             if (live) dslash_hops_ahead_f32r12<NRHS, MODE>(G, op, h, site_of(G.g, op, h), act, acc, pre_p);
             __shared__ double sh[32];
-            dslash_epilogue<R, NRHS, MODE, BS>(G, act, live, h, acc, sh, MODE != 0 ? pre_p : nullptr);
+            dslash_epilogue<R, NRHS, MODE, BS>(G, bx, act, live, h, acc, sh, MODE != 0 ? pre_p : nullptr);
             return;
         }
     } else if (live) {
@@ -380,7 +397,7 @@ __global__ void __launch_bounds__(BS) k_dslash(const __grid_constant__ DArgs a)
     }
 
     __shared__ double sh[32];
-    dslash_epilogue<R, NRHS, MODE, BS>(G, act, live, h, acc, sh);
+    dslash_epilogue<R, NRHS, MODE, BS>(G, bx, act, live, h, acc, sh);
 }
 
 // Shared-link variant for groups of several right-hand sides on FP32 / 16-bit links (R = float).
@@ -403,11 +420,13 @@ __global__ void __launch_bounds__(512) k_dslash_sh(const __grid_constant__ DArgs
     int *sh_nb = reinterpret_cast<int *>(sh_links + 8 * 18 * kShSites);
     __shared__ double sh_part[16];
     pdl_enter();
-    const DGroup &G = a.grp[blockIdx.y];
+    const BlockPos pos = block_pos();
+    const int bx = pos.bx;
+    const DGroup &G = a.grp[pos.group];
     const int Vh = G.g.Vh;
     const int nout = G.g.h_end - G.g.h_begin;
-    if ((int)(blockIdx.x * kShSites) >= nout) return;  // block-uniform
-    const int h0 = G.g.h_begin + blockIdx.x * kShSites;
+    if (bx * kShSites >= nout) return;  // block-uniform
+    const int h0 = G.g.h_begin + bx * kShSites;
     const int hend = G.g.h_end;
     const int op = a.out_par;
     // stage the links: hop k = 2 mu (forward) or 2 mu + 1 (backward) of site s
@@ -503,7 +522,7 @@ __global__ void __launch_bounds__(512) k_dslash_sh(const __grid_constant__ DArgs
         const int jj = threadIdx.x;  // one thread per rhs writes its 64-site partial
         if (jj < G.nrhs && 2 * jj + 1 < (int)(blockDim.x >> 5) && G.partial[jj] != nullptr &&
             !(G.skip[jj] != nullptr && *G.skip[jj] != 0))
-            G.partial[jj][blockIdx.x] = sh_part[2 * jj] + sh_part[2 * jj + 1];
+            G.partial[jj][bx] = sh_part[2 * jj] + sh_part[2 * jj + 1];
     }
 }
 

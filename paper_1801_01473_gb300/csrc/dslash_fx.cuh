@@ -115,12 +115,14 @@ template <int MODE, int BS>
 __global__ void __launch_bounds__(BS, (BS == 64 ? 512 : 640) / BS) k_dslash_fx(const __grid_constant__ DArgs a)
 {
     pdl_enter();
-    const DGroup &G = a.grp[blockIdx.y];
+    const BlockPos pos = block_pos();
+    const int bx = pos.bx;
+    const DGroup &G = a.grp[pos.group];
     const int Vh = G.g.Vh;
-    if ((int)(blockIdx.x * BS) >= G.g.h_end - G.g.h_begin) return;  // block-uniform
+    if (bx * BS >= G.g.h_end - G.g.h_begin) return;  // block-uniform
     if (G.nrhs < 1 || (G.skip[0] != nullptr && *G.skip[0] != 0)) return;  // block-uniform
 
-    const int h = G.g.h_begin + blockIdx.x * BS + threadIdx.x;
+    const int h = G.g.h_begin + bx * BS + threadIdx.x;
     const bool live = h < G.g.h_end;
     const int op = a.out_par;
     cx<double> acc[1][3];
@@ -214,7 +216,7 @@ __global__ void __launch_bounds__(BS, (BS == 64 ? 512 : 640) / BS) k_dslash_fx(c
 
     const bool act[1] = {true};
     __shared__ double sh[32];
-    dslash_epilogue<double, 1, MODE, BS>(G, act, live, h, acc, sh);
+    dslash_epilogue<double, 1, MODE, BS>(G, bx, act, live, h, acc, sh);
 }
 
 }  // namespace stg
