@@ -11,6 +11,7 @@
 // the number of 3x3 products decides their time and the extra memory traffic does not show.
 #pragma once
 
+#include "dslash.cuh"  // launch_pdl
 #include "su3.cuh"
 
 namespace stg {
@@ -65,6 +66,41 @@ __device__ __forceinline__ void ws_st(typename C2<T>::type *__restrict__ base, i
         v.y = a.m[k / 3][k % 3].im;
         p[(long long)k * V] = v;
     }
+}
+
+// link (mu, i) of canonical links or of a workspace of 4 fields
+template <bool WS, typename T>
+__device__ __forceinline__ M3T<T> link_of(const typename C2<T>::type *__restrict__ U, const LinkGeo &g, int mu, int i)
+{
+    if constexpr (WS) return ws_ld<T>(U, g.V, mu, i);
+    return link_at<T>(U, g, mu, i);
+}
+
+// Canonical links -> workspace of 4 fields, through shared memory so that both sides are contiguous.
+// A thread's 9 loads of a canonical FP32 link are 72 bytes apart between lanes and touch 18 lines
+// per instruction where the workspace's touch 2; the FP32 link kernels were bound by that.
+constexpr int kWsTile = 128;
+template <typename T>
+__global__ void __launch_bounds__(kWsTile) k_links_to_ws(const typename C2<T>::type *__restrict__ src,
+                                                         typename C2<T>::type *__restrict__ dst, int V)
+{
+    using C = typename C2<T>::type;
+    pdl_enter();
+    __shared__ C tile[kWsTile * 9];
+    const int i0 = blockIdx.x * kWsTile, n = min(kWsTile, V - i0), mu = blockIdx.y;
+    const C *s = src + ((long long)mu * V + i0) * 9;
+    for (int k = threadIdx.x; k < n * 9; k += kWsTile) tile[k] = s[k];
+    __syncthreads();
+    if ((int)threadIdx.x < n)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) dst[((long long)mu * 9 + k) * V + i0 + threadIdx.x] = tile[threadIdx.x * 9 + k];
+}
+
+template <typename T>
+cudaError_t links_to_ws(const void *links, typename C2<T>::type *ws, int V, cudaStream_t st)
+{
+    const dim3 tiles((unsigned)((V + kWsTile - 1) / kWsTile), 4);
+    return launch_pdl(k_links_to_ws<T>, tiles, dim3(kWsTile), st, static_cast<const typename C2<T>::type *>(links), ws, V);
 }
 
 // acc += w a

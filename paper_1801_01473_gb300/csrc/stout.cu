@@ -44,17 +44,17 @@ __device__ M3T<T> staple_sum(const typename C2<T>::type *__restrict__ U, const L
         if (nu == mu) continue;
         M3T<T> a, b, t;
         // U_nu(x) U_mu(x+nu) U_nu(x+mu)^dag
-        ld(U, g, nu, i, a);
-        ld(U, g, mu, up(g, i, nu), b);
+        a = link_at<T>(U, g, nu, i);
+        b = link_at<T>(U, g, mu, up(g, i, nu));
         t = mul<false, false>(a, b);
-        ld(U, g, nu, up(g, i, mu), a);
+        a = link_at<T>(U, g, nu, up(g, i, mu));
         mul_acc<false, true>(c, t, a);
         // U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)
         const int xm = down(g, i, nu);
-        ld(U, g, nu, xm, a);
-        ld(U, g, mu, xm, b);
+        a = link_at<T>(U, g, nu, xm);
+        b = link_at<T>(U, g, mu, xm);
         t = mul<true, false>(a, b);
-        ld(U, g, nu, up(g, xm, mu), a);
+        a = link_at<T>(U, g, nu, up(g, xm, mu));
         mul_acc<false, false>(c, t, a);
     }
 #pragma unroll
@@ -153,45 +153,60 @@ struct StoutArgs {
     LinkGeo g;
     T rho;
     const C *U;  // links of this step
+    const C *Uws;  // their workspace copy (WS)
     const C *G;  // gradient of the step's output (backward)
     C *out;      // smeared links (forward) / gradient of U (backward)
+    C *acc;      // the links' own gradient terms, between the backward kernels
     C *Y;        // rho G_Omega U (backward)
+    int g_canon, out_canon, proj;  // G, out canonical; last step of kind 0: F = TA(U G^dag) instead of G
 };
+
+template <bool WS, typename T>
+__device__ __forceinline__ void put(typename C2<T>::type *base, const LinkGeo &g, int mu, int i, const M3T<T> &a)
+{
+    if constexpr (WS)
+        ws_st(base, g.V, mu, i, a);
+    else
+        st(base, g, mu, i, a);
+}
 
 constexpr int kStoutBlock = 128;
 
 template <typename T>
 __global__ void __launch_bounds__(kStoutBlock) k_stout_fwd(const __grid_constant__ StoutArgs<T> a)
 {
+    pdl_enter();
     const int mu = blockIdx.y;
     const int i = blockIdx.x * kStoutBlock + threadIdx.x;
     if (i >= a.g.V) return;
     const M3T<T> u = link_at<T>(a.U, a.g, mu, i);
-    const H9<T> q = q_of(anti_mul<false, true>(staple_sum(a.U, a.g, mu, i, a.rho), u), T(1)), q2 = square9(q);
+    const H9<T> q = q_of(anti_mul<false, true>(staple_sum<T>(a.U, a.g, mu, i, a.rho), u), T(1)), q2 = square9(q);
     T c0, c1;
     char_coefs9(q, q2, c0, c1);
     const ExpCoefT<T> e = exp_sums<false>(c0, c1);
     st(a.out, a.g, mu, i, mul<false, false>(poly9(e.f, q, q2), u));
 }
 
-template <typename T>
+template <bool WS, typename T>
 __global__ void __launch_bounds__(kStoutBlock) k_stout_back_link(const __grid_constant__ StoutArgs<T> a)
 {
+    pdl_enter();
     const int mu = blockIdx.y;
     const int i = blockIdx.x * kStoutBlock + threadIdx.x;
     if (i >= a.g.V) return;
-    const M3T<T> C = staple_sum(a.U, a.g, mu, i, a.rho);
+    const M3T<T> C = staple_sum<T>(a.U, a.g, mu, i, a.rho);
     const M3T<T> u = link_at<T>(a.U, a.g, mu, i);
     M3T<T> gu;
     H9<T> go;
-    exp_gradient(q_of(anti_mul<false, true>(C, u), T(1)), u, link_at<T>(a.G, a.g, mu, i), T(1), gu, go);
+    const M3T<T> gp = WS && !a.g_canon ? ws_ld<T>(a.G, a.g.V, mu, i) : link_at<T>(a.G, a.g, mu, i);
+    exp_gradient(q_of(anti_mul<false, true>(C, u), T(1)), u, gp, T(1), gu, go);
     M3T<T> y = zero3<T>();
     anti_mul_acc(y, go, u);
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
         for (int c = 0; c < 3; ++c) y.m[r][c] = cx<T>{a.rho * y.m[r][c].re, a.rho * y.m[r][c].im};
-    st(a.Y, a.g, mu, i, y);
+    put<WS>(a.Y, a.g, mu, i, y);
     // the link's own terms: E^dag G' + G_Omega^dag C
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -199,7 +214,7 @@ __global__ void __launch_bounds__(kStoutBlock) k_stout_back_link(const __grid_co
         go.o[k] = cx<T>{-go.o[k].re, -go.o[k].im};
     }
     anti_mul_acc(gu, go, C);
-    st(a.out, a.g, mu, i, gu);
+    put<WS>(a.acc, a.g, mu, i, gu);
 }
 
 // Adds to the gradient of link (y, nu) the staple terms: for every mu != nu, the link sits in
@@ -210,14 +225,15 @@ __global__ void __launch_bounds__(kStoutBlock) k_stout_back_link(const __grid_co
 //   C_mu(y-mu+nu) as the last factor of the lower staple       -> U_mu(y-mu)^dag U_nu(y-mu) Y_mu(y-mu+nu)
 //   C_nu(y-mu)    as the middle factor of the upper staple     -> U_mu(y-mu)^dag Y_nu(y-mu) U_mu(y-mu+nu)
 // with Y the gradient of the unweighted staple sums.
-template <typename T>
-__global__ void __launch_bounds__(kStoutBlock) k_stout_back_staples(const __grid_constant__ StoutArgs<T> a)
+template <bool WS, typename T>
+__global__ void __launch_bounds__(kStoutBlock, sizeof(T) == 4 ? 5 : 1) k_stout_back_staples(const __grid_constant__ StoutArgs<T> a)
 {
+    pdl_enter();
     const int nu = blockIdx.y;
     const int i = blockIdx.x * kStoutBlock + threadIdx.x;
     if (i >= a.g.V) return;
-    M3T<T> acc;
-    ld(a.out, a.g, nu, i, acc);
+    const typename C2<T>::type *U = WS ? a.Uws : a.U;
+    M3T<T> acc = link_of<WS, T>(a.acc, a.g, nu, i);
 #pragma unroll 1
     for (int mu = 0; mu < 4; ++mu) {
         if (mu == nu) continue;
@@ -225,47 +241,38 @@ __global__ void __launch_bounds__(kStoutBlock) k_stout_back_staples(const __grid
         const int ym = down(a.g, i, mu), ymn = up(a.g, ym, nu);
         M3T<T> p, q, t;
         // forward side: U_nu(y+mu) shared by the first two terms
-        ld(a.U, a.g, nu, yp, p);   // U_nu(y+mu)
-        ld(a.U, a.g, mu, yn, q);   // U_mu(y+nu)
+        p = link_of<WS, T>(U, a.g, nu, yp);   // U_nu(y+mu)
+        q = link_of<WS, T>(U, a.g, mu, yn);   // U_mu(y+nu)
         t = mul<false, true>(p, q);
-        ld(a.Y, a.g, mu, i, q);    // Y_mu(y)
+        q = link_of<WS, T>(a.Y, a.g, mu, i);    // Y_mu(y)
         mul_acc<false, false>(acc, q, t);
-        ld(a.U, a.g, mu, i, q);    // U_mu(y)
+        q = link_of<WS, T>(U, a.g, mu, i);    // U_mu(y)
         t = mul<false, false>(q, p);
-        ld(a.Y, a.g, mu, yn, p);   // Y_mu(y+nu)
+        p = link_of<WS, T>(a.Y, a.g, mu, yn);   // Y_mu(y+nu)
         mul_acc<false, true>(acc, t, p);
-        ld(a.Y, a.g, nu, yp, p);   // Y_nu(y+mu)
+        p = link_of<WS, T>(a.Y, a.g, nu, yp);   // Y_nu(y+mu)
         t = mul<false, false>(q, p);
-        ld(a.U, a.g, mu, yn, q);   // U_mu(y+nu)
+        q = link_of<WS, T>(U, a.g, mu, yn);   // U_mu(y+nu)
         mul_acc<false, true>(acc, t, q);
         // backward side: U_mu(y-mu)^dag leads the last two terms
-        ld(a.U, a.g, nu, ym, p);   // U_nu(y-mu)
-        ld(a.U, a.g, mu, ymn, q);  // U_mu(y-mu+nu)
+        p = link_of<WS, T>(U, a.g, nu, ym);   // U_nu(y-mu)
+        q = link_of<WS, T>(U, a.g, mu, ymn);  // U_mu(y-mu+nu)
         t = mul<false, false>(p, q);
-        ld(a.Y, a.g, mu, ym, q);   // Y_mu(y-mu)
+        q = link_of<WS, T>(a.Y, a.g, mu, ym);   // Y_mu(y-mu)
         mul_acc<true, false>(acc, q, t);
-        ld(a.Y, a.g, mu, ymn, q);  // Y_mu(y-mu+nu)
+        q = link_of<WS, T>(a.Y, a.g, mu, ymn);  // Y_mu(y-mu+nu)
         t = mul<false, false>(p, q);
-        ld(a.Y, a.g, nu, ym, p);   // Y_nu(y-mu)
-        ld(a.U, a.g, mu, ymn, q);  // U_mu(y-mu+nu)
+        p = link_of<WS, T>(a.Y, a.g, nu, ym);   // Y_nu(y-mu)
+        q = link_of<WS, T>(U, a.g, mu, ymn);  // U_mu(y-mu+nu)
         mul_acc<false, false>(t, p, q);
-        ld(a.U, a.g, mu, ym, p);   // U_mu(y-mu)
+        p = link_of<WS, T>(U, a.g, mu, ym);   // U_mu(y-mu)
         mul_acc<true, false>(acc, p, t);
     }
-    st(a.out, a.g, nu, i, acc);
-}
-
-// F = TA(U G^dag) in place over G
-template <typename T>
-__global__ void __launch_bounds__(kStoutBlock) k_lie_force(const __grid_constant__ StoutArgs<T> a)
-{
-    const int mu = blockIdx.y;
-    const int i = blockIdx.x * kStoutBlock + threadIdx.x;
-    if (i >= a.g.V) return;
-    M3T<T> u, gr;
-    ld(a.U, a.g, mu, i, u);
-    ld(a.out, a.g, mu, i, gr);
-    st(a.out, a.g, mu, i, ta(mul<false, true>(u, gr)));
+    if (a.proj) acc = expand_anti_traceless(anti_mul<false, true>(link_of<WS, T>(U, a.g, nu, i), acc));
+    if (WS && !a.out_canon)
+        ws_st(a.out, a.g.V, nu, i, acc);
+    else
+        st(a.out, a.g, nu, i, acc);
 }
 
 // ------------------------------------------------------------------ by shared plaquettes
@@ -538,6 +545,10 @@ bool force_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
     return true;
 }
 
+// The per-link kernels, on canonical links.  The FP32 chain rule keeps its intermediate fields, and a
+// copy of the links for the staple terms (k_links_to_ws), as workspace fields when there is room:
+// 32^4 3.53 -> 2.97 ms, 16^4 266 -> 200 us.  Smearing and the first chain-rule kernel read the
+// canonical links (a smearing step from the workspace form took 690 us against 550).
 template <typename T>
 cudaError_t smear_t(const LinkGeo &g, int nstep, double rho, const void *links, void *levels, cudaStream_t st)
 {
@@ -551,8 +562,7 @@ cudaError_t smear_t(const LinkGeo &g, int nstep, double rho, const void *links, 
     for (int k = 0; k < nstep; ++k) {
         a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
         a.out = static_cast<C *>(levels) + (size_t)k * level;
-        k_stout_fwd<T><<<grid, kStoutBlock, 0, st>>>(a);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_pdl(k_stout_fwd<T>, grid, dim3(kStoutBlock), st, a);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -569,28 +579,45 @@ cudaError_t force_t(const LinkGeo &g, int nstep, double rho, const void *links, 
     a.rho = (T)rho;
     const size_t level = (size_t)4 * g.V * 9;
     C *ws = nullptr;
-    cudaError_t e = cudaMallocAsync((void **)&ws, 2 * level * sizeof(C), st);
-    if (e != cudaSuccess) return e;
-    C *Y = ws, *tmp = ws + level, *out = static_cast<C *>(out_v);
-    const dim3 grid((unsigned)((g.V + kStoutBlock - 1) / kStoutBlock), 4);
-    const C *g_in = static_cast<const C *>(grad);
-    for (int k = nstep - 1; k >= 0 && e == cudaSuccess; --k) {
-        // the last step (k = 0) lands in out; earlier ones alternate so that it does
-        C *dst = (k % 2 == 0) ? out : tmp;
-        a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
-        a.G = g_in;
-        a.out = dst;
-        a.Y = Y;
-        k_stout_back_link<T><<<grid, kStoutBlock, 0, st>>>(a);
-        k_stout_back_staples<T><<<grid, kStoutBlock, 0, st>>>(a);
-        e = cudaGetLastError();
-        g_in = dst;
+    keep_pool_mapped(st);
+    bool soa = sizeof(T) == 4;
+    cudaError_t e = cudaMallocAsync((void **)&ws, (soa ? 3 : 2) * level * sizeof(C), st);
+    if (e != cudaSuccess && soa) {
+        cudaGetLastError();
+        soa = false;
+        e = cudaMallocAsync((void **)&ws, 2 * level * sizeof(C), st);
     }
-    if (e == cudaSuccess && kind == 0) {
-        a.U = static_cast<const C *>(links);
-        a.out = out;
-        k_lie_force<T><<<grid, kStoutBlock, 0, st>>>(a);
-        e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    C *tmp = ws + level, *U = ws + 2 * level, *out = static_cast<C *>(out_v);
+    a.Y = ws;
+    const dim3 grid((unsigned)((g.V + kStoutBlock - 1) / kStoutBlock), 4), block(kStoutBlock);
+    a.G = static_cast<const C *>(grad);
+    a.g_canon = 1;
+    for (int k = nstep - 1; k >= 0 && e == cudaSuccess; --k) {
+        a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
+        a.proj = k == 0 && kind == 0;
+        bool done = false;
+        if constexpr (sizeof(T) == 4) {
+            if (soa) {
+                // each link's G, own terms and result share one place of tmp; the last result goes to out
+                e = links_to_ws<T>(a.U, U, g.V, st);
+                a.Uws = U;
+                a.acc = tmp;
+                a.out = k == 0 ? out : tmp;
+                a.out_canon = k == 0;
+                if (e == cudaSuccess) e = launch_pdl(k_stout_back_link<true, T>, grid, block, st, a);
+                if (e == cudaSuccess) e = launch_pdl(k_stout_back_staples<true, T>, grid, block, st, a);
+                a.g_canon = 0;
+                done = true;
+            }
+        }
+        if (!done) {
+            // the last step (k = 0) lands in out; earlier ones alternate so that it does
+            a.acc = a.out = (k % 2 == 0) ? out : tmp;
+            e = launch_pdl(k_stout_back_link<false, T>, grid, block, st, a);
+            if (e == cudaSuccess) e = launch_pdl(k_stout_back_staples<false, T>, grid, block, st, a);
+        }
+        a.G = a.out;
     }
     const cudaError_t f = cudaFreeAsync(ws, st);
     return e != cudaSuccess ? e : f;
