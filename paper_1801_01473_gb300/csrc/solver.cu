@@ -171,6 +171,63 @@ __device__ __forceinline__ int advance_sys(const WorkList &w, int s, int b)
     return s;
 }
 
+// r -= alpha q of one site in iteration `iters`, its |r|^2 added to pr
+template <typename R>
+__device__ __forceinline__ void update_r_site(const SysVecs &V, int h, R a, int iters, ProdSum<R> &pr)
+{
+    // in a ring, r^(k+1) goes to the next slot and r^k stays for the window flush
+    void *rin = V.nslot ? ring_slot<R>(V, iters) : V.r;
+    void *rout = V.nslot ? ring_slot<R>(V, iters + 1) : V.r;
+    cx<R> r[3], q[3];
+    Field<R>::load_rw(rin, V.Vh, h, r);
+    Field<R>::load_rw(V.q, V.Vh, h, q);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) r[c] = cx<R>{fma(-a, q[c].re, r[c].re), fma(-a, q[c].im, r[c].im)};
+    Field<R>::store(rout, V.Vh, h, r);
+    norm2_site(pr, r);
+}
+
+// p = zr r + bb p of one site, r the field r_in
+template <typename R>
+__device__ __forceinline__ void update_p_site(const void *r_in, void *p_io, int Vh, int h, R zr, R bb)
+{
+    cx<R> r[3], p[3];
+    Field<R>::load_rw(r_in, Vh, h, r);
+    Field<R>::load_rw(p_io, Vh, h, p);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) p[c] = cx<R>{fma(zr, r[c].re, bb * p[c].re), fma(zr, r[c].im, bb * p[c].im)};
+    Field<R>::store(p_io, Vh, h, p);
+}
+
+// x_i += cx_i p_i ; p_i = cr_i r + cp_i p_i of one site, for the shifts flagged in ux, up
+template <typename R, typename X>
+__device__ __forceinline__ void update_shifts_site(const SysVecs &V, int h, int ns, const X *cx_, const R *cr, const R *cp,
+                                                   const int *uxs, const int *ups)
+{
+    cx<R> r[3];
+    Field<R>::load_rw(V.r, V.Vh, h, r);
+    for (int i = 0; i < ns; ++i) {
+        const int ux = uxs[i], up = ups[i];
+        if (!ux && !up) continue;
+        cx<R> p[3];
+        Field<R>::load_rw(V.p[i], V.Vh, h, p);
+        if (ux) {
+            cx<X> x[3];
+            Field<X>::load_rw(V.x[i], V.Vh, h, x);
+            const X a = cx_[i];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) x[c] = cx<X>{fma(a, X(p[c].re), x[c].re), fma(a, X(p[c].im), x[c].im)};
+            Field<X>::store(V.x[i], V.Vh, h, x);
+        }
+        if (up) {
+            const R zr = cr[i], bb = cp[i];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) p[c] = cx<R>{fma(zr, r[c].re, bb * p[c].re), fma(zr, r[c].im, bb * p[c].im)};
+            Field<R>::store(V.p[i], V.Vh, h, p);
+        }
+    }
+}
+
 // r -= alpha q, partial |r|^2
 template <typename R>
 __global__ void __launch_bounds__(kVecBlock) k_update_r(const SysScal *__restrict__ sc, const SysVecs *__restrict__ sv,
@@ -186,19 +243,7 @@ __global__ void __launch_bounds__(kVecBlock) k_update_r(const SysScal *__restric
         const int lb = b - w.start[s];
         const int h = lb * kVecBlock + threadIdx.x;
         ProdSum<R> pr;
-        if (h < V.Vh) {
-            const R a = (R)S.alpha;
-            // in a ring, r^(k+1) goes to the next slot and r^k stays for the window flush
-            void *rin = V.nslot ? ring_slot<R>(V, S.iters) : V.r;
-            void *rout = V.nslot ? ring_slot<R>(V, S.iters + 1) : V.r;
-            cx<R> r[3], q[3];
-            Field<R>::load_rw(rin, V.Vh, h, r);
-            Field<R>::load_rw(V.q, V.Vh, h, q);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) r[c] = cx<R>{fma(-a, q[c].re, r[c].re), fma(-a, q[c].im, r[c].im)};
-            Field<R>::store(rout, V.Vh, h, r);
-            norm2_site(pr, r);
-        }
+        if (h < V.Vh) update_r_site<R>(V, h, (R)S.alpha, S.iters, pr);
         warp_partial(pr, h, V.Vh, V.part_v);
     }
 }
@@ -234,31 +279,7 @@ __global__ void __launch_bounds__(kVecBlock) k_update_shifts(const SysScal *__re
             loaded = s;
         }
         const int h = (b - w.start[s]) * kVecBlock + threadIdx.x;
-        if (h >= V.Vh) continue;
-        cx<R> r[3];
-        Field<R>::load_rw(V.r, V.Vh, h, r);
-        for (int i = 0; i < ns; ++i) {
-            const int ux = s_ux[i], up = s_up[i];
-            if (!ux && !up) continue;
-            cx<R> p[3];
-            Field<R>::load_rw(V.p[i], V.Vh, h, p);
-            if (ux) {
-                cx<X> x[3];
-                Field<X>::load_rw(V.x[i], V.Vh, h, x);
-                const X a = s_cx[i];
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    x[c] = cx<X>{fma(a, X(p[c].re), x[c].re), fma(a, X(p[c].im), x[c].im)};
-                Field<X>::store(V.x[i], V.Vh, h, x);
-            }
-            if (up) {
-                const R zr = s_cr[i], bb = s_cp[i];
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    p[c] = cx<R>{fma(zr, r[c].re, bb * p[c].re), fma(zr, r[c].im, bb * p[c].im)};
-                Field<R>::store(V.p[i], V.Vh, h, p);
-            }
-        }
+        if (h < V.Vh) update_shifts_site<R, X>(V, h, ns, s_cx, s_cr, s_cp, s_ux, s_up);
     }
 }
 
@@ -286,14 +307,8 @@ __global__ void __launch_bounds__(kVecBlock) k_update_pbase(const SysScal *__res
         if (!S.running || !S.upd_p[S.i0]) continue;  // uniform over the block
         const SysVecs &V = sv[s];
         const int h = (b - w.start[s]) * kVecBlock + threadIdx.x;
-        if (h >= V.Vh) continue;
-        const R zr = (R)S.cr[S.i0], bb = (R)S.cp[S.i0];
-        cx<R> r[3], p[3];
-        Field<R>::load_rw(ring_slot<R>(V, S.iters), V.Vh, h, r);
-        Field<R>::load_rw(V.p[S.i0], V.Vh, h, p);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) p[c] = cx<R>{fma(zr, r[c].re, bb * p[c].re), fma(zr, r[c].im, bb * p[c].im)};
-        Field<R>::store(V.p[S.i0], V.Vh, h, p);
+        if (h < V.Vh)
+            update_p_site<R>(ring_slot<R>(V, S.iters), V.p[S.i0], V.Vh, h, (R)S.cr[S.i0], (R)S.cp[S.i0]);
     }
 }
 
@@ -558,20 +573,9 @@ __global__ void k_p1_init_scal(SysScal *sc, const SysVecs *sv, int *done, double
     }
 }
 
-template <int kScalBlock>
-__global__ void __launch_bounds__(kScalBlock) k_alpha(SysScal *sc, const SysVecs *sv, const int *done)
+// Scalars of an iteration after alpha, by one warp
+__device__ __forceinline__ void alpha_scalars(SysScal &S, double alpha)
 {
-    pdl_enter();
-    SysScal &S = sc[blockIdx.x];
-    if (done[blockIdx.x]) {
-        if (threadIdx.x == 0) S.running = 0;
-        return;
-    }
-    const SysVecs &V = sv[blockIdx.x];
-    __shared__ double sh[33];
-    const double pq = block_sum_strided<kScalBlock>(V.part_d, V.nblk_d, sh);
-    if (threadIdx.x >= 32) return;  // the per-shift recurrences run in warp 0
-    const double alpha = S.rr / pq;
     for (int i = threadIdx.x; i < S.nshift; i += 32) {
         if (!S.active[i]) continue;
         const double z = S.zeta[i], zo = S.zeta_old[i];
@@ -587,16 +591,25 @@ __global__ void __launch_bounds__(kScalBlock) k_alpha(SysScal *sc, const SysVecs
 }
 
 template <int kScalBlock>
-__global__ void __launch_bounds__(kScalBlock) k_beta(SysScal *sc, const SysVecs *sv, int *done, int *need_rel,
-                                                      double *log, int log_rows)
+__global__ void __launch_bounds__(kScalBlock) k_alpha(SysScal *sc, const SysVecs *sv, const int *done)
 {
     pdl_enter();
     SysScal &S = sc[blockIdx.x];
-    if (!S.running) return;
+    if (done[blockIdx.x]) {
+        if (threadIdx.x == 0) S.running = 0;
+        return;
+    }
     const SysVecs &V = sv[blockIdx.x];
     __shared__ double sh[33];
-    const double rr_new = block_sum_strided<kScalBlock>(V.part_v, V.npart_v, sh);
-    if (threadIdx.x >= 32) return;  // the per-shift recurrences run in warp 0
+    const double pq = block_sum_strided<kScalBlock>(V.part_d, V.nblk_d, sh);
+    if (threadIdx.x < 32) alpha_scalars(S, S.rr / pq);
+}
+
+// Scalars of an iteration after |r|^2 (rr_new) of system `sys`, by one warp: beta, the shifts'
+// coefficients and stop tests, the history entry and the rotation to the next iteration
+__device__ __forceinline__ void beta_scalars(SysScal &S, const SysVecs &V, double rr_new, int sys, int *done,
+                                             int *need_rel, double *log, int log_rows)
+{
     const double beta = rr_new / S.rr;
     const int ns = S.nshift;
     int nact = 0;
@@ -641,12 +654,12 @@ __global__ void __launch_bounds__(kScalBlock) k_beta(SysScal *sc, const SysVecs 
             h.pp = S.upd_p[i] ? S.cp[i] : 1.0;
             V.hist[slot * kMaxShifts + i] = h;
         }
-        if (log != nullptr && blockIdx.x == 0 && S.iters < log_rows)
+        if (log != nullptr && sys == 0 && S.iters < log_rows)
             log[(size_t)S.iters * (2 + ns) + 2 + i] = S.upd_x[i] ? S.zeta[i] : 0.0;
     }
     __syncwarp();
     if (threadIdx.x == 0) {
-        if (log != nullptr && blockIdx.x == 0 && S.iters < log_rows) {
+        if (log != nullptr && sys == 0 && S.iters < log_rows) {
             log[(size_t)S.iters * (2 + ns)] = S.alpha;
             log[(size_t)S.iters * (2 + ns) + 1] = beta;
         }
@@ -656,9 +669,119 @@ __global__ void __launch_bounds__(kScalBlock) k_beta(SysScal *sc, const SysVecs 
         S.iters += 1;
         S.nactive = nact;
         if (V.hist != nullptr && slot >= V.nslot - 1) S.hist_overflow = 1;
-        if (!cont) done[blockIdx.x] = 1;
-        if (S.phase2 && (!cont || rr_new < S.delta2 * S.rr_last)) need_rel[blockIdx.x] = 1;
+        if (!cont) done[sys] = 1;
+        if (S.phase2 && (!cont || rr_new < S.delta2 * S.rr_last)) need_rel[sys] = 1;
     }
+}
+
+template <int kScalBlock>
+__global__ void __launch_bounds__(kScalBlock) k_beta(SysScal *sc, const SysVecs *sv, int *done, int *need_rel,
+                                                      double *log, int log_rows)
+{
+    pdl_enter();
+    SysScal &S = sc[blockIdx.x];
+    if (!S.running) return;
+    const SysVecs &V = sv[blockIdx.x];
+    __shared__ double sh[33];
+    const double rr_new = block_sum_strided<kScalBlock>(V.part_v, V.npart_v, sh);
+    if (threadIdx.x < 32) beta_scalars(S, V, rr_new, blockIdx.x, done, need_rel, log, log_rows);
+}
+
+// ------------------------------------------------------------------ fused iteration (small lattices)
+// On small lattices an iteration is six launches of a few microseconds each.  Here the vector kernels
+// take the scalar kernels' work along: every block sums the partials itself (the same fixed-order sum
+// in every block, as in k_alpha and k_beta) and keeps the coefficients it needs; one block per system
+// writes the scalars back.  Used while a launch is one wave of blocks with one item each and a sum
+// is at most kFusedPartials long; results are bitwise those of the separate kernels.  Mixed solve on
+// 8x6x8x6 2.95 -> 2.85 ms, 12^4 (324 partials) force evaluation 2.47 -> 2.39 ms; at 16^4 (1024 partials)
+// the sum in every block costs more than the launches (FP64 solve 12.8 against 14.7 ms).
+constexpr int kFusedPartials = 400;
+
+// k_alpha + k_update_r
+template <typename R>
+__global__ void __launch_bounds__(kVecBlock) k_alpha_update_r(SysScal *__restrict__ sc, const SysVecs *__restrict__ sv,
+                                                              const int *__restrict__ done, const WorkList w)
+{
+    pdl_enter();
+    __shared__ double sh[33];
+    const int b = blockIdx.x, s = advance_sys(w, 0, b);
+    SysScal &S = sc[s];
+    const SysVecs &V = sv[s];
+    const bool first = b == w.start[s];  // this block keeps the system's scalars
+    if (done[s]) {
+        if (first && threadIdx.x == 0) S.running = 0;
+        return;
+    }
+    const int iters = S.iters;
+    const double alpha = S.rr / block_sum_strided<kVecBlock>(V.part_d, V.nblk_d, sh);
+    if (first && threadIdx.x < 32) alpha_scalars(S, alpha);
+    const int h = (b - w.start[s]) * kVecBlock + threadIdx.x;
+    ProdSum<R> pr;
+    if (h < V.Vh) update_r_site<R>(V, h, (R)alpha, iters, pr);
+    warp_partial(pr, h, V.Vh, V.part_v);
+}
+
+// k_beta + k_update_pbase (BASE) or k_update_shifts.  ticket: one zeroed counter per system; the last
+// block to have read a system's scalars writes the new ones (and zeroes the counter).
+template <typename R, typename X, bool BASE>
+__global__ void __launch_bounds__(kVecBlock) k_beta_update(SysScal *__restrict__ sc, const SysVecs *__restrict__ sv,
+                                                           int *done, int *need_rel, double *log, int log_rows,
+                                                           const WorkList w, int *ticket)
+{
+    pdl_enter();
+    __shared__ double sh[33];
+    __shared__ X s_cx[kMaxShifts];
+    __shared__ R s_cr[kMaxShifts], s_cp[kMaxShifts];
+    __shared__ int s_ux[kMaxShifts], s_up[kMaxShifts], s_last;
+    const int b = blockIdx.x, s = advance_sys(w, 0, b);
+    SysScal &S = sc[s];
+    const SysVecs &V = sv[s];
+    if (!S.running) return;  // uniform over the block
+    const int ns = S.nshift, i0 = S.i0, iters = S.iters;
+    const double rr_new = block_sum_strided<kVecBlock>(V.part_v, V.npart_v, sh);
+    if (threadIdx.x < 32) {
+        // the coefficients that beta_scalars will write
+        const double beta = rr_new / S.rr;
+        int nact = 0;
+        for (int i = threadIdx.x; i < ns; i += 32) {
+            const int act = S.active[i];
+            const double zn = S.zeta_new[i], ratio = act ? zn / S.zeta[i] : 0.0;
+            const bool goes_on = act && !(zn * zn * rr_new <= S.tol2);
+            nact += goes_on;
+            s_ux[i] = act;
+            s_up[i] = goes_on;
+            s_cx[i] = X(S.cx[i]);
+            s_cr[i] = (R)zn;
+            s_cp[i] = (R)(beta * ratio * ratio);
+        }
+        nact = warp_sum_int(nact);
+        const bool cont = nact > 0 && iters + 1 < S.max_iter;
+        __syncwarp();
+        for (int i = threadIdx.x; i < ns; i += 32) {
+            if (!cont) {
+                s_up[i] = 0;
+            } else if (i == i0) {
+                s_up[i] = 1;
+                s_cr[i] = R(1);
+                s_cp[i] = (R)beta;
+            }
+        }
+        if (threadIdx.x == 0) {
+            __threadfence();
+            const int blocks = w.start[s + 1] - w.start[s];
+            s_last = atomicAdd(ticket + s, 1) == blocks - 1;
+            if (s_last) ticket[s] = 0;
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    if (s_last && threadIdx.x < 32) beta_scalars(S, V, rr_new, s, done, need_rel, log, log_rows);
+    const int h = (b - w.start[s]) * kVecBlock + threadIdx.x;
+    if (h >= V.Vh) return;
+    if (!BASE)
+        update_shifts_site<R, X>(V, h, ns, s_cx, s_cr, s_cp, s_ux, s_up);
+    else if (s_up[i0])
+        update_p_site<R>(ring_slot<R>(V, iters + 1), V.p[i0], V.Vh, h, s_cr[i0], s_cp[i0]);
 }
 
 // ------------------------------------------------------------------ phase-2 kernels
@@ -1107,15 +1230,17 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
     SysScal *d_s1 = static_cast<SysScal *>(mem.alloc(sizeof(SysScal) * nsys));
     SysVecs *d_v2 = static_cast<SysVecs *>(mem.alloc(sizeof(SysVecs) * npair));
     SysScal *d_s2 = static_cast<SysScal *>(mem.alloc(sizeof(SysScal) * npair));
-    // int flags: done1[nsys], need1[nsys], done2[npair], need2[npair], noupd[npair], finished[npair], relcnt[npair]
-    int *d_flags = static_cast<int *>(mem.alloc(sizeof(int) * (2 * nsys + 5 * npair)));
+    // int flags: done1[nsys], need1[nsys], done2[npair], need2[npair], noupd[npair], finished[npair], relcnt[npair],
+    // ticket1[nsys], ticket2[npair]
+    int *d_flags = static_cast<int *>(mem.alloc(sizeof(int) * (3 * nsys + 6 * npair)));
     double *d_true_rr = static_cast<double *>(mem.alloc(sizeof(double) * npair));
     double *d_log = prm->log_rows > 0 ? static_cast<double *>(mem.alloc(sizeof(double) * prm->log_rows * (2 + ns)))
                                       : nullptr;
     ConvPair *d_pairs = static_cast<ConvPair *>(mem.alloc(sizeof(ConvPair) * (2 * npair + nsys)));
     if (mem.err != cudaSuccess) return cuda_error(mem.err, "stg_mscg_solve: workspace allocation");
     int *done1 = d_flags, *need1 = d_flags + nsys, *done2 = d_flags + 2 * nsys, *need2 = done2 + npair,
-        *noupd = need2 + npair, *finished = noupd + npair, *relcnt = finished + npair;
+        *noupd = need2 + npair, *finished = noupd + npair, *relcnt = finished + npair, *ticket1 = relcnt + npair,
+        *ticket2 = ticket1 + nsys;
 
     // phase-2 inner vectors (allocated after the FP64 ones so phase 1 stays compact)
     for (int s = 0; s < nsys; ++s)
@@ -1134,7 +1259,7 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
     STG_CUDA_TRY(cudaMemcpyAsync(d_s1, s1.data(), sizeof(SysScal) * nsys, cudaMemcpyHostToDevice, ws));
     STG_CUDA_TRY(cudaMemcpyAsync(d_v2, v2.data(), sizeof(SysVecs) * npair, cudaMemcpyHostToDevice, ws));
     STG_CUDA_TRY(cudaMemcpyAsync(d_s2, s2.data(), sizeof(SysScal) * npair, cudaMemcpyHostToDevice, ws));
-    STG_CUDA_TRY(cudaMemsetAsync(d_flags, 0, sizeof(int) * (2 * nsys + 5 * npair), ws));
+    STG_CUDA_TRY(cudaMemsetAsync(d_flags, 0, sizeof(int) * (3 * nsys + 6 * npair), ws));
 
     // ---------------- dslash plans
     // phase 1: rhs of one instance share link loads (groups of up to kMaxRhs)
@@ -1265,6 +1390,12 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
     const dim3 g_s2 = wave((const void *)k_update_shifts<R, R>, wl2.total);
     cudaGetLastError();
 
+    // the fused iteration kernels, per phase: one wave of single-item blocks, short partial sums
+    bool fused1 = true, fused2 = true;
+    for (int q = 0; q < nsys; ++q) fused1 = fused1 && v1[q].npart_v <= kFusedPartials;
+    fused2 = fused1;
+    fused1 = fused1 && wl1.total <= (int)std::min(g_r1.x, hist_w > 0 ? g_pb.x : g_s1.x);
+    fused2 = fused2 && wl2.total <= (int)std::min(g_r2.x, g_s2.x);
     const bool scal_wide = getenv("STG_SCALAR_BLOCK") && atoi(getenv("STG_SCALAR_BLOCK")) == 1024;
     auto iterate = [&](int kind, const DPlan &pl, SysScal *dS, SysVecs *dV, int *dn, int *nr, int n, dim3 /*vg*/,
                        double *log, int log_rows) -> cudaError_t {
@@ -1275,6 +1406,20 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
             if ((e = launch_dslash(kind, a, 0, ws)) != cudaSuccess) return e;
         for (const DArgs &a : pl.eo)
             if ((e = launch_dslash(kind, a, 1, ws)) != cudaSuccess) return e;
+        if (ph1 ? fused1 : fused2) {
+            const dim3 items(wl.total);
+            int *tk = ph1 ? ticket1 : ticket2;
+            e = launch_pdl(k_alpha_update_r<R>, items, dim3(kVecBlock), ws, dS, (const SysVecs *)dV, (const int *)dn, wl);
+            if (e != cudaSuccess) return e;
+            if (ph1 && hist_w > 0)
+                return launch_pdl(k_beta_update<R, R, true>, items, dim3(kVecBlock), ws, dS, (const SysVecs *)dV, dn, nr,
+                                  log, log_rows, wl, tk);
+            if (ph1)
+                return launch_pdl(k_beta_update<R, H, false>, items, dim3(kVecBlock), ws, dS, (const SysVecs *)dV, dn, nr,
+                                  log, log_rows, wl, tk);
+            return launch_pdl(k_beta_update<R, R, false>, items, dim3(kVecBlock), ws, dS, (const SysVecs *)dV, dn, nr, log,
+                              log_rows, wl, tk);
+        }
         e = scal_wide ? launch_pdl(k_alpha<1024>, dim3(n), dim3(1024), ws, dS, (const SysVecs *)dV, (const int *)dn)
                       : launch_pdl(k_alpha<256>, dim3(n), dim3(256), ws, dS, (const SysVecs *)dV, (const int *)dn);
         if (e != cudaSuccess) return e;
