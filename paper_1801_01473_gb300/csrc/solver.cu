@@ -1456,12 +1456,13 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
         return cudaGetLastError();
     };
 
-    // Chunks of `kChunk` iterations are captured once per phase into a CUDA graph and replayed;
+    // Chunks of `kChunk` iterations are replayed from one CUDA graph per phase;
     // converged systems make every kernel of the chunk a no-op, so overshooting is cheap.
     struct GraphCache {
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
-        int state = 0;  // 0 not built, 1 graph, 2 direct launches
+        int state = 0;   // 0 not built, 1 graph, 2 direct launches
+        int direct = 0;  // chunks launched directly so far
         ~GraphCache()
         {
             if (exec) cudaGraphExecDestroy(exec);
@@ -1469,35 +1470,41 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
         }
     };
     constexpr int kChunk = 8;
+    // The first chunks of a phase are launched one kernel at a time (which also settles the autotuned
+    // block sizes outside capture); the graph is built on the host while the next one runs.  Capture
+    // and instantiation cost ~150 us, which a short solve does not earn back (8^4 force evaluation:
+    // 2055 us with a graph from the start, 1817 us so).
+    constexpr int kDirectChunks = 4;
     // Runs chunks until every system's done flag is set (or, with stop_on_need, until some
     // system asks for a reliable update).
     auto run_until_done = [&](GraphCache &gc, int kind, const DPlan &pl, SysScal *dS, SysVecs *dV, int *dn, int *nr, int n,
                               dim3 vg, double *log, int log_rows, bool stop_on_need, std::vector<int> &h_done,
                               std::vector<int> &h_need, int flush_every = 0) -> stg_status {
-        if (gc.state == 0) {
-            // the D launches of one iteration, outside capture, settle the autotuned block sizes;
-            // their outputs (t, q, partials) are recomputed by the first captured iteration
-            for (const DArgs &a : pl.oe) STG_CUDA_TRY(launch_dslash(kind, a, 0, ws));
-            for (const DArgs &a : pl.eo) STG_CUDA_TRY(launch_dslash(kind, a, 1, ws));
+        auto run_chunk = [&]() -> cudaError_t {
+            cudaError_t e = cudaSuccess;
+            for (int k = 0; k < kChunk && e == cudaSuccess; ++k)
+                e = iterate(kind, pl, dS, dV, dn, nr, n, vg, log, log_rows);
+            return e;
+        };
+        auto build_graph = [&]() {
             gc.state = 2;
             if (cudaStreamBeginCapture(ws, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-                cudaError_t e = cudaSuccess;
-                for (int k = 0; k < kChunk && e == cudaSuccess; ++k)
-                    e = iterate(kind, pl, dS, dV, dn, nr, n, vg, log, log_rows);
-                cudaError_t e2 = cudaStreamEndCapture(ws, &gc.graph);
+                const cudaError_t e = run_chunk();
+                const cudaError_t e2 = cudaStreamEndCapture(ws, &gc.graph);
                 if (e == cudaSuccess && e2 == cudaSuccess && cudaGraphInstantiate(&gc.exec, gc.graph, 0) == cudaSuccess)
                     gc.state = 1;
-                else
-                    cudaGetLastError();
-            } else {
-                cudaGetLastError();
             }
-        }
+            if (gc.state == 2) cudaGetLastError();
+        };
         const long long cap = (long long)prm->max_iter / kChunk + 4;
         for (long long c = 0; c <= cap; ++c) {
-            cudaError_t e = gc.state == 1 ? cudaGraphLaunch(gc.exec, ws) : cudaSuccess;
-            for (int k = 0; gc.state != 1 && k < kChunk && e == cudaSuccess; ++k)
-                e = iterate(kind, pl, dS, dV, dn, nr, n, vg, log, log_rows);
+            cudaError_t e = cudaSuccess;
+            if (gc.state == 1) {
+                e = cudaGraphLaunch(gc.exec, ws);
+            } else {
+                e = run_chunk();
+                if (e == cudaSuccess && gc.state == 0 && ++gc.direct > kDirectChunks) build_graph();
+            }
             if (e == cudaSuccess && flush_every > 0 && (c + 1) % flush_every == 0) e = flush(false);
             if (e == cudaSuccess) e = cudaMemcpyAsync(h_done.data(), dn, sizeof(int) * n, cudaMemcpyDeviceToHost, ws);
             if (e == cudaSuccess && stop_on_need)
