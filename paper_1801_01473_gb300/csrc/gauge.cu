@@ -68,13 +68,15 @@ __device__ __forceinline__ double retr_mul(const M3 &a, const M3 &b)
 // its three forms with one factor replaced by that link's outer staple: 11 products a side (each summed
 // before it is added to the larger total, which keeps the rounding of the loop-by-loop form), 66 per
 // link (84 when every loop is multiplied out).  Bound by latency at two blocks of 250 registers per SM;
-// three blocks of 168 ran 3 % slower at 32^4, four spill.  FP32, 32^4: 2.79 -> 1.75 ms with 32-bit site
-// arithmetic (neighbours by multiplication instead of 64-bit division), 16^4: 182 -> 118 us.
+// three blocks of 168 ran 3 % slower at 32^4, four spill.  FP32, 32^4: 2.79 -> 1.86 ms with 32-bit site
+// arithmetic (neighbours by multiplication instead of 64-bit division); 1.71 ms with the four directions
+// of 32 sites in one block, which share the links of their staples through L1 (one direction per
+// grid row re-read them from L2).  16^4: 182 -> 118 us.
 template <typename T>
 __global__ void __launch_bounds__(kGaugeBlock, 2) k_gauge_force(const __grid_constant__ GaugeArgs<T> a)
 {
-    const int mu = blockIdx.y;
-    const int x = blockIdx.x * kGaugeBlock + threadIdx.x;
+    const int mu = threadIdx.x >> 5;  // warp-uniform
+    const int x = blockIdx.x * 32 + (threadIdx.x & 31);
     if (x >= a.g.V) return;
     const LinkGeo &g = a.g;
     const typename C2<T>::type *__restrict__ Ub = a.U;
@@ -354,11 +356,11 @@ static cudaError_t gauge_force_t(const stg_lattice *lat, double beta, const void
     a.out = static_cast<typename C2<T>::type *>(out);
     a.kind = kind;
     // FP64: the shared staples wherever they fit (figures at the kernels).
-    // FP32: the loops one by one, which need no workspace traffic (32^4: 1.75 ms against 2.77 ms shared)
+    // FP32: the loops one by one, which need no workspace traffic (32^4: 1.71 ms against 2.77 ms shared)
     if constexpr (sizeof(T) == 8) {
         if (gauge_force_plaq<T>(lat, beta, links, out, kind, st, err)) return err;
     }
-    const dim3 grid((unsigned)((a.g.V + kGaugeBlock - 1) / kGaugeBlock), 4);
+    const unsigned grid = (unsigned)((a.g.V + 31) / 32);  // 32 sites, one warp per direction
     k_gauge_force<T><<<grid, kGaugeBlock, 0, st>>>(a);
     return cudaGetLastError();
 }

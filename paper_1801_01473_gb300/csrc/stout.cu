@@ -176,8 +176,8 @@ template <typename T>
 __global__ void __launch_bounds__(kStoutBlock) k_stout_fwd(const __grid_constant__ StoutArgs<T> a)
 {
     pdl_enter();
-    const int mu = blockIdx.y;
-    const int i = blockIdx.x * kStoutBlock + threadIdx.x;
+    const int mu = threadIdx.x >> 5;  // warp-uniform
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31);
     if (i >= a.g.V) return;
     const M3T<T> u = link_at<T>(a.U, a.g, mu, i);
     const H9<T> q = q_of(anti_mul<false, true>(staple_sum<T>(a.U, a.g, mu, i, a.rho), u), T(1)), q2 = square9(q);
@@ -191,8 +191,8 @@ template <bool WS, typename T>
 __global__ void __launch_bounds__(kStoutBlock) k_stout_back_link(const __grid_constant__ StoutArgs<T> a)
 {
     pdl_enter();
-    const int mu = blockIdx.y;
-    const int i = blockIdx.x * kStoutBlock + threadIdx.x;
+    const int mu = threadIdx.x >> 5;  // warp-uniform
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31);
     if (i >= a.g.V) return;
     const M3T<T> C = staple_sum<T>(a.U, a.g, mu, i, a.rho);
     const M3T<T> u = link_at<T>(a.U, a.g, mu, i);
@@ -229,8 +229,8 @@ template <bool WS, typename T>
 __global__ void __launch_bounds__(kStoutBlock, sizeof(T) == 4 ? 5 : 1) k_stout_back_staples(const __grid_constant__ StoutArgs<T> a)
 {
     pdl_enter();
-    const int nu = blockIdx.y;
-    const int i = blockIdx.x * kStoutBlock + threadIdx.x;
+    const int nu = threadIdx.x >> 5;  // warp-uniform
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31);
     if (i >= a.g.V) return;
     const typename C2<T>::type *U = WS ? a.Uws : a.U;
     M3T<T> acc = link_of<WS, T>(a.acc, a.g, nu, i);
@@ -447,7 +447,7 @@ E *take(char *&p, int V, int count)
 }
 
 // Whether the steps go by shared plaquettes.  FP32 stays with the per-link kernels, which are not
-// bound by their products (32^4 chain rule: 3.5 ms against 5.1 ms shared).  In FP64 every warp has a
+// bound by their products (32^4 chain rule: 2.8 ms against 5.1 ms shared).  In FP64 every warp has a
 // quarter SM's pipe to itself while a launch has no more warps than quarters; the one window where
 // the per-link kernels fit that once and the 6 planes of a site do not (3243 to 4864 sites on 152
 // SMs) is theirs: 8^4 smears in 191 us against 220 us, 6^4 (191 against 94) and 5120 sites (351
@@ -547,7 +547,8 @@ bool force_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
 
 // The per-link kernels, on canonical links.  The FP32 chain rule keeps its intermediate fields, and a
 // copy of the links for the staple terms (k_links_to_ws), as workspace fields when there is room:
-// 32^4 3.53 -> 2.97 ms, 16^4 266 -> 200 us.  Smearing and the first chain-rule kernel read the
+// 32^4 3.53 -> 2.97 ms, 16^4 266 -> 200 us (2.79 ms with the four directions of 32 sites in one block, which
+// share links through L1; smearing 1.10 -> 1.01 ms).  Smearing and the first chain-rule kernel read the
 // canonical links (a smearing step from the workspace form took 690 us against 550).
 template <typename T>
 cudaError_t smear_t(const LinkGeo &g, int nstep, double rho, const void *links, void *levels, cudaStream_t st)
@@ -558,7 +559,7 @@ cudaError_t smear_t(const LinkGeo &g, int nstep, double rho, const void *links, 
     a.g = g;
     a.rho = (T)rho;
     const size_t level = (size_t)4 * g.V * 9;  // complex numbers per level
-    const dim3 grid((unsigned)((g.V + kStoutBlock - 1) / kStoutBlock), 4);
+    const dim3 grid((unsigned)((g.V + 31) / 32));  // 32 sites, one warp per direction
     for (int k = 0; k < nstep; ++k) {
         a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
         a.out = static_cast<C *>(levels) + (size_t)k * level;
@@ -590,7 +591,7 @@ cudaError_t force_t(const LinkGeo &g, int nstep, double rho, const void *links, 
     if (e != cudaSuccess) return e;
     C *tmp = ws + level, *U = ws + 2 * level, *out = static_cast<C *>(out_v);
     a.Y = ws;
-    const dim3 grid((unsigned)((g.V + kStoutBlock - 1) / kStoutBlock), 4), block(kStoutBlock);
+    const dim3 grid((unsigned)((g.V + 31) / 32)), block(kStoutBlock);  // 32 sites, one warp per direction
     a.G = static_cast<const C *>(grad);
     a.g_canon = 1;
     for (int k = nstep - 1; k >= 0 && e == cudaSuccess; --k) {
