@@ -1,11 +1,11 @@
 // D_eo / D_oe instantiations for FP64 links (18-real and 12-real) on FP64 fields.
+#include <cstring>
+
 #include "dslash_fx.cuh"
 #include "stg_common.h"
 
 namespace stg {
 
-// Blocks of 64 threads (the choice of small lattices) keep 128 registers, larger ones 96 with a few
-// spills: 24^4 58.7 -> 57.0 us with the higher occupancy, 8^4 12.1 -> 13.3 us.
 template <int BS>
 static cudaError_t launch_fx_b(const DArgs &a, int mode, int maxv, cudaStream_t st)
 {
@@ -13,6 +13,14 @@ static cudaError_t launch_fx_b(const DArgs &a, int mode, int maxv, cudaStream_t 
     if (mode == 0) return launch_pdl(k_dslash_fx<0, BS>, grid, dim3(BS), st, a);
     if (mode == 1) return launch_pdl(k_dslash_fx<1, BS>, grid, dim3(BS), st, a);
     return launch_pdl(k_dslash_fx<2, BS>, grid, dim3(BS), st, a);
+}
+
+static cudaError_t launch_fx4(const DArgs &a, int mode, int maxv, cudaStream_t st)
+{
+    const dim3 grid((maxv + kFxSites - 1) / kFxSites, a.ngroups), block(4 * kFxSites);
+    if (mode == 0) return launch_pdl(k_dslash_fx4<0>, grid, block, st, a);
+    if (mode == 1) return launch_pdl(k_dslash_fx4<1>, grid, block, st, a);
+    return launch_pdl(k_dslash_fx4<2>, grid, block, st, a);
 }
 
 cudaError_t launch_dslash_f64r18(const DArgs &a, int mode, int bs, cudaStream_t st)
@@ -24,6 +32,22 @@ cudaError_t launch_dslash_f64r18(const DArgs &a, int mode, int bs, cudaStream_t 
     bool fx = maxr == 1;
     for (int k = 0; k < a.ngroups; ++k) fx = fx && a.grp[k].fx_links;
     if (!fx) return launch_dslash_t<LinkF64R18>(a, mode, bs, st);
+    // small lattices by four threads per site; a launch with both kinds becomes two
+    int nsplit = 0;
+    for (int k = 0; k < a.ngroups; ++k) nsplit += a.grp[k].g.Vh <= kFxSplitVh;
+    if (nsplit == a.ngroups) return launch_fx4(a, mode, maxv, st);
+    if (nsplit > 0) {
+        for (int split = 0; split < 2; ++split) {
+            DArgs b;
+            memset(&b, 0, sizeof(b));
+            b.out_par = a.out_par;
+            for (int k = 0; k < a.ngroups; ++k)
+                if ((a.grp[k].g.Vh <= kFxSplitVh) == (split == 1)) b.grp[b.ngroups++] = a.grp[k];
+            const cudaError_t e = launch_dslash_f64r18(b, mode, bs, st);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
     if (bs == 64) return launch_fx_b<64>(a, mode, maxv, st);
     if (bs == 256) return launch_fx_b<256>(a, mode, maxv, st);
     return launch_fx_b<128>(a, mode, maxv, st);

@@ -11,10 +11,11 @@
 // output, with B the power of two above the largest component of the 8 neighbours: ~2^-55 B rms from
 // the dropped term, the limbs' rounding and the final rounding together, against ~2^-53 B for the
 // FP64 chain of 48 rounded multiply-adds (whole operator on the exp(0.3 i H) links: 1.46e-16 against
-// 1.62e-16 of the 64-bit reference).  D at 32^4 312 -> 152 us (of 100 us at the copy bandwidth), 24^4
-// 108 -> 57 us, 16^4 46 -> 20 us, 8^4 15 -> 12 us.  What bounds it now: the integer pipes (864 products
-// and ~1400 other operations a site) and loads in flight at 16 to 20 warps per SM.  Links of 2 and above, infinities, NaNs, subnormal numbers
-// and vectors near the ends of the exponent range go through the FP64 loop, thread by thread.
+// 1.62e-16 of the 64-bit reference).  Links of 2 and above, infinities, NaNs, subnormal numbers and
+// vectors near the ends of the exponent range go through the FP64 loop, thread by thread.
+// D at 32^4 312 -> 152 us (of 100 us at the copy bandwidth), 24^4 108 -> 57 us, 16^4 46 -> 15 us, 8^4 15 ->
+// 10 us.  What bounds it now: the integer pipes (864 products and ~1400 other operations a site)
+// and, with one thread per site, loads in flight at 16 to 20 warps per SM.
 #pragma once
 
 #include "dslash.cuh"
@@ -57,11 +58,11 @@ __device__ __forceinline__ void fx_mac(long long &hh, long long &mid, const FxNu
 
 __device__ __forceinline__ FxNum fx_neg(const FxNum &a) { return FxNum{-a.l1, -a.l0}; }
 
-// x 2^-d rounded, 1 <= d
+// x 2^-d rounded, 0 <= d
 __device__ __forceinline__ long long fx_shift(long long x, int d)
 {
     d = min(d, 62);
-    return (x + (1ll << (d - 1))) >> d;
+    return (x + ((1ll << d) >> 1)) >> d;
 }
 
 // Fixed-point links: per (mu, parity) block 9 chunks over Vh of (re.l1, re.l0, im.l1, im.l0)
@@ -111,6 +112,8 @@ __device__ __forceinline__ void dp_hop(cx<double> acc[3], const cx<double> U[3][
     }
 }
 
+// One thread per output site.  Blocks of 64 threads keep 128 registers, larger ones 96 with a few
+// spills: 24^4 58.7 -> 57.0 us with the higher occupancy.
 template <int MODE, int BS>
 __global__ void __launch_bounds__(BS, (BS == 64 ? 512 : 640) / BS) k_dslash_fx(const __grid_constant__ DArgs a)
 {
@@ -217,6 +220,152 @@ __global__ void __launch_bounds__(BS, (BS == 64 ? 512 : 640) / BS) k_dslash_fx(c
     const bool act[1] = {true};
     __shared__ double sh[32];
     dslash_epilogue<double, 1, MODE, BS>(G, bx, act, live, h, acc, sh);
+}
+
+// Small lattices (up to kFxSplitVh sites per parity): a block covers 64 output sites with four threads
+// each.  Thread (mu, site) does the two hops of one direction, so that every load of a site is in
+// flight at once and few sites fill the chip; the four partial sums meet in shared memory in the unit
+// of the largest neighbour.  One right-hand side, against one thread per site: 12^4 13.6 -> 9.2 us, 16^4
+// 22.5 -> 14.8 us, 20^4 34.7 -> 30.4 us, but 24^4 56.4 -> 57.3 us (normal operator 122 -> 128 us) and 32^4
+// 151 -> 168 us, where the exchange costs more than the parallelism gives.  The choice depends on
+// the lattice alone, so that results do not depend on what else a launch carries.
+constexpr int kFxSites = 64;
+constexpr int kFxSplitVh = 90000;
+
+template <int MODE>
+__global__ void __launch_bounds__(4 * kFxSites, 3) k_dslash_fx4(const __grid_constant__ DArgs a)
+{
+    pdl_enter();
+    const BlockPos pos = block_pos();
+    const DGroup &G = a.grp[pos.group];
+    const int Vh = G.g.Vh;
+    if (pos.bx * kFxSites >= G.g.h_end - G.g.h_begin) return;             // block-uniform
+    if (G.nrhs < 1 || (G.skip[0] != nullptr && *G.skip[0] != 0)) return;  // block-uniform
+
+    __shared__ long long s_part[3][12][kFxSites];  // sums of mu = 1..3 (as doubles on the FP64 path)
+    __shared__ int s_e[4][kFxSites];               // exponent of each sum's unit; -1: no fixed-point form
+    __shared__ double sh[32];
+    const int mu = threadIdx.x / kFxSites, sl = threadIdx.x % kFxSites;  // mu is warp-uniform
+    const int h = G.g.h_begin + pos.bx * kFxSites + sl;
+    const bool live = h < G.g.h_end;
+    const int op = a.out_par;
+    Hop hp;
+    if (live) hp = hop_of(G.g, site_of(G.g, op, h), mu);
+
+    long long hh[3][2], mid[3][2];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) hh[r][0] = hh[r][1] = mid[r][0] = mid[r][1] = 0;
+    int E = 0;  // 0 while both neighbours are zero
+    if (live) {
+        cx<double> v[2][3];
+        Field<double>::load(G.in[0], Vh, hp.hf, v[0]);
+        Field<double>::load(G.in[0], Vh, hp.hb, v[1]);
+        bool ok = *G.fx_bad == 0;
+        int e = 0, tiny = 0;
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                e = max(e, max(__double2hiint(v[k][c].re) & 0x7fffffff, __double2hiint(v[k][c].im) & 0x7fffffff));
+        E = e >> 20;
+        if (E == 0) {  // zeros, or subnormal numbers, which have no fixed-point form here
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) tiny |= v[k][c].re != 0.0 || v[k][c].im != 0.0;
+        }
+        ok = ok && !tiny && (E == 0 || (E >= 100 && E < 2046));
+        if (E != 0) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const bool back = k == 1;
+                const bool flip = back ? hp.sb > 0.f : hp.sf < 0.f;  // the backward hop enters with -u
+                FxNum u[3][3][2];
+                LinkFX::load(link_block<LinkFX>(G.fx_links, Vh, mu, back ? 1 - op : op), Vh, back ? hp.hb : h, u);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const FxNum xr = fx_limbs(flip ? -v[k][c].re : v[k][c].re, E);
+                    const FxNum xi = fx_limbs(flip ? -v[k][c].im : v[k][c].im, E);
+                    const FxNum n = fx_neg(back ? xr : xi);
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) {
+                        const FxNum &re = back ? u[c][r][0] : u[r][c][0], &im = back ? u[c][r][1] : u[r][c][1];
+                        fx_mac(hh[r][0], mid[r][0], re, xr);
+                        fx_mac(hh[r][0], mid[r][0], im, back ? xi : n);
+                        fx_mac(hh[r][1], mid[r][1], re, xi);
+                        fx_mac(hh[r][1], mid[r][1], im, back ? n : xr);
+                    }
+                }
+            }
+        }
+        s_e[mu][sl] = ok ? E : -1;
+        if (!ok) E = -1;
+        if (mu > 0) {
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    s_part[mu - 1][4 * r + 2 * q][sl] = hh[r][q];
+                    s_part[mu - 1][4 * r + 2 * q + 1][sl] = mid[r][q];
+                }
+        }
+    }
+    cx<double> acc[1][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) acc[0][c] = cx<double>{0.0, 0.0};
+    const bool any_bad = __syncthreads_or(E < 0);
+    const bool bad = any_bad && live && min(min(s_e[0][sl], s_e[1][sl]), min(s_e[2][sl], s_e[3][sl])) < 0;
+    if (any_bad) {
+        if (bad) {  // this direction in FP64
+            cx<double> U[3][3], v[3];
+            LinkF64R18::load(link_block<LinkF64R18>(G.links, Vh, mu, op), Vh, h, U);
+            Field<double>::load(G.in[0], Vh, hp.hf, v);
+            dp_hop<false>(acc[0], U, v, hp.sf);
+            LinkF64R18::load(link_block<LinkF64R18>(G.links, Vh, mu, 1 - op), Vh, hp.hb, U);
+            Field<double>::load(G.in[0], Vh, hp.hb, v);
+            dp_hop<true>(acc[0], U, v, -hp.sb);
+            if (mu > 0)
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    s_part[mu - 1][2 * r][sl] = __double_as_longlong(acc[0][r].re);
+                    s_part[mu - 1][2 * r + 1][sl] = __double_as_longlong(acc[0][r].im);
+                }
+        }
+        __syncthreads();
+    }
+    if (live && mu == 0) {
+        if (bad) {
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    acc[0][r].re += __longlong_as_double(s_part[m][2 * r][sl]);
+                    acc[0][r].im += __longlong_as_double(s_part[m][2 * r + 1][sl]);
+                }
+        } else {
+            const int em[4] = {E, s_e[1][sl], s_e[2][sl], s_e[3][sl]};
+            const int top = max(max(em[0], em[1]), max(em[2], em[3]));
+            const double unit = __hiloint2double(max(top - 54, 0) << 20, 0);  // of hh: 2^56 2^(top - 1078) 2^-55
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    long long sum = fx_shift(hh[r][q], top - em[0]), low = fx_shift(mid[r][q], top - em[0]);
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) {
+                        sum += fx_shift(s_part[m][4 * r + 2 * q][sl], top - em[m + 1]);
+                        low += fx_shift(s_part[m][4 * r + 2 * q + 1][sl], top - em[m + 1]);
+                    }
+                    const double w = unit * (double)(sum + ((low + (1 << 27)) >> 28));
+                    if (q == 0)
+                        acc[0][r].re = w;
+                    else
+                        acc[0][r].im = w;
+                }
+        }
+    }
+    const bool act[1] = {true};
+    dslash_epilogue<double, 1, MODE, kFxSites>(G, pos.bx, act, live && mu == 0, h, acc, sh);
 }
 
 }  // namespace stg

@@ -1,4 +1,4 @@
-"""The FP64 operator's fixed-point kernel (k_dslash_fx) against the FP64 oracle, and the sites that it
+"""The FP64 operator's fixed-point kernels (k_dslash_fx, k_dslash_fx4) against the FP64 oracle, and the sites that it
 hands to its FP64 loop: components of very different size at neighbouring sites and within a site,
 zero neighbourhoods, the ends of the exponent range, infinities and NaNs, links of 2 and above; one
 and several right-hand sides, the smallest lattice that takes it (2048 sites), one below it, extents
@@ -16,6 +16,8 @@ import oracle
 import synthetic as S
 
 pytestmark = pytest.mark.gpu
+
+LARGE = (24, 24, 24, 14)  # 96768 sites per parity: one thread per site (four below 90000)
 
 
 def _gpu(a):
@@ -45,21 +47,21 @@ def _check(dims, u, psi, factor=1.0):
         assert (np.abs(got - want) <= bound).all()
 
 
-@pytest.mark.parametrize("dims", [(8, 8, 8, 4), (2, 2, 32, 16), (6, 10, 4, 14), (4, 4, 4, 4)])
+@pytest.mark.parametrize("dims", [(8, 8, 8, 4), (2, 2, 32, 16), (6, 10, 4, 14), (4, 4, 4, 4), LARGE])
 def test_matches_oracle(dims):
     _check(dims, S.gauge_links(dims, "haar", 171), S.gaussian_field(dims, 172))
 
 
+@pytest.mark.parametrize("dims", [(8, 6, 6, 8), LARGE])
 @pytest.mark.parametrize("scale", [1e-290, 1e-30, 1e30, 1e290])
-def test_scales(scale):
+def test_scales(scale, dims):
     """Vectors far from one, and (1e-290) below the exponents that the fixed-point form takes."""
-    dims = (8, 6, 6, 8)
     _check(dims, S.gauge_links(dims, "haar", 173), scale * S.gaussian_field(dims, 174))
 
 
-def test_uneven_sizes_and_zeros():
+@pytest.mark.parametrize("dims", [(8, 6, 8, 6), LARGE])
+def test_uneven_sizes_and_zeros(dims):
     """Sizes spread over 60 decades site by site and colour by colour, with zeros and zero sites."""
-    dims = (8, 6, 8, 6)
     rng = np.random.default_rng(175)
     psi = S.gaussian_field(dims, 176)
     psi = psi * 10.0 ** rng.uniform(-60, 0, psi.shape[:1])[:, None] * 10.0 ** rng.uniform(-8, 0, psi.shape)
@@ -71,17 +73,17 @@ def test_uneven_sizes_and_zeros():
     _check(dims, S.gauge_links(dims, "haar", 177), point)
 
 
-def test_links_outside_the_fixed_point_range():
-    dims = (4, 8, 8, 8)
+@pytest.mark.parametrize("dims", [(4, 8, 8, 8), LARGE])
+def test_links_outside_the_fixed_point_range(dims):
     u = S.gauge_links(dims, "haar", 178).copy()
     u[2, 17] *= 1e3
     _check(dims, u, S.gaussian_field(dims, 179), factor=1e3)
 
 
-def test_non_finite_inputs_stay_local():
+@pytest.mark.parametrize("dims", [(8, 6, 8, 8), LARGE])
+def test_non_finite_inputs_stay_local(dims):
     """Sites with a NaN or infinite neighbour are not finite, as in the FP64 loop; the others are the same."""
     import paper_1801_01473_gb300 as p
-    dims = (8, 6, 8, 8)
     u = S.gauge_links(dims, "haar", 180)
     psi = S.gaussian_field(dims, 181)
     g = p.Gauge(p.Lattice(dims), _gpu(u), "f64", 18)
@@ -113,3 +115,16 @@ def test_several_right_hand_sides_and_update(nrhs):
         assert torch.equal(out[j], p.dslash_eo_(g, torch.empty_like(inp[j]), inp[j].contiguous()))
     want = oracle.dslash_eo(dims, u, psi[nrhs - 1])
     assert np.abs(p.unpack(lat, out[nrhs - 1]).cpu().numpy() - want).max() <= 1e-13
+
+
+def test_lattices_of_both_kinds_in_one_batch():
+    """A batched FP64 solve over a lattice of each kernel gives bitwise the single solves."""
+    import paper_1801_01473_gb300 as p
+    insts = []
+    for k, dims in enumerate(((8, 8, 8, 8), LARGE)):
+        g = p.Gauge(p.Lattice(dims), _gpu(S.gauge_links(dims, "expih", 185 + k)), "f64", 18)
+        insts.append((g, None, [_gpu(S.gaussian_field(dims, 187 + k))]))
+    both = p.mscg_batched(insts, [0.01, 0.5], 0.3, tol=1e-10)
+    for (g, _, (b,)), (x, _) in zip(insts, both):
+        one, _ = p.mscg(g, b, [0.01, 0.5], 0.3, tol=1e-10)
+        assert torch.equal(x[0], one)
