@@ -22,14 +22,14 @@
 namespace stg {
 
 constexpr int kMaxRhs = 8;
-constexpr int kMaxGroups = 16;  // groups per launch (gridDim.y): a DArgs of 16 groups is ~8.5 KB of kernel parameters
+constexpr int kMaxGroups = 16;  // groups per launch (gridDim.x): a DArgs of 16 groups is ~8.5 KB of kernel parameters
 constexpr int kDslashBlock = 128;   // default block; the autotuner may pick 64, 128 or 256
 constexpr int kPartialSites = 64;   // one FP64 partial per 64 output sites, whatever the block size
 
 // Number of FP64 partial sums an epilogue launch writes for a lattice of Vh sites per parity.
 __host__ __device__ inline int dslash_partials(int Vh) { return (Vh + kPartialSites - 1) / kPartialSites; }
 
-// A set of right-hand sides on one lattice and gauge; a launch has gridDim.y of them.
+// A set of right-hand sides on one lattice and gauge; a launch has gridDim.x of them.
 struct DGroup {
     Geom g;
     const void *links;
@@ -65,20 +65,13 @@ __device__ __forceinline__ void lazy_mac(float &hi, float &lo, const dsf &a, con
     lo = __fadd_rn(lo, __fadd_rn(err, e));
 }
 
-// Block index bx along the output sites and group of this thread block.  The groups of a launch are
-// dealt out in turn, so that blocks of all groups on the same sites run together: groups on one
-// gauge then read each link from DRAM once and from L2 for the others.
-// 12 double-single D on 24^3x32 493 -> 405 us (one group after the other re-read 255 MB of links for each).
-struct BlockPos {
-    int bx, group;
-};
-__device__ __forceinline__ BlockPos block_pos()
-{
-    const unsigned ng = gridDim.y;
-    if (ng == 1) return BlockPos{(int)blockIdx.x, 0};
-    const unsigned id = blockIdx.y * gridDim.x + blockIdx.x;
-    return BlockPos{(int)(id / ng), (int)(id % ng)};
-}
+// Block of a D launch along the output sites: x = group, y = block.  x runs fastest, so the groups are
+// dealt out in turn and blocks of all groups on the same sites run together: groups on one gauge
+// then read each link from DRAM once and from L2 for the others.  12 double-single D on 24^3x32 493 ->
+// 405 us (one group after the other re-read 255 MB of links for each).  More blocks than y can
+// count go in several launches (launch_sites).  (Any arithmetic here, a division or an offset, gave
+// the one-group FP32 kernel a schedule of 40 registers instead of 48, 2 % slower.)
+__device__ __forceinline__ int block_along_sites() { return (int)blockIdx.y; }
 
 template <typename R>
 __device__ __forceinline__ void neg3(cx<R> v[3])
@@ -89,7 +82,7 @@ __device__ __forceinline__ void neg3(cx<R> v[3])
 
 // Epilogue of the D kernels: scale (MODE 0) or fuse the shifted normal operator and its FP64
 // partial sums (MODE 1, 2), store, and write one partial per 64 output sites.  `sh` holds >= 32
-// doubles of shared memory; `act` is uniform over the block.
+// doubles of shared memory; `act` is uniform over the block; bx is the block's index along the sites.
 template <typename R, int NRHS, int MODE, int BS>
 __device__ __forceinline__ void dslash_epilogue(const DGroup &G, int bx, const bool act[NRHS], bool live, int h,
                                                 const cx<R> acc[NRHS][3], double *sh,
@@ -253,9 +246,8 @@ __global__ void __launch_bounds__(BS) k_dslash(const __grid_constant__ DArgs a)
 {
     using R = typename LinkT::R;
     pdl_enter();
-    const BlockPos pos = block_pos();
-    const int bx = pos.bx;
-    const DGroup &G = a.grp[pos.group];
+    const int bx = block_along_sites();
+    const DGroup &G = a.grp[blockIdx.x];
     const int Vh = G.g.Vh;
     const int nout = G.g.h_end - G.g.h_begin;
     if (bx * BS >= nout) return;  // block-uniform
@@ -420,9 +412,8 @@ __global__ void __launch_bounds__(512) k_dslash_sh(const __grid_constant__ DArgs
     int *sh_nb = reinterpret_cast<int *>(sh_links + 8 * 18 * kShSites);
     __shared__ double sh_part[16];
     pdl_enter();
-    const BlockPos pos = block_pos();
-    const int bx = pos.bx;
-    const DGroup &G = a.grp[pos.group];
+    const int bx = block_along_sites();
+    const DGroup &G = a.grp[blockIdx.x];
     const int Vh = G.g.Vh;
     const int nout = G.g.h_end - G.g.h_begin;
     if (bx * kShSites >= nout) return;  // block-uniform
@@ -563,15 +554,38 @@ cudaError_t launch_pdl_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args &&>(args)...);
 }
 
+// Launches a D kernel on blocks of `sites` output sites of every group (maxv: the largest group's).
+// Beyond what grid y counts, further launches start at a later site, with the partials moved along.
+constexpr int kMaxBlocksY = 65535;
+inline cudaError_t launch_sites(void (*kernel)(const DArgs), int maxv, int sites, int threads, size_t smem,
+                                cudaStream_t st, const DArgs &a)
+{
+    const int nb = (maxv + sites - 1) / sites;
+    if (nb <= kMaxBlocksY) return launch_pdl_smem(kernel, dim3(a.ngroups, nb), dim3(threads), smem, st, a);
+    DArgs b = a;
+    const int step = kMaxBlocksY / 64 * 64 * sites;  // whole 64-site partials
+    for (long long h0 = 0; h0 < maxv; h0 += step) {
+        const int n = (int)((maxv - h0 < step ? maxv - h0 : step) + sites - 1) / sites;
+        const cudaError_t e = launch_pdl_smem(kernel, dim3(a.ngroups, n), dim3(threads), smem, st, b);
+        if (e != cudaSuccess) return e;
+        for (int k = 0; k < b.ngroups; ++k) {
+            DGroup &G = b.grp[k];
+            G.g.h_begin = G.g.h_end - G.g.h_begin > step ? G.g.h_begin + step : G.g.h_end;
+            for (int j = 0; j < G.nrhs; ++j)
+                if (G.partial[j]) G.partial[j] += step / kPartialSites;
+        }
+    }
+    return cudaSuccess;
+}
+
 // Host-side launcher: picks the NRHS instantiation (>= the largest group's nrhs) and the
 // block size `bs` (64, 128 or 256; anything else falls back to 128).
 template <typename LinkT, int NRHS, int BS>
 cudaError_t launch_dslash_nb(const DArgs &a, int mode, int maxv, cudaStream_t st)
 {
-    dim3 grid((maxv + BS - 1) / BS, a.ngroups);
-    if (mode == 0) return launch_pdl(k_dslash<LinkT, NRHS, 0, BS>, grid, dim3(BS), st, a);
-    if (mode == 1) return launch_pdl(k_dslash<LinkT, NRHS, 1, BS>, grid, dim3(BS), st, a);
-    return launch_pdl(k_dslash<LinkT, NRHS, 2, BS>, grid, dim3(BS), st, a);
+    if (mode == 0) return launch_sites(k_dslash<LinkT, NRHS, 0, BS>, maxv, BS, BS, 0, st, a);
+    if (mode == 1) return launch_sites(k_dslash<LinkT, NRHS, 1, BS>, maxv, BS, BS, 0, st, a);
+    return launch_sites(k_dslash<LinkT, NRHS, 2, BS>, maxv, BS, BS, 0, st, a);
 }
 
 template <typename LinkT, int NRHS>
@@ -611,10 +625,9 @@ cudaError_t launch_dslash_t(const DArgs &a, int mode, int bs, cudaStream_t st)
     if (bs == kSharedLinks) {
         if constexpr (sizeof(typename LinkT::R) == sizeof(float) && !LinkTraits<LinkT>::kU1) {
             if (maxr > kMaxRhs) return cudaErrorInvalidValue;
-            const dim3 grid((maxv + kShSites - 1) / kShSites, a.ngroups), block(64 * maxr);
-            if (mode == 0) return launch_pdl_smem(k_dslash_sh<LinkT, 0>, grid, block, kShBytes, st, a);
-            if (mode == 1) return launch_pdl_smem(k_dslash_sh<LinkT, 1>, grid, block, kShBytes, st, a);
-            return launch_pdl_smem(k_dslash_sh<LinkT, 2>, grid, block, kShBytes, st, a);
+            if (mode == 0) return launch_sites(k_dslash_sh<LinkT, 0>, maxv, kShSites, 64 * maxr, kShBytes, st, a);
+            if (mode == 1) return launch_sites(k_dslash_sh<LinkT, 1>, maxv, kShSites, 64 * maxr, kShBytes, st, a);
+            return launch_sites(k_dslash_sh<LinkT, 2>, maxv, kShSites, 64 * maxr, kShBytes, st, a);
         } else {
             return cudaErrorInvalidValue;
         }
@@ -622,10 +635,9 @@ cudaError_t launch_dslash_t(const DArgs &a, int mode, int bs, cudaStream_t st)
     if (bs == kLoadsAhead) {
         if constexpr (std::is_same<LinkT, LinkF32R12>::value) {
             if (dslash_nrhs_template(maxr) != 4) return cudaErrorInvalidValue;
-            const dim3 grid((maxv + 63) / 64, a.ngroups);
-            if (mode == 0) return launch_pdl(k_dslash<LinkT, 4, 0, 64, true>, grid, dim3(64), st, a);
-            if (mode == 1) return launch_pdl(k_dslash<LinkT, 4, 1, 64, true>, grid, dim3(64), st, a);
-            return launch_pdl(k_dslash<LinkT, 4, 2, 64, true>, grid, dim3(64), st, a);
+            if (mode == 0) return launch_sites(k_dslash<LinkT, 4, 0, 64, true>, maxv, 64, 64, 0, st, a);
+            if (mode == 1) return launch_sites(k_dslash<LinkT, 4, 1, 64, true>, maxv, 64, 64, 0, st, a);
+            return launch_sites(k_dslash<LinkT, 4, 2, 64, true>, maxv, 64, 64, 0, st, a);
         } else {
             return cudaErrorInvalidValue;
         }

@@ -9,18 +9,16 @@ namespace stg {
 template <int BS>
 static cudaError_t launch_fx_b(const DArgs &a, int mode, int maxv, cudaStream_t st)
 {
-    const dim3 grid((maxv + BS - 1) / BS, a.ngroups);
-    if (mode == 0) return launch_pdl(k_dslash_fx<0, BS>, grid, dim3(BS), st, a);
-    if (mode == 1) return launch_pdl(k_dslash_fx<1, BS>, grid, dim3(BS), st, a);
-    return launch_pdl(k_dslash_fx<2, BS>, grid, dim3(BS), st, a);
+    if (mode == 0) return launch_sites(k_dslash_fx<0, BS>, maxv, BS, BS, 0, st, a);
+    if (mode == 1) return launch_sites(k_dslash_fx<1, BS>, maxv, BS, BS, 0, st, a);
+    return launch_sites(k_dslash_fx<2, BS>, maxv, BS, BS, 0, st, a);
 }
 
 static cudaError_t launch_fx4(const DArgs &a, int mode, int maxv, cudaStream_t st)
 {
-    const dim3 grid((maxv + kFxSites - 1) / kFxSites, a.ngroups), block(4 * kFxSites);
-    if (mode == 0) return launch_pdl(k_dslash_fx4<0>, grid, block, st, a);
-    if (mode == 1) return launch_pdl(k_dslash_fx4<1>, grid, block, st, a);
-    return launch_pdl(k_dslash_fx4<2>, grid, block, st, a);
+    if (mode == 0) return launch_sites(k_dslash_fx4<0>, maxv, kFxSites, 4 * kFxSites, 0, st, a);
+    if (mode == 1) return launch_sites(k_dslash_fx4<1>, maxv, kFxSites, 4 * kFxSites, 0, st, a);
+    return launch_sites(k_dslash_fx4<2>, maxv, kFxSites, 4 * kFxSites, 0, st, a);
 }
 
 cudaError_t launch_dslash_f64r18(const DArgs &a, int mode, int bs, cudaStream_t st)

@@ -118,9 +118,8 @@ template <int MODE, int BS>
 __global__ void __launch_bounds__(BS, (BS == 64 ? 512 : 640) / BS) k_dslash_fx(const __grid_constant__ DArgs a)
 {
     pdl_enter();
-    const BlockPos pos = block_pos();
-    const int bx = pos.bx;
-    const DGroup &G = a.grp[pos.group];
+    const int bx = block_along_sites();
+    const DGroup &G = a.grp[blockIdx.x];
     const int Vh = G.g.Vh;
     if (bx * BS >= G.g.h_end - G.g.h_begin) return;  // block-uniform
     if (G.nrhs < 1 || (G.skip[0] != nullptr && *G.skip[0] != 0)) return;  // block-uniform
@@ -236,17 +235,17 @@ template <int MODE>
 __global__ void __launch_bounds__(4 * kFxSites, 3) k_dslash_fx4(const __grid_constant__ DArgs a)
 {
     pdl_enter();
-    const BlockPos pos = block_pos();
-    const DGroup &G = a.grp[pos.group];
+    const int bx = block_along_sites();
+    const DGroup &G = a.grp[blockIdx.x];
     const int Vh = G.g.Vh;
-    if (pos.bx * kFxSites >= G.g.h_end - G.g.h_begin) return;             // block-uniform
+    if (bx * kFxSites >= G.g.h_end - G.g.h_begin) return;             // block-uniform
     if (G.nrhs < 1 || (G.skip[0] != nullptr && *G.skip[0] != 0)) return;  // block-uniform
 
     __shared__ long long s_part[3][12][kFxSites];  // sums of mu = 1..3 (as doubles on the FP64 path)
     __shared__ int s_e[4][kFxSites];               // exponent of each sum's unit; -1: no fixed-point form
     __shared__ double sh[32];
     const int mu = threadIdx.x / kFxSites, sl = threadIdx.x % kFxSites;  // mu is warp-uniform
-    const int h = G.g.h_begin + pos.bx * kFxSites + sl;
+    const int h = G.g.h_begin + bx * kFxSites + sl;
     const bool live = h < G.g.h_end;
     const int op = a.out_par;
     Hop hp;
@@ -365,7 +364,7 @@ __global__ void __launch_bounds__(4 * kFxSites, 3) k_dslash_fx4(const __grid_con
         }
     }
     const bool act[1] = {true};
-    dslash_epilogue<double, 1, MODE, kFxSites>(G, pos.bx, act, live && mu == 0, h, acc, sh);
+    dslash_epilogue<double, 1, MODE, kFxSites>(G, bx, act, live && mu == 0, h, acc, sh);
 }
 
 }  // namespace stg
