@@ -63,6 +63,17 @@ __device__ __forceinline__ double retr_mul(const M3 &a, const M3 &b)
     return s;
 }
 
+// Re tr(a b^dag)
+__device__ __forceinline__ double retr_mul_dag(const M3 &a, const M3 &b)
+{
+    double s = 0.0;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s = fma(a.m[r][k].im, b.m[r][k].im, fma(a.m[r][k].re, b.m[r][k].re, s));
+    return s;
+}
+
 // G = wr [sum of rectangle staples + kPlaq * sum of plaquette staples], kPlaq = 2 c0 / c1.  Each side
 // (upper, lower) of a plane is one plaquette staple U_nu U_mu U_nu^dag (lower: U_nu^dag U_mu U_nu) and
 // its three forms with one factor replaced by that link's outer staple: 11 products a side (each summed
@@ -221,6 +232,38 @@ __global__ void __launch_bounds__(kPlaqBlock) k_gauge_gather(const __grid_consta
     st(a.out, a.g, mu, x, G);
 }
 
+// Action from the same staples: the plaquette of a plane is Re tr[P(m, n) P(n, m)^dag], the rectangle
+// across link (x, mu) in direction nu Re tr[Sup(mu, nu)(x) Slo(mu, nu)(x-nu)^dag], 18 multiply-adds each
+// where k_gauge_action takes 10 products a plane.  One thread per site over the planes of the pass.
+__global__ void __launch_bounds__(kGaugeBlock) k_gauge_traces(const __grid_constant__ GaugePlaqArgs<double> a,
+                                                              double *partial)
+{
+    using namespace plaq;
+    pdl_enter();
+    __shared__ double sh[33];
+    const int x = blockIdx.x * kGaugeBlock + threadIdx.x, V = a.g.V;
+    double ps = 0.0, rs = 0.0;
+    if (x < V) {
+#pragma unroll 1
+        for (int p = a.p0; p < a.p1; ++p) {
+            int m, n;
+            plane_dirs(p, m, n);
+            const int f = 2 * (p - a.p0);
+            ps += retr_mul_dag(ws_ld<double>(a.P, V, f, x), ws_ld<double>(a.P, V, f + 1, x));
+            rs += retr_mul_dag(ws_ld<double>(a.Sup, V, f, x), ws_ld<double>(a.Slo, V, f, down(a.g, x, n)));
+            rs += retr_mul_dag(ws_ld<double>(a.Sup, V, f + 1, x), ws_ld<double>(a.Slo, V, f + 1, down(a.g, x, m)));
+        }
+    }
+    ps = block_sum(ps, sh);
+    __syncthreads();
+    rs = block_sum(rs, sh);
+    if (threadIdx.x == 0) {
+        double *q = partial + blockIdx.x;
+        q[0] = a.first ? ps : q[0] + ps;
+        q[gridDim.x] = a.first ? rs : q[gridDim.x] + rs;
+    }
+}
+
 __global__ void __launch_bounds__(kGaugeBlock, 1) k_gauge_action(const __grid_constant__ GaugeArgs<double> a)
 {
     __shared__ double sh[33];
@@ -295,12 +338,30 @@ using namespace stg;
 // one plane.
 constexpr size_t kGaugeWorkspace = (size_t)4 << 30;
 
+// The planes per pass and the workspace of `fields` matrices per plane and site; false when there is
+// no room for one plane.
+template <typename C>
+static bool plaq_workspace(long long V, int fields, cudaStream_t st, int &np, C *&ws)
+{
+    if (V > INT_MAX) return false;
+    const size_t per_plane = (size_t)fields * 9 * V * sizeof(C);
+    np = (int)std::min<size_t>(6, std::max<size_t>(1, kGaugeWorkspace / per_plane));
+    keep_pool_mapped(st);
+    cudaError_t e = cudaMallocAsync((void **)&ws, np * per_plane, st);
+    if (e != cudaSuccess && np > 1) {
+        cudaGetLastError();
+        np = 1;
+        e = cudaMallocAsync((void **)&ws, per_plane, st);
+    }
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
+}
+
 template <typename T>
 static bool gauge_force_plaq(const stg_lattice *lat, double beta, const void *links, void *out, int kind,
                              cudaStream_t st, cudaError_t &err)
 {
     using C = typename C2<T>::type;
-    if (lat->V > INT_MAX) return false;
     GaugePlaqArgs<T> a;
     memset(&a, 0, sizeof(a));
     a.g = link_geo(lat->g);
@@ -309,20 +370,11 @@ static bool gauge_force_plaq(const stg_lattice *lat, double beta, const void *li
     a.wp = T(-beta / 3.0 * 2.0 * kC0);
     a.wr = T(-beta / 3.0 * kC1);
     a.kind = kind;
-    const size_t field = (size_t)9 * a.g.V, per_plane = 8 * field * sizeof(C);
-    int np = (int)std::min<size_t>(6, std::max<size_t>(1, kGaugeWorkspace / per_plane));
+    int np = 0;
     C *ws = nullptr;
-    keep_pool_mapped(st);
-    err = cudaMallocAsync((void **)&ws, np * per_plane, st);
-    if (err != cudaSuccess && np > 1) {
-        cudaGetLastError();
-        np = 1;
-        err = cudaMallocAsync((void **)&ws, per_plane, st);
-    }
-    if (err != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
+    if (!plaq_workspace(lat->V, 8, st, np, ws)) return false;
+    err = cudaSuccess;
+    const size_t field = (size_t)9 * a.g.V;
     a.P = ws;
     a.Sup = ws + 2 * np * field;
     a.Slo = ws + 4 * np * field;
@@ -402,7 +454,34 @@ extern "C" stg_status stg_gauge_action(const stg_lattice *lat, double beta, cons
     a.out3 = out3_dev;
     a.nblocks = (int)((a.g.V + kGaugeBlock - 1) / kGaugeBlock);
     STG_CUDA_TRY(cudaMallocAsync((void **)&a.partial, 2 * sizeof(double) * a.nblocks, st));
-    k_gauge_action<<<a.nblocks, kGaugeBlock, 0, st>>>(a);
+    GaugePlaqArgs<double> q;
+    memset(&q, 0, sizeof(q));
+    int np = 0;
+    double2 *ws = nullptr;
+    if (plaq_workspace(lat->V, 6, st, np, ws)) {
+        const size_t field = (size_t)9 * a.g.V;
+        q.g = a.g;
+        q.U = a.U;
+        q.P = ws;
+        q.Sup = ws + 2 * np * field;
+        q.Slo = ws + 4 * np * field;
+        cudaError_t e = cudaSuccess;
+        for (int p = 0; p < 6 && e == cudaSuccess; p += np) {
+            q.p0 = p;
+            q.p1 = std::min(6, p + np);
+            q.first = p == 0;
+            const dim3 pairs((unsigned)((a.g.V + kPlaqBlock - 1) / kPlaqBlock), 2 * (q.p1 - q.p0));
+            e = launch_pdl(k_gauge_staples<double>, pairs, dim3(kPlaqBlock), st, q);
+            if (e == cudaSuccess) e = launch_pdl(k_gauge_traces, dim3(a.nblocks), dim3(kGaugeBlock), st, q, a.partial);
+        }
+        cudaFreeAsync(ws, st);
+        if (e != cudaSuccess) {
+            cudaFreeAsync(a.partial, st);
+            STG_CUDA_TRY(e);
+        }
+    } else {
+        k_gauge_action<<<a.nblocks, kGaugeBlock, 0, st>>>(a);
+    }
     k_gauge_action_finish<<<1, 256, 0, st>>>(a);
     const cudaError_t e = cudaGetLastError();
     cudaFreeAsync(a.partial, st);
