@@ -1290,8 +1290,12 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
         }
     }
     // phase 2: the (rhs, shift) pairs of one instance share link loads, in groups of `rg`
-    // right-hand sides per thread (STG_REFINE_GROUP, 1..8, default 4: faster than 8 at 32^4)
-    int rg = 4;
+    // right-hand sides per thread (STG_REFINE_GROUP, 1..8).  Two by default while their groups fit one
+    // launch: groups share the links through L2 there, and two rhs per thread keep more warps in
+    // flight than four (whole solves, 4 -> 2 rhs: 32^4 16 poles 78.0 -> 73.9 ms, 20^4 14 poles 12.9 -> 12.5 ms,
+    // 16^4 6.84 -> 6.72 ms; 1 rhs 77.0, 8 rhs 80.2 ms at 32^4).  Larger batches would need more launches
+    // per iteration and stay at four.
+    int rg = npair <= 2 * kMaxGroups ? 2 : 4;
     if (const char *e = getenv("STG_REFINE_GROUP")) rg = std::max(1, std::min(kMaxRhs, atoi(e)));
     DPlan p2, p64, p64f;  // p64: residuals with gh; p64f: the same with the F64 gauge (verification)
     DPlan pinc;           // anchored refinement: r_hi = r_hi - A y_hi with gh
