@@ -14,8 +14,9 @@
 // 1.62e-16 of the 64-bit reference).  Links of 2 and above, infinities, NaNs, subnormal numbers and
 // vectors near the ends of the exponent range go through the FP64 loop, thread by thread.
 // D at 32^4 312 -> 152 us (of 100 us at the copy bandwidth), 24^4 108 -> 57 us, 16^4 46 -> 15 us, 8^4 15 ->
-// 10 us.  What bounds it now: the integer pipes (864 products and ~1400 other operations a site)
-// and, with one thread per site, loads in flight at 16 to 20 warps per SM.
+// 10 us.  What bounds it now: the integer pipes (864 products and ~1400 other operations a site; at
+// 24^4 the multiply pipe is 57 % and the ALU 41 % busy) and, with one thread per site, loads in flight
+// at 16 to 20 warps per SM.
 #pragma once
 
 #include "dslash.cuh"
@@ -65,6 +66,19 @@ __device__ __forceinline__ long long fx_shift(long long x, int d)
     return (x + ((1ll << d) >> 1)) >> d;
 }
 
+// |d| < 2 (false for NaN), and d 2^55 rounded, both on the integer pipes: in FP64 the copy of a gauge
+// was bound by the multiplications and conversions
+__device__ __forceinline__ bool fx_below_two(double d) { return (__double2hiint(d) & 0x7fffffff) < 0x40000000; }
+__device__ __forceinline__ long long fx_round55(double d)
+{
+    const int hi = __double2hiint(d);
+    const int e = (hi & 0x7fffffff) >> 20;  // d = significand 2^(e - 1075)
+    const long long m = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(d);
+    const int s = 1020 - e;  // significand 2^(e - 1075 + 55)
+    const long long v = s <= 0 ? m << -s : fx_shift(m, s);  // s >= -3: below 2^56
+    return hi < 0 ? -v : v;
+}
+
 // Fixed-point links: per (mu, parity) block 9 chunks over Vh of (re.l1, re.l0, im.l1, im.l0)
 struct LinkFX {
     static constexpr int kBytes = 144;
@@ -84,9 +98,8 @@ struct LinkFX {
         int4 *p = static_cast<int4 *>(blk);
         bool ok = true;
         for (int k = 0; k < 9; ++k) {
-            ok &= fabs(m[k].x) < 2.0 && fabs(m[k].y) < 2.0;  // false for NaN
-            const FxNum re = fx_split(ok ? __double2ll_rn(m[k].x * 36028797018963968.0) : 0);  // 2^55
-            const FxNum im = fx_split(ok ? __double2ll_rn(m[k].y * 36028797018963968.0) : 0);
+            ok &= fx_below_two(m[k].x) && fx_below_two(m[k].y);
+            const FxNum re = fx_split(ok ? fx_round55(m[k].x) : 0), im = fx_split(ok ? fx_round55(m[k].y) : 0);
             p[(size_t)k * Vh + h] = make_int4(re.l1, re.l0, im.l1, im.l0);
         }
         return ok;
