@@ -98,7 +98,9 @@ int64_t stg_lattice_sites(const stg_lattice *lat, int32_t parity);
  * [mu][parity][chunk][Vh] at precision `prec`.  recon = STG_RECON12 keeps only rows 1 and
  * 2 and rebuilds row 3 = (r1 x r2)^* in registers (Sec. 4.1); this is exact only for
  * SU(3) links.  BF16/F16 require STG_RECON12.  The copy is finished when the work on
- * `stream` is.  The lattice must outlive the gauge. */
+ * `stream` is.  The lattice must outlive the gauge.  An F64 / STG_RECON18 gauge of 2048 sites or
+ * more keeps a fixed-point copy of its links (the same size), made by the first operator or solve
+ * that uses them (not while a stream captures; without memory for it, FP64 arithmetic is used). */
 stg_status stg_gauge_create(const stg_lattice *lat, const void *links_c128_dev, stg_prec prec, stg_recon recon,
                             void *stream, stg_gauge **out);
 /* As stg_gauge_create, with a U(1) phase field: theta_dev (device, FP64, canonical [4][V], radians)
@@ -116,7 +118,7 @@ stg_status stg_gauge_create_u1(const stg_lattice *lat, const void *links_c128_de
  * without allocating: the MD evolution changes the links every step (Sec. 3), and a production
  * loop keeps one gauge per precision and refreshes it.  theta_dev must be given (device, FP64,
  * [4][V]) exactly when the gauge was created with stg_gauge_create_u1, NULL otherwise.  The
- * double-single and FP32 companions that solves and forces created for an F64 gauge are refreshed
+ * double-single, FP32 and fixed-point companions that solves and forces created for an F64 gauge are refreshed
  * too.  Stream-ordered: work already queued on `stream` sees the old links, later work the new;
  * the gauge may not be in use on another stream meanwhile.  STG_ERR_ARG on null, misaligned or
  * mismatched arguments. */
@@ -322,7 +324,7 @@ stg_status stg_mscg_solve_batched(int32_t ninst, const stg_instance *inst, const
  *           U -> exp(eps X) U, X in su(3)), or
  *   kind 1: W^dag = dS/dRe U + i dS/dIm U.
  * y_i is computed with a double-single (FP32-pair, 48-bit significand) copy of the links, which
- * the F64 gauge creates on first use and keeps; W and F are accumulated in FP64.
+ * the F64 gauge creates on first use and keeps; W and F are formed in double-single and widened.
  * x_c128_dev[nshift]: canonical complex128 even fields (device);
  * out_c128_dev: canonical complex128 [4][V][3][3] (device).  g_f64 must be an F64 gauge. */
 stg_status stg_fermion_force(const stg_gauge *g_f64, int32_t nshift, const double *residues,

@@ -15,7 +15,7 @@
 // direction mu gathers its rank-nshift sum of outer products (no atomics: every link is owned by
 // exactly one thread) -- in double-single on the FP32 pipes (k_force_ds, the default: GB300 issues
 // FP64 at 1/64 of FP32, and the FP64 gather was FP64-pipe bound at ~94 %), or in FP64 (k_force,
-// with STG_FORCE_FP64=1).  F = TA(U W) and W^dag are formed in FP64 from the double-single W.
+// with STG_FORCE_FP64=1).  F = TA(U W) is formed in double-single too, its 9 numbers then widened.
 #include <cstdlib>
 #include <cstring>
 #include <vector>
