@@ -34,7 +34,7 @@ struct DGroup {
     Geom g;
     const void *links;
     const void *fx_links;  // fixed-point copy of F64 18-real links (set_fx), or null
-    const int *fx_bad;     // device flag beside it: nonzero when some link has no fixed-point form
+    const int *fx_state;   // device words beside it: nonzero when some link has no fixed-point form; exponent of the unit
     int nrhs;
     const void *in[kMaxRhs];
     void *out[kMaxRhs];

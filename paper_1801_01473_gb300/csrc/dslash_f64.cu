@@ -52,8 +52,27 @@ cudaError_t launch_dslash_f64r18(const DArgs &a, int mode, int bs, cudaStream_t 
 }
 cudaError_t launch_dslash_f64r12(const DArgs &a, int mode, int bs, cudaStream_t st) { return launch_dslash_t<LinkF64R12>(a, mode, bs, st); }
 
-// FP64 18-real links -> fixed-point links; *bad is set when some link has no fixed-point form
-__global__ void k_links_to_fx(int Vh, const void *__restrict__ src, void *__restrict__ dst, int *bad)
+// The state beside a fixed-point copy before its links are written: no link without the form yet, and the
+// exponent of the links' unit, the power of two at or above the first link's |U| / sqrt 3 (1 for SU(3)).
+__global__ void k_fx_begin(const double2 *__restrict__ first, size_t stride, int *state)
+{
+    double n = 0.0;
+    for (int k = 0; k < 9; ++k) {
+        const double2 u = first[k * stride];
+        n = fma(u.x, u.x, fma(u.y, u.y, n));
+    }
+    n = sqrt(n / 3.0) * (1.0 - 0x1p-20);
+    int ke = 0;
+    if (n > 0x1p-400 && n < 0x1p400) {
+        const int hi = __double2hiint(n);
+        ke = (hi >> 20) - 1023 + ((hi & 0xfffff) != 0 || __double2loint(n) != 0 ? 1 : 0);
+    }
+    state[0] = 0;
+    state[1] = ke;
+}
+
+// FP64 18-real links -> fixed-point links; state[0] is set when some link has no fixed-point form
+__global__ void k_links_to_fx(int Vh, const void *__restrict__ src, void *__restrict__ dst, int *state)
 {
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (tid >= 8LL * Vh) return;
@@ -61,14 +80,13 @@ __global__ void k_links_to_fx(int Vh, const void *__restrict__ src, void *__rest
     const double2 *p = reinterpret_cast<const double2 *>(static_cast<const char *>(src) + (size_t)blk * Vh * LinkF64R18::kBytes);
     double2 m[9];
     for (int k = 0; k < 9; ++k) m[k] = p[(size_t)k * Vh + h];
-    if (!LinkFX::pack(static_cast<char *>(dst) + (size_t)blk * Vh * LinkFX::kBytes, Vh, h, m)) *bad = 1;
+    if (!LinkFX::pack(static_cast<char *>(dst) + (size_t)blk * Vh * LinkFX::kBytes, Vh, h, m, state[1])) state[0] = 1;
 }
 
-cudaError_t launch_links_to_fx(int Vh, const void *links, void *fx_links, int *bad, cudaStream_t st)
+cudaError_t launch_links_to_fx(int Vh, const void *links, void *fx_links, int *state, cudaStream_t st)
 {
-    cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    k_links_to_fx<<<(unsigned)((8LL * Vh + 255) / 256), 256, 0, st>>>(Vh, links, fx_links, bad);
+    k_fx_begin<<<1, 1, 0, st>>>(static_cast<const double2 *>(links), (size_t)Vh, state);
+    k_links_to_fx<<<(unsigned)((8LL * Vh + 255) / 256), 256, 0, st>>>(Vh, links, fx_links, state);
     return cudaGetLastError();
 }
 }  // namespace stg

@@ -65,8 +65,8 @@ stg_status ds_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge *
 // synchronisation and the next call pays for mapping them again).  Does nothing while `st` captures.
 void keep_pool_mapped(cudaStream_t st);
 
-// F64 18-real links -> the fixed-point layout of dslash_fx.cuh, *bad = 0 or 1 (dslash_f64.cu)
-cudaError_t launch_links_to_fx(int Vh, const void *links, void *fx_links, int *bad, cudaStream_t st);
+// F64 18-real links -> the fixed-point layout of dslash_fx.cuh and its two words of state (dslash_f64.cu)
+cudaError_t launch_links_to_fx(int Vh, const void *links, void *fx_links, int *state, cudaStream_t st);
 // Gives the group the fixed-point copy of its F64 18-real links, created on first use and owned by
 // the gauge.  Leaves the group on the FP64 kernel for other links, while `st` captures before the
 // first use, and when there is no memory for the copy.

@@ -447,7 +447,7 @@ stg_status ds_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge *
     return STG_OK;
 }
 
-static int *fx_flag(const stg_gauge *g) { return reinterpret_cast<int *>(static_cast<char *>(g->fx_links) + g->bytes); }
+static int *fx_state(const stg_gauge *g) { return reinterpret_cast<int *>(static_cast<char *>(g->fx_links) + g->bytes); }
 
 void set_fx(DGroup &G, const stg_gauge *g, cudaStream_t st)
 {
@@ -463,7 +463,7 @@ void set_fx(DGroup &G, const stg_gauge *g, cudaStream_t st)
         }
         // same bytes per link as the FP64 layout, the flag behind them
         cudaError_t e = cudaMalloc(&g->fx_links, g->bytes + 256);
-        if (e == cudaSuccess) e = launch_links_to_fx(g->g.Vh, g->links, g->fx_links, fx_flag(g), st);
+        if (e == cudaSuccess) e = launch_links_to_fx(g->g.Vh, g->links, g->fx_links, fx_state(g), st);
         // other streams may use the copy from now on
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) {
@@ -474,7 +474,7 @@ void set_fx(DGroup &G, const stg_gauge *g, cudaStream_t st)
         }
     }
     G.fx_links = g->fx_links;
-    G.fx_bad = fx_flag(g);
+    G.fx_state = fx_state(g);
 }
 
 stg_status f32_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge **out)
@@ -753,7 +753,7 @@ stg_status stg_gauge_update(stg_gauge *g, const void *links_c128_dev, const doub
     std::lock_guard<std::mutex> lk(g_companion_mu);
     if (g->ds_copy) STG_CUDA_TRY(fill_ds_companion(g, g->ds_copy, st));
     if (g->f32_copy) STG_CUDA_TRY(fill_f32_companion(g, g->f32_copy, st));
-    if (g->fx_links) STG_CUDA_TRY(launch_links_to_fx(g->g.Vh, g->links, g->fx_links, fx_flag(g), st));
+    if (g->fx_links) STG_CUDA_TRY(launch_links_to_fx(g->g.Vh, g->links, g->fx_links, fx_state(g), st));
     return STG_OK;
 }
 
