@@ -99,8 +99,8 @@ int64_t stg_lattice_sites(const stg_lattice *lat, int32_t parity);
  * 2 and rebuilds row 3 = (r1 x r2)^* in registers (Sec. 4.1); this is exact only for
  * SU(3) links.  BF16/F16 require STG_RECON12.  The copy is finished when the work on
  * `stream` is.  The lattice must outlive the gauge.  An F64 / STG_RECON18 gauge of 2048 sites or
- * more keeps a fixed-point copy of its links (the same size), made by the first operator or solve
- * that uses them (not while a stream captures; without memory for it, FP64 arithmetic is used). */
+ * more whose links take up to 16 GiB has a fixed-point copy of them beside them (the same size again,
+ * not in stg_gauge_bytes); without memory for it the gauge does without, on FP64 arithmetic. */
 stg_status stg_gauge_create(const stg_lattice *lat, const void *links_c128_dev, stg_prec prec, stg_recon recon,
                             void *stream, stg_gauge **out);
 /* As stg_gauge_create, with a U(1) phase field: theta_dev (device, FP64, canonical [4][V], radians)
@@ -118,8 +118,8 @@ stg_status stg_gauge_create_u1(const stg_lattice *lat, const void *links_c128_de
  * without allocating: the MD evolution changes the links every step (Sec. 3), and a production
  * loop keeps one gauge per precision and refreshes it.  theta_dev must be given (device, FP64,
  * [4][V]) exactly when the gauge was created with stg_gauge_create_u1, NULL otherwise.  The
- * double-single, FP32 and fixed-point companions that solves and forces created for an F64 gauge are refreshed
- * too.  Stream-ordered: work already queued on `stream` sees the old links, later work the new;
+ * double-single and FP32 companions that solves and forces created for an F64 gauge are refreshed
+ * too (by a captured update: those that existed at its capture).  Stream-ordered: work already queued on `stream` sees the old links, later work the new;
  * the gauge may not be in use on another stream meanwhile.  STG_ERR_ARG on null, misaligned or
  * mismatched arguments. */
 stg_status stg_gauge_update(stg_gauge *g, const void *links_c128_dev, const double *theta_dev, void *stream);

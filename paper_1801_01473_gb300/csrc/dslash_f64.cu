@@ -54,11 +54,11 @@ cudaError_t launch_dslash_f64r12(const DArgs &a, int mode, int bs, cudaStream_t 
 
 // The state beside a fixed-point copy before its links are written: no link without the form yet, and the
 // exponent of the links' unit, the power of two at or above the first link's |U| / sqrt 3 (1 for SU(3)).
-__global__ void k_fx_begin(const double2 *__restrict__ first, size_t stride, int *state)
+__global__ void k_fx_begin(const double2 *__restrict__ first, int *state)
 {
     double n = 0.0;
     for (int k = 0; k < 9; ++k) {
-        const double2 u = first[k * stride];
+        const double2 u = first[k];
         n = fma(u.x, u.x, fma(u.y, u.y, n));
     }
     n = sqrt(n / 3.0) * (1.0 - 0x1p-20);
@@ -71,22 +71,30 @@ __global__ void k_fx_begin(const double2 *__restrict__ first, size_t stride, int
     state[1] = ke;
 }
 
-// FP64 18-real links -> fixed-point links; state[0] is set when some link has no fixed-point form
-__global__ void k_links_to_fx(int Vh, const void *__restrict__ src, void *__restrict__ dst, int *state)
+// One thread per link (mu, i), as k_pack_links; state[0] is set when some link has no fixed-point form.
+// Bound by HBM (a link read once and written twice): update of a 32^4 gauge 294 us, links alone 210.
+__global__ void k_pack_links_fx(Geom g, const double2 *__restrict__ canon, void *__restrict__ links,
+                                void *__restrict__ fx_links, int *state)
 {
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= 8LL * Vh) return;
-    const int blk = (int)(tid / Vh), h = (int)(tid - (long long)blk * Vh);
-    const double2 *p = reinterpret_cast<const double2 *>(static_cast<const char *>(src) + (size_t)blk * Vh * LinkF64R18::kBytes);
+    const long long V = 2LL * g.Vh, tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (tid >= 4 * V) return;
+    const int mu = (int)(tid / V), i = (int)(tid - mu * V), ke = state[1];
+    const int x = i % g.L[0], r = i / g.L[0], y = r % g.L[1], r2 = r / g.L[1], z = r2 % g.L[2], t = r2 / g.L[2];
     double2 m[9];
-    for (int k = 0; k < 9; ++k) m[k] = p[(size_t)k * Vh + h];
-    if (!LinkFX::pack(static_cast<char *>(dst) + (size_t)blk * Vh * LinkFX::kBytes, Vh, h, m, state[1])) state[0] = 1;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m[k] = canon[tid * 9 + k];
+    const size_t blk = (size_t)(mu * 2 + ((x + y + z + t) & 1)) * g.Vh * LinkF64R18::kBytes;
+    LinkF64R18::pack(static_cast<char *>(links) + blk, g.Vh, i >> 1, m);
+    if (!LinkFX::pack(static_cast<char *>(fx_links) + blk, g.Vh, i >> 1, m, ke)) state[0] = 1;
 }
 
-cudaError_t launch_links_to_fx(int Vh, const void *links, void *fx_links, int *state, cudaStream_t st)
+cudaError_t launch_pack_links_fx(const Geom &g, const void *canon, void *links, void *fx_links, int *state,
+                                 cudaStream_t st)
 {
-    k_fx_begin<<<1, 1, 0, st>>>(static_cast<const double2 *>(links), (size_t)Vh, state);
-    k_links_to_fx<<<(unsigned)((8LL * Vh + 255) / 256), 256, 0, st>>>(Vh, links, fx_links, state);
+    static_assert(LinkFX::kBytes == LinkF64R18::kBytes, "the copy has the size and the blocks of the links");
+    const double2 *c = static_cast<const double2 *>(canon);
+    k_fx_begin<<<1, 1, 0, st>>>(c, state);
+    k_pack_links_fx<<<(unsigned)((8LL * g.Vh + 255) / 256), 256, 0, st>>>(g, c, links, fx_links, state);
     return cudaGetLastError();
 }
 }  // namespace stg

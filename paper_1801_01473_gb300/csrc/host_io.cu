@@ -114,7 +114,7 @@ extern "C" stg_status stg_dslash_host(const stg_gauge *g, int32_t out_parity, st
     a.out_par = out_parity;
     a.grp[0].g = g->g;
     a.grp[0].links = g->links;
-    set_fx(a.grp[0], g, P.s_cmp);
+    set_fx(a.grp[0], g);
     a.grp[0].nrhs = 1;
     for (int k = 0; k < nfield; ++k) {
         const int s = k % kSlots;

@@ -118,7 +118,7 @@ extern "C" stg_status stg_slab_dslash_part(const stg_gauge *g, int32_t out_parit
         G.g.h_begin = s0 * hs;
         G.g.h_end = s1 * hs;
         G.links = g->links;
-        set_fx(G, g, (cudaStream_t)stream);
+        set_fx(G, g);
         G.nrhs = 1;
         G.in[0] = in_dev;
         G.out[0] = out_dev;
@@ -150,7 +150,7 @@ extern "C" stg_status stg_slab_dslash_xpay(const stg_gauge *g, int32_t out_parit
     DGroup &G = a.grp[0];
     G.g = g->g;
     G.links = g->links;
-    set_fx(G, g, st);
+    set_fx(G, g);
     G.nrhs = 1;
     G.in[0] = in_dev;
     G.out[0] = out_dev;

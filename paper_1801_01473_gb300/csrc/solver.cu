@@ -1270,7 +1270,7 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
             memset(&Goe, 0, sizeof(Goe));
             Goe.g = ii[k].gi->g;
             Goe.links = ii[k].gi->links;
-            set_fx(Goe, ii[k].gi, ws);
+            set_fx(Goe, ii[k].gi);
             Goe.nrhs = std::min(kMaxRhs, ii[k].nrhs - r0);
             Geo = Goe;
             for (int j = 0; j < Goe.nrhs; ++j) {
@@ -1306,13 +1306,12 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
             memset(&Goe, 0, sizeof(Goe));
             Goe.g = ii[k].gr->g;
             Goe.links = ii[k].gr->links;
-            set_fx(Goe, ii[k].gr, ws);
+            set_fx(Goe, ii[k].gr);
             Goe.nrhs = std::min(rg, cnt - q0);
             Geo = Goe;
             Hoe = Goe;
             Hoe.links = ii[k].gh->links;
-            Hoe.fx_links = nullptr;
-            set_fx(Hoe, ii[k].gh, ws);
+            set_fx(Hoe, ii[k].gh);
             Heo = Hoe;
             for (int j = 0; j < Goe.nrhs; ++j) {
                 const int pidx = first + q0 + j;
@@ -1354,20 +1353,12 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
                 add_group(pinc.eo, Ieo, 0);
             }
             Hoe.links = Heo.links = ii[k].g64->links;
+            set_fx(Hoe, ii[k].g64);
+            set_fx(Heo, ii[k].g64);
             add_group(p64f.oe, Hoe, 1);
             add_group(p64f.eo, Heo, 0);
         }
     }
-
-    // the fixed-point copies of the F64 gauges, for p64f only once it is launched: a loose mixed solve
-    // never does, and would have its gauge refresh a copy at every update (419 us at 32^4)
-    auto fx_p64f = [&]() {
-        for (std::vector<DArgs> *lst : {&p64f.oe, &p64f.eo})
-            for (DArgs &a : *lst)
-                for (int q = 0; q < a.ngroups; ++q)
-                    for (int k = 0; k < ninst; ++k)
-                        if (a.grp[q].links == ii[k].g64->links) set_fx(a.grp[q], ii[k].g64, ws);
-    };
 
     const dim3 vgrid1(nblkv_max, nsys), vgrid2(nblkv_max, npair);
 
@@ -1591,7 +1582,6 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
             // the FP64 anchor: r_hi = b - A x_hi with the F64 gauge, then everything back to H
             stg_status cs = convert_xb(true, false);
             if (cs != STG_OK) return cs;
-            fx_p64f();
             for (const DArgs &a : p64f.oe) STG_CUDA_TRY(launch_dslash(kind_64, a, 0, ws));
             for (const DArgs &a : p64f.eo) STG_CUDA_TRY(launch_dslash(kind_64, a, 2, ws));
             cs = convert_xb(false, true);
@@ -1676,7 +1666,6 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
         }
         STG_CUDA_TRY(cudaMemcpyAsync(noupd, h_noupd.data(), sizeof(int) * npair, cudaMemcpyHostToDevice, ws));
         if (any_verify) {
-            fx_p64f();
             for (const DArgs &a : p64f.oe) STG_CUDA_TRY(launch_dslash(kind_64, a, 0, ws));
             for (const DArgs &a : p64f.eo) STG_CUDA_TRY(launch_dslash(kind_64, a, 2, ws));
             k_verify<<<npair, 32, 0, ws>>>(d_v2, d_true_rr, noupd);

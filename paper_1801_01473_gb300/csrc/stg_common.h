@@ -65,12 +65,12 @@ stg_status ds_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge *
 // synchronisation and the next call pays for mapping them again).  Does nothing while `st` captures.
 void keep_pool_mapped(cudaStream_t st);
 
-// F64 18-real links -> the fixed-point layout of dslash_fx.cuh and its two words of state (dslash_f64.cu)
-cudaError_t launch_links_to_fx(int Vh, const void *links, void *fx_links, int *state, cudaStream_t st);
-// Gives the group the fixed-point copy of its F64 18-real links, created on first use and owned by
-// the gauge.  Leaves the group on the FP64 kernel for other links, while `st` captures before the
-// first use, and when there is no memory for the copy.
-void set_fx(DGroup &G, const stg_gauge *g, cudaStream_t st);
+// Canonical links -> F64 18-real links and their fixed-point copy with its two words of state (dslash_f64.cu)
+cudaError_t launch_pack_links_fx(const Geom &g, const void *canon, void *links, void *fx_links, int *state,
+                                 cudaStream_t st);
+// Gives the group the fixed-point copy of the gauge's links, or none where the gauge has none (the group
+// then takes the FP64 kernel).
+void set_fx(DGroup &G, const stg_gauge *g);
 
 // Error reporting (thread-local message read by stg_last_error).
 stg_status set_error(stg_status s, const std::string &msg);
@@ -95,7 +95,7 @@ struct stg_gauge {
     size_t scratch_count;  // doubles in scratch
     mutable stg_gauge *f32_copy;  // lazily created F32 12-real companion (F64 gauges only)
     mutable stg_gauge *ds_copy;   // lazily created double-single companion (F64 gauges only)
-    mutable void *fx_links;       // lazily created fixed-point copy of F64 18-real links, its flag behind it
+    void *fx_links;  // fixed-point copy of F64 18-real links, its state behind it (in the allocation of links), or null
 };
 
 #define STG_CUDA_TRY(call)                                       \

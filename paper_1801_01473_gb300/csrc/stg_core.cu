@@ -449,32 +449,10 @@ stg_status ds_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge *
 
 static int *fx_state(const stg_gauge *g) { return reinterpret_cast<int *>(static_cast<char *>(g->fx_links) + g->bytes); }
 
-void set_fx(DGroup &G, const stg_gauge *g, cudaStream_t st)
+void set_fx(DGroup &G, const stg_gauge *g)
 {
-    // a lattice below 2048 sites is bound by the launch (4^4 15 us against 11 us in fixed point): not
-    // worth the copy
-    if (g->kind != kF64R18 || g->lat->V < 2048) return;
-    std::lock_guard<std::mutex> lk(g_companion_mu);
-    if (!g->fx_links) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            return;
-        }
-        // same bytes per link as the FP64 layout, the flag behind them
-        cudaError_t e = cudaMalloc(&g->fx_links, g->bytes + 256);
-        if (e == cudaSuccess) e = launch_links_to_fx(g->g.Vh, g->links, g->fx_links, fx_state(g), st);
-        // other streams may use the copy from now on
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            cudaFree(g->fx_links);
-            g->fx_links = nullptr;
-            return;
-        }
-    }
     G.fx_links = g->fx_links;
-    G.fx_state = fx_state(g);
+    G.fx_state = g->fx_links ? fx_state(g) : nullptr;
 }
 
 stg_status f32_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge **out)
@@ -683,6 +661,23 @@ int64_t stg_lattice_sites(const stg_lattice *lat, int32_t parity)
     return -1;
 }
 
+// Bytes of the fixed-point copy that comes with the links.  A lattice below 2048 sites is bound by the launch
+// (4^4 15 us against 11 us in fixed point) and has none; nor do links of more than 16 GiB (beyond ~74^4), so
+// that the copy never decides what fits the card.
+static size_t fx_copy_bytes(int kind, long long V, size_t bytes)
+{
+    return kind == kF64R18 && V >= 2048 && bytes <= ((size_t)16 << 30) ? bytes + 256 : 0;
+}
+
+// canonical links (and phases) into the gauge, with the fixed-point copy where it has one.  The copy is
+// written with the links wherever they are, so that no operator makes it, waits for it or sees an old one.
+static cudaError_t fill_links(const stg_gauge *g, const void *links, const double *theta, cudaStream_t st)
+{
+    if (theta) return launch_pack_links_u1(g->kind, g->g, links, theta, g->links, st);
+    if (g->fx_links) return launch_pack_links_fx(g->g, links, g->links, g->fx_links, fx_state(g), st);
+    return launch_pack_links(g->kind, g->g, links, g->links, st);
+}
+
 static stg_status gauge_create(const stg_lattice *lat, const void *links_c128_dev, const double *theta_dev,
                                stg_prec prec, stg_recon recon, void *stream, stg_gauge **out)
 {
@@ -716,11 +711,16 @@ static stg_status gauge_create(const stg_lattice *lat, const void *links_c128_de
     g->ds_copy = nullptr;
     g->fx_links = nullptr;
     g->scratch_count = (size_t)dslash_partials(lat->g.Vh);
-    cudaError_t e = cudaMalloc(&g->links, g->bytes);
+    size_t fx = fx_copy_bytes(kind, lat->V, g->bytes);
+    cudaError_t e = cudaMalloc(&g->links, g->bytes + fx);
+    if (e != cudaSuccess && fx) {  // no room for the copy
+        cudaGetLastError();
+        fx = 0;
+        e = cudaMalloc(&g->links, g->bytes);
+    }
+    if (e == cudaSuccess && fx) g->fx_links = static_cast<char *>(g->links) + g->bytes;
     if (e == cudaSuccess) e = cudaMalloc(&g->scratch, g->scratch_count * sizeof(double));
-    if (e == cudaSuccess)
-        e = theta_dev ? launch_pack_links_u1(kind, lat->g, links_c128_dev, theta_dev, g->links, (cudaStream_t)stream)
-                      : launch_pack_links(kind, lat->g, links_c128_dev, g->links, (cudaStream_t)stream);
+    if (e == cudaSuccess) e = fill_links(g, links_c128_dev, theta_dev, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         stg_status s = cuda_error(e, "stg_gauge_create");
         cudaFree(g->links);
@@ -748,12 +748,10 @@ stg_status stg_gauge_update(stg_gauge *g, const void *links_c128_dev, const doub
     if (theta_dev && (reinterpret_cast<uintptr_t>(theta_dev) & 7))
         return set_error(STG_ERR_ARG, "stg_gauge_update: theta not 8-byte aligned");
     cudaStream_t st = (cudaStream_t)stream;
-    STG_CUDA_TRY(u1 ? launch_pack_links_u1(g->kind, g->g, links_c128_dev, theta_dev, g->links, st)
-                    : launch_pack_links(g->kind, g->g, links_c128_dev, g->links, st));
+    STG_CUDA_TRY(fill_links(g, links_c128_dev, theta_dev, st));
     std::lock_guard<std::mutex> lk(g_companion_mu);
     if (g->ds_copy) STG_CUDA_TRY(fill_ds_companion(g, g->ds_copy, st));
     if (g->f32_copy) STG_CUDA_TRY(fill_f32_companion(g, g->f32_copy, st));
-    if (g->fx_links) STG_CUDA_TRY(launch_links_to_fx(g->g.Vh, g->links, g->fx_links, fx_state(g), st));
     return STG_OK;
 }
 
@@ -771,7 +769,6 @@ void stg_gauge_destroy(stg_gauge *g)
     if (g->f32_copy) stg_gauge_destroy(g->f32_copy);
     if (g->ds_copy) stg_gauge_destroy(g->ds_copy);
     cudaFree(g->links);
-    cudaFree(g->fx_links);
     cudaFree(g->scratch);
     delete g;
 }
@@ -854,7 +851,7 @@ stg_status stg_dslash_multi(const stg_gauge *g, int32_t out_parity, int32_t nrhs
             DGroup &G = a.grp[ng++];
             G.g = g->g;
             G.links = g->links;
-            set_fx(G, g, (cudaStream_t)stream);
+            set_fx(G, g);
             G.nrhs = (nrhs - base) < kMaxRhs ? (nrhs - base) : kMaxRhs;
             for (int j = 0; j < G.nrhs; ++j) {
                 G.in[j] = ib + (size_t)(base + j) * stride_bytes;
@@ -901,7 +898,7 @@ stg_status stg_normal_op(const stg_gauge *g, double mass, double shift, void *ou
     DGroup &G = a.grp[0];
     G.g = g->g;
     G.links = g->links;
-    set_fx(G, g, st);
+    set_fx(G, g);
     G.nrhs = 1;
     // D_oe: even -> odd
     a.out_par = 1;
