@@ -108,10 +108,22 @@ static cudaError_t launch_dslash_tuned(int kind, const DArgs &a, int mode, cudaS
 // 152 us) and of links with a U(1) phase field (instantiated for one rhs only).
 cudaError_t launch_dslash(int kind, const DArgs &a, int mode, cudaStream_t st)
 {
-    int maxv, maxr;
+    int maxv, maxr, nfx = 0;
     dslash_extent(a, maxv, maxr);
-    bool fx = kind == kF64R18;
-    for (int k = 0; k < a.ngroups; ++k) fx = fx && a.grp[k].fx_links;
+    for (int k = 0; k < a.ngroups; ++k) nfx += a.grp[k].fx_links != nullptr;
+    if (nfx > 0 && nfx < a.ngroups) {  // each group on its own kernel, whatever else the launch carries
+        for (int fixed = 0; fixed < 2; ++fixed) {
+            DArgs b;
+            memset(&b, 0, sizeof(b));
+            b.out_par = a.out_par;
+            for (int k = 0; k < a.ngroups; ++k)
+                if ((a.grp[k].fx_links != nullptr) == (fixed == 1)) b.grp[b.ngroups++] = a.grp[k];
+            const cudaError_t e = launch_dslash(kind, b, mode, st);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
+    const bool fx = nfx > 0;
     if ((!kind_is_ds(kind) && !kind_has_u1(kind) && !fx) || maxr <= 1) return launch_dslash_tuned(kind, a, mode, st);
     DArgs b;
     memset(&b, 0, sizeof(b));
@@ -147,7 +159,8 @@ static cudaError_t launch_dslash_tuned(int kind, const DArgs &a, int mode, cudaS
     const int nt = dslash_nrhs_template(maxr);
     int dev = 0;
     cudaGetDevice(&dev);
-    const auto key = std::make_tuple(dev, kind, mode, nt, maxv);
+    // (groups of fixed-point links run another kernel than the FP64 links of the same kind: 16)
+    const auto key = std::make_tuple(dev, kind | (a.grp[0].fx_links ? 16 : 0), mode, nt, maxv);
     // the lookahead kernel exists for FP32 12-real links with 3 or 4 right-hand sides
     const bool ahead_ok = kind == kF32R12 && nt == 4;
     // STG_DSLASH_SHAPE=64|128|256|shared|ahead fixes the launch shape (tests use it to run each variant)

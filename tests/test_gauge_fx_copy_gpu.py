@@ -73,3 +73,18 @@ def test_first_operator_neither_allocates_nor_waits():
     assert not torch.cuda.current_stream().query()  # the call returned before the work ahead of it was done
     torch.cuda.synchronize()
     assert torch.cuda.mem_get_info()[0] == free
+
+
+@pytest.mark.parametrize("others", [[(4, 4, 6, 4)], [(24, 24, 24, 14), (4, 4, 6, 4)]])
+def test_batch_with_lattices_without_a_copy(others):
+    """A batched FP64 solve over lattices with and without a copy gives bitwise the single solves."""
+    import paper_1801_01473_gb300 as p
+    insts = []
+    for k, dims in enumerate([DIMS] + others):
+        u = _gpu(S.gauge_links(dims, "expih", 211 + k))
+        insts.append((p.Gauge(p.Lattice(dims), u, "f64", 18), None, [_gpu(S.gaussian_field(dims, 215 + k + 3 * j)) for j in range(2)]))
+    both = p.mscg_batched(insts, [0.01, 0.5], 0.3, tol=1e-10)
+    for (g, _, bs), (x, _) in zip(insts, both):
+        for b, xb in zip(bs, x):
+            one, _ = p.mscg(g, b, [0.01, 0.5], 0.3, tol=1e-10)
+            assert torch.equal(xb, one)
