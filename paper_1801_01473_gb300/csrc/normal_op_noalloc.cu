@@ -95,6 +95,7 @@ extern "C" stg_status stg_normal_op_noalloc(const stg_gauge *g, double mass, dou
     DGroup &G = a.grp[0];
     G.g = g->g;
     G.links = g->links;
+    set_fx(G, g);  // the gauge's own copy: nothing is allocated here
     G.nrhs = 1;
     a.out_par = 1;  // D_oe: even -> odd, into the static temporary
     G.in[0] = in_even_dev;

@@ -88,3 +88,16 @@ def test_batch_with_lattices_without_a_copy(others):
         for b, xb in zip(bs, x):
             one, _ = p.mscg(g, b, [0.01, 0.5], 0.3, tol=1e-10)
             assert torch.equal(xb, one)
+
+
+@pytest.mark.parametrize("dims", [DIMS, (24, 24, 24, 14)])
+def test_noalloc_operator_is_the_normal_operator(dims):
+    import paper_1801_01473_gb300 as p
+    lat = p.Lattice(dims)
+    g = p.Gauge(lat, _links(221, dims), "f64", 18)
+    x = p.pack(lat, _gpu(S.gaussian_field(dims, 222)), "f64")
+    want, got, tmp = torch.empty_like(x), torch.empty_like(x), torch.empty_like(x)
+    pq = torch.empty(2, dtype=torch.float64, device="cuda")
+    p.normal_op_(g, 0.1, 0.03, want, x, tmp, pq[:1])
+    p.normal_op_noalloc_(g, 0.1, 0.03, got, x, pq[1:])
+    assert torch.equal(got, want) and float(pq[0]) == float(pq[1])
