@@ -351,7 +351,13 @@ stg_status stg_fermion_force_prec(const stg_gauge *g_f64, stg_prec prec, int32_t
  * links_dev: canonical [4][V][3][3] U^(0) (device, read only);
  * levels_dev: nstep consecutive canonical arrays U^(1) .. U^(nstep) (device, written).
  * 1 <= nstep <= 16, |rho| <= 0.5 (larger rho is refused: the series would cancel digits);
- * no aliasing between the two buffers; both 16-byte aligned.  Async on `stream`. */
+ * no aliasing between the two buffers; both 16-byte aligned.  Async on `stream`.
+ *
+ * Workspaces of smearing, its chain rule, the gauge action and the gauge force: for the time of the call, from a
+ * memory pool of the library's own, which keeps up to 8 GiB mapped between calls and gives it back when
+ * the last lattice is destroyed.  FP64 smearing takes 1.3 kB per site (none beyond 8 GiB of it).  Without
+ * room, and while `stream` captures, slower kernels run that need no such workspace; their results agree to
+ * rounding. */
 stg_status stg_stout_smear(const stg_lattice *lat, stg_prec prec, int32_t nstep, double rho, const void *links_dev,
                            void *levels_dev, void *stream);
 
@@ -367,8 +373,9 @@ stg_status stg_stout_smear(const stg_lattice *lat, stg_prec prec, int32_t nstep,
  * grad_dev: G_k; out_dev: kind 1: G_0 = dS/dRe U^(0) + i dS/dIm U^(0), kind 0:
  * F = TA(U^(0) G_0^dag) (dS/deps = tr(X F) along U^(0) -> exp(eps X) U^(0)).
  * All canonical [4][V][3][3] device arrays of prec (F64: complex128, F32: complex64); out must not
- * alias the inputs.  Allocates 2 link-sized work arrays from the stream-ordered allocator.  Same
- * limits as smearing. */
+ * alias the inputs.  Workspace: FP64 7.3 kB per site and one link-sized array more for nstep > 1 (up to
+ * 8 GiB in all), FP32 three link-sized arrays; beyond, without room and under capture two link-sized arrays
+ * from the device's default stream-ordered pool.  Same limits as smearing. */
 stg_status stg_stout_force(const stg_lattice *lat, stg_prec prec, int32_t nstep, double rho, const void *links_dev,
                            const void *levels_dev, const void *grad_dev, void *out_dev, int32_t kind, void *stream);
 
@@ -382,7 +389,8 @@ stg_status stg_stout_force(const stg_lattice *lat, stg_prec prec, int32_t nstep,
  * out3_dev (device, 3 doubles, written): S_g, the plaquette sum sum_{x, mu<nu} Re tr P (each
  * plaquette once) and the rectangle sum sum_{x, mu!=nu} Re tr R (each rectangle once).  The block
  * partial sums are added in a fixed order (bitwise reproducible).  FP64.  Allocates
- * 16 bytes per 128 sites from the stream-ordered allocator; async on `stream`. */
+ * 16 bytes per 128 sites from the stream-ordered allocator, and a workspace (see stg_stout_smear) of up to
+ * 4 GiB or 864 bytes per site, whichever is more; async on `stream`. */
 stg_status stg_gauge_action(const stg_lattice *lat, double beta, const void *links_c128_dev, double *out3_dev,
                             void *stream);
 
@@ -391,7 +399,8 @@ stg_status stg_gauge_action(const stg_lattice *lat, double beta, const void *lin
  * other direction), written as kind 1: G, or kind 0: F = TA(U G^dag) (dS/deps = tr(X F) along
  * U -> exp(eps X) U).  prec STG_F64: complex128 arrays, FP64; STG_F32: complex64 arrays, FP32 (the
  * single-precision MD, Sec. 5.4).  links_dev / out_dev: canonical [4][V][3][3] (device), no
- * aliasing.  Async on `stream`. */
+ * aliasing.  FP64 takes a workspace (see stg_stout_smear) of up to 4 GiB or 1152 bytes per site, whichever is
+ * more.  Async on `stream`. */
 stg_status stg_gauge_force(const stg_lattice *lat, stg_prec prec, double beta, const void *links_dev, void *out_dev,
                            int32_t kind, void *stream);
 

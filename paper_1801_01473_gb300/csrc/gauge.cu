@@ -333,27 +333,23 @@ bool misaligned(const void *p) { return p == nullptr || (reinterpret_cast<uintpt
 
 using namespace stg;
 
-// Workspace of the shared-staple force: as many planes per pass as fit kGaugeWorkspace (all 6 up to
-// 24^4 in FP64), at least one.  Returns false (nothing launched) when the pool has no room for even
-// one plane.
+// Workspace of the shared-staple force and action: as many planes per pass as fit kGaugeWorkspace (all 6 up to
+// 24^4 in the force), at least one (1152 bytes per site for the force, 864 for the action: 6.1 GB at 48^4).
 constexpr size_t kGaugeWorkspace = (size_t)4 << 30;
 
 // The planes per pass and the workspace of `fields` matrices per plane and site; false when there is
-// no room for one plane.
+// no room for one plane, and while st captures: the kernels that need none then do the work.
 template <typename C>
 static bool plaq_workspace(long long V, int fields, cudaStream_t st, int &np, C *&ws)
 {
     if (V > INT_MAX) return false;
     const size_t per_plane = (size_t)fields * 9 * V * sizeof(C);
     np = (int)std::min<size_t>(6, std::max<size_t>(1, kGaugeWorkspace / per_plane));
-    keep_pool_mapped(st);
-    cudaError_t e = cudaMallocAsync((void **)&ws, np * per_plane, st);
-    if (e != cudaSuccess && np > 1) {
-        cudaGetLastError();
+    cudaError_t e = link_workspace((void **)&ws, np * per_plane, st);
+    if (e == cudaErrorMemoryAllocation && np > 1) {
         np = 1;
-        e = cudaMallocAsync((void **)&ws, per_plane, st);
+        e = link_workspace((void **)&ws, per_plane, st);
     }
-    if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess;
 }
 

@@ -972,13 +972,23 @@ struct DevBuf {
     char *cur = nullptr;
     size_t left = 0;
     static constexpr size_t kChunk = (size_t)64 << 20, kAlign = 256;
+    cudaError_t pool_alloc(void **p, size_t bytes)
+    {
+        cudaError_t e = cudaMallocAsync(p, bytes, st);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            trim_link_pools();
+            e = cudaMallocAsync(p, bytes, st);
+        }
+        return e;
+    }
     void *alloc(size_t bytes)
     {
         if (err != cudaSuccess) return nullptr;
         bytes = (std::max<size_t>(bytes, 16) + kAlign - 1) & ~(kAlign - 1);
         if (bytes >= kChunk / 4) {  // large fields (residual rings) get pool blocks of their own
             void *p = nullptr;
-            err = cudaMallocAsync(&p, bytes, st);
+            err = pool_alloc(&p, bytes);
             if (err != cudaSuccess) return nullptr;
             ptrs.push_back(p);
             return p;
@@ -986,7 +996,7 @@ struct DevBuf {
         if (bytes > left) {
             const size_t want = std::max(bytes, kChunk);
             void *p = nullptr;
-            err = cudaMallocAsync(&p, want, st);
+            err = pool_alloc(&p, want);
             if (err != cudaSuccess) return nullptr;
             ptrs.push_back(p);
             cur = static_cast<char *>(p);
@@ -1105,7 +1115,18 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
         }
     const int vb = Field<R>::kBytesPerSite;
 
-    keep_pool_mapped(user_st);  // the workspace comes from the default stream-ordered pool
+    // The workspace comes from the device's default stream-ordered memory pool.  Keep up to
+    // 64 GiB of freed pool memory mapped between solves (the default threshold of 0 returns it at
+    // every synchronisation and the next solve pays for mapping it again).
+    {
+        int dev = 0;
+        cudaMemPool_t pool;
+        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
+            uint64_t thr = 64ull << 30;
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
+        }
+        cudaGetLastError();
+    }
     const bool verbose = getenv("STG_VERBOSE") && getenv("STG_VERBOSE")[0] == '1';
     auto t_start = std::chrono::steady_clock::now();
     auto stamp = [&](const char *what) {

@@ -60,10 +60,16 @@ stg_status f32_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge 
 // gauge): the operator of the mixed solver's FP64-accurate residuals, run on the FP32 pipes.
 stg_status ds_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge **out);
 
-// Sets the release threshold of the device's default stream-ordered memory pool to 64 GiB, so that
-// freed workspaces stay mapped between calls (the default threshold of 0 returns them at every
-// synchronisation and the next call pays for mapping them again).  Does nothing while `st` captures.
-void keep_pool_mapped(cudaStream_t st);
+// Workspace of a link operation (gauge force and action, smearing and its chain rule), freed with
+// cudaFreeAsync: from a pool of the library's own, one per device, which keeps at most 8 GiB mapped between
+// calls (with the default pool's threshold of 0 every call after a synchronisation maps its workspace again)
+// and gives everything back with the last lattice.  An error, and *p null, where there is no room, and while
+// `st` captures: a captured graph is left without memory nodes of that size.
+cudaError_t link_workspace(void **p, size_t bytes, cudaStream_t st);
+// Unused memory of those pools back to the device (for another allocation that found no room).
+void trim_link_pools();
+// Lattices alive; with the last one link_workspace's pools are emptied.
+void count_lattice(int change);
 
 // Canonical links -> F64 18-real links and their fixed-point copy with its two words of state (dslash_f64.cu)
 cudaError_t launch_pack_links_fx(const Geom &g, const void *canon, void *links, void *fx_links, int *state,

@@ -64,17 +64,69 @@ cudaError_t launch_dslash_bs(int kind, const DArgs &a, int mode, int bs, cudaStr
     return cudaErrorInvalidValue;
 }
 
-void keep_pool_mapped(cudaStream_t st)
+namespace {
+constexpr int kMaxPoolDevices = 64;
+constexpr uint64_t kLinkPoolKept = 8ull << 30;
+std::mutex g_link_pool_mu;
+cudaMemPool_t g_link_pool[kMaxPoolDevices];
+long long g_lattices = 0;
+
+void set_kept(cudaMemPool_t pool, uint64_t bytes)
 {
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &bytes);
+}
+}  // namespace
+
+cudaError_t link_workspace(void **p, size_t bytes, cudaStream_t st)
+{
+    *p = nullptr;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     int dev = 0;
-    cudaMemPool_t pool;
-    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-        cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
-        uint64_t thr = 64ull << 30;
-        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && dev >= kMaxPoolDevices) e = cudaErrorInvalidDevice;
+    cudaMemPool_t pool = nullptr;  // lives as long as the process
+    if (e == cudaSuccess) {
+        std::lock_guard<std::mutex> lk(g_link_pool_mu);
+        if (!g_link_pool[dev]) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            e = cudaMemPoolCreate(&g_link_pool[dev], &props);
+            if (e != cudaSuccess) g_link_pool[dev] = nullptr;
+        }
+        pool = g_link_pool[dev];
+        if (pool) set_kept(pool, kLinkPoolKept);
     }
+    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        *p = nullptr;
+    }
+    return e;
+}
+
+void trim_link_pools()
+{
+    std::lock_guard<std::mutex> lk(g_link_pool_mu);
+    for (cudaMemPool_t pool : g_link_pool)
+        if (pool) cudaMemPoolTrimTo(pool, 0);
     cudaGetLastError();
+}
+
+void count_lattice(int change)
+{
+    {
+        std::lock_guard<std::mutex> lk(g_link_pool_mu);
+        g_lattices += change;
+        if (g_lattices > 0) return;
+        // what is still in use on a stream goes at that stream's next synchronisation
+        for (cudaMemPool_t pool : g_link_pool)
+            if (pool) set_kept(pool, 0);
+    }
+    trim_link_pools();
 }
 
 bool pdl_enabled()
@@ -606,6 +658,7 @@ stg_status stg_lattice_create(const int32_t dims[4], int32_t t_antiperiodic, stg
     l->g.antiperiodic = t_antiperiodic ? 1 : 0;
     geom_init(l->g);
     l->V = V;
+    count_lattice(1);
     *out = l;
     return STG_OK;
 }
@@ -664,7 +717,12 @@ stg_status stg_slab_layout(const stg_lattice *lat, stg_prec vec_prec, int32_t *n
     return set_error(STG_ERR_ARG, "stg_slab_layout: vec_prec must be F64, DS or F32");
 }
 
-void stg_lattice_destroy(stg_lattice *lat) { delete lat; }
+void stg_lattice_destroy(stg_lattice *lat)
+{
+    if (!lat) return;
+    delete lat;
+    count_lattice(-1);
+}
 
 int64_t stg_lattice_sites(const stg_lattice *lat, int32_t parity)
 {
@@ -726,8 +784,9 @@ static stg_status gauge_create(const stg_lattice *lat, const void *links_c128_de
     g->scratch_count = (size_t)dslash_partials(lat->g.Vh);
     size_t fx = fx_copy_bytes(kind, lat->V, g->bytes);
     cudaError_t e = cudaMalloc(&g->links, g->bytes + fx);
-    if (e != cudaSuccess && fx) {  // no room for the copy
+    if (e != cudaSuccess) {  // no room, or none for the copy
         cudaGetLastError();
+        trim_link_pools();
         fx = 0;
         e = cudaMalloc(&g->links, g->bytes);
     }

@@ -433,8 +433,8 @@ stg_status check_common(const stg_lattice *lat, int nstep, double rho, const cha
 bool misaligned(const void *p) { return p == nullptr || (reinterpret_cast<uintptr_t>(p) & 15) != 0; }
 
 // Workspaces of the shared-plaquette steps: 1.3 kB (smearing) and 7.3 kB (chain rule) per site in
-// FP64.  Up to kStoutWorkspace they are taken from the pool; beyond, or when the pool has no room,
-// the per-link kernels above do the step.
+// FP64.  Beyond kStoutWorkspace, without room for them and while the stream captures, the per-link
+// kernels above do the step.
 constexpr size_t kStoutWorkspace = (size_t)8 << 30;
 
 // Bump allocation of [count] fields of 9 V entries
@@ -469,12 +469,8 @@ bool smear_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
     using C = typename C2<T>::type;
     const size_t bytes = (size_t)18 * 9 * lat->V * sizeof(T) + 4096;
     if (!use_plaq<T>(lat->V, bytes)) return false;
-    keep_pool_mapped(st);
     char *ws = nullptr, *w;
-    if (cudaMallocAsync((void **)&ws, bytes, st) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
+    if (link_workspace((void **)&ws, bytes, st) != cudaSuccess) return false;
     StoutPlaqArgs<T> a;
     memset(&a, 0, sizeof(a));
     a.g = link_geo(lat->g);
@@ -505,12 +501,8 @@ bool force_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
     const size_t bytes = (size_t)(22 * 9 + (36 + 4) * 18) * lat->V * sizeof(T) +
                          (nstep > 1 ? level * sizeof(C) : 0) + 4096;
     if (!use_plaq<T>(lat->V, bytes)) return false;
-    keep_pool_mapped(st);
     char *ws = nullptr, *w;
-    if (cudaMallocAsync((void **)&ws, bytes, st) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
+    if (link_workspace((void **)&ws, bytes, st) != cudaSuccess) return false;
     StoutPlaqArgs<T> a;
     memset(&a, 0, sizeof(a));
     a.g = link_geo(lat->g);
@@ -580,14 +572,9 @@ cudaError_t force_t(const LinkGeo &g, int nstep, double rho, const void *links, 
     a.rho = (T)rho;
     const size_t level = (size_t)4 * g.V * 9;
     C *ws = nullptr;
-    keep_pool_mapped(st);
-    bool soa = sizeof(T) == 4;
-    cudaError_t e = cudaMallocAsync((void **)&ws, (soa ? 3 : 2) * level * sizeof(C), st);
-    if (e != cudaSuccess && soa) {
-        cudaGetLastError();
-        soa = false;
-        e = cudaMallocAsync((void **)&ws, 2 * level * sizeof(C), st);
-    }
+    // without room, and while st captures, in the canonical form with two arrays of the default pool
+    const bool soa = sizeof(T) == 4 && link_workspace((void **)&ws, 3 * level * sizeof(C), st) == cudaSuccess;
+    cudaError_t e = soa ? cudaSuccess : cudaMallocAsync((void **)&ws, 2 * level * sizeof(C), st);
     if (e != cudaSuccess) return e;
     C *tmp = ws + level, *U = ws + 2 * level, *out = static_cast<C *>(out_v);
     a.Y = ws;
