@@ -691,11 +691,12 @@ __global__ void __launch_bounds__(kScalBlock) k_beta(SysScal *sc, const SysVecs 
 // On small lattices an iteration is six launches of a few microseconds each.  Here the vector kernels
 // take the scalar kernels' work along: every block sums the partials itself (the same fixed-order sum
 // in every block, as in k_alpha and k_beta) and keeps the coefficients it needs; one block per system
-// writes the scalars back.  Used while a launch is one wave of blocks with one item each and a sum
-// is at most kFusedPartials long; results are bitwise those of the separate kernels.  Mixed solve on
-// 8x6x8x6 2.95 -> 2.85 ms, 12^4 (324 partials) force evaluation 2.47 -> 2.39 ms; at 16^4 (1024 partials)
-// the sum in every block costs more than the launches (FP64 solve 12.8 against 14.7 ms).
-constexpr int kFusedPartials = 400;
+// writes the scalars back.  Results are bitwise those of the separate kernels.  Used while a launch is one
+// wave of blocks with one item each and the repeated sums are at most kFusedWork reads (blocks x partials, over
+// its systems), for either phase by itself.  Whole solves, separate -> fused: phase 1 of 4^4 to 10^4 (3140 reads)
+// 1 to 3 % faster (10^4 FP64 12 poles 4938 -> 4798 us), 10x10x12x12 (6525) 2 % slower; phase 2 of 8^4 with 10 pairs
+// (5120) 3395 -> 3377 us, 16 pairs (8192) 3529 -> 3557, 12^4 10 pairs 4356 -> 4574, FP16 5310 -> 5780.
+constexpr long long kFusedWork = 6000;
 
 // k_alpha + k_update_r
 template <typename R>
@@ -1415,11 +1416,11 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
     cudaGetLastError();
 
     // the fused iteration kernels, per phase: one wave of single-item blocks, short partial sums
-    bool fused1 = true, fused2 = true;
-    for (int q = 0; q < nsys; ++q) fused1 = fused1 && v1[q].npart_v <= kFusedPartials;
-    fused2 = fused1;
-    fused1 = fused1 && wl1.total <= (int)std::min(g_r1.x, hist_w > 0 ? g_pb.x : g_s1.x);
-    fused2 = fused2 && wl2.total <= (int)std::min(g_r2.x, g_s2.x);
+    long long reads1 = 0, reads2 = 0;
+    for (int q = 0; q < nsys; ++q) reads1 += (long long)v1[q].nblk_v * v1[q].npart_v;
+    for (int q = 0; q < npair; ++q) reads2 += (long long)v2[q].nblk_v * v2[q].npart_v;
+    const bool fused1 = reads1 <= kFusedWork && wl1.total <= (int)std::min(g_r1.x, hist_w > 0 ? g_pb.x : g_s1.x);
+    const bool fused2 = reads2 <= kFusedWork && wl2.total <= (int)std::min(g_r2.x, g_s2.x);
     const bool scal_wide = getenv("STG_SCALAR_BLOCK") && atoi(getenv("STG_SCALAR_BLOCK")) == 1024;
     auto iterate = [&](int kind, const DPlan &pl, SysScal *dS, SysVecs *dV, int *dn, int *nr, int n, dim3 /*vg*/,
                        double *log, int log_rows) -> cudaError_t {
