@@ -1312,12 +1312,17 @@ static stg_status solve_impl(int ninst, const stg_instance *inst, const stg_mscg
         }
     }
     // phase 2: the (rhs, shift) pairs of one instance share link loads, in groups of `rg`
-    // right-hand sides per thread (STG_REFINE_GROUP, 1..8).  Two by default while their groups fit one
-    // launch: groups share the links through L2 there, and two rhs per thread keep more warps in
-    // flight than four (whole solves, 4 -> 2 rhs: 32^4 16 poles 78.0 -> 73.9 ms, 20^4 14 poles 12.9 -> 12.5 ms,
-    // 16^4 6.84 -> 6.72 ms; 1 rhs 77.0, 8 rhs 80.2 ms at 32^4).  Larger batches would need more launches
-    // per iteration and stay at four.
-    int rg = npair <= 2 * kMaxGroups ? 2 : 4;
+    // right-hand sides per thread (STG_REFINE_GROUP, 1..8).  The groups of a launch (kMaxGroups) share the links
+    // through L2 anyway, and fewer right-hand sides per thread keep more warps in flight; more launches
+    // cost more than that on small lattices.  Whole solves, FP32 and FP16 inner links, 4 / 2 / 1 rhs:
+    //   12 pairs  8^4 FP16 3690 / 3840 / 3500 us, 12^4 FP32 4530 / 4530 / 4350, 18^4 FP16 10650 / 10340 / 10130,
+    //             20^4 FP16 13930 / 13170 / 13500, 24^4 (16 pairs) FP16 32900 / 29460 / 30190
+    //   20 pairs  8^4 FP16 3970 / 4130 / 4020, 12^4 FP16 6160 / 6290 / 6190, 16^4 FP16 9880 / 9720 / 10120
+    //   32 pairs  12^4 FP32 5470 / 5520 / 5810, 16^4 9800 / 9680 / 10220, 24^4 29930 / 29600 / 30470
+    // Beyond 32 pairs (two launches of pairs) groups of 4.
+    int max_vh = 0;
+    for (int k = 0; k < ninst; ++k) max_vh = std::max(max_vh, ii[k].gr->g.Vh);
+    int rg = npair <= kMaxGroups ? (max_vh <= 60000 ? 1 : 2) : npair <= 2 * kMaxGroups && max_vh > 16000 ? 2 : 4;
     if (const char *e = getenv("STG_REFINE_GROUP")) rg = std::max(1, std::min(kMaxRhs, atoi(e)));
     DPlan p2, p64, p64f;  // p64: residuals with gh; p64f: the same with the F64 gauge (verification)
     DPlan pinc;           // anchored refinement: r_hi = r_hi - A y_hi with gh
