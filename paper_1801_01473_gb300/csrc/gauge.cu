@@ -376,15 +376,16 @@ static bool gauge_force_plaq(const stg_lattice *lat, double beta, const void *li
     a.Slo = ws + 4 * np * field;
     a.Pb = ws + 6 * np * field;
     const unsigned nb = (unsigned)((a.g.V + kPlaqBlock - 1) / kPlaqBlock);
+    const bool ov = plaq::overlap(a.g.V, 24, 4, 8192);
     for (int p = 0; p < 6 && err == cudaSuccess; p += np) {
         a.p0 = p;
         a.p1 = std::min(6, p + np);
         a.first = p == 0;
         a.last = a.p1 == 6;
         const dim3 pairs(nb, 2 * (a.p1 - a.p0));
-        err = launch_pdl(k_gauge_staples<T>, pairs, dim3(kPlaqBlock), st, a);
-        if (err == cudaSuccess) err = launch_pdl(k_gauge_bent<T>, pairs, dim3(kPlaqBlock), st, a);
-        if (err == cudaSuccess) err = launch_pdl(k_gauge_gather<T>, dim3(nb, 4), dim3(kPlaqBlock), st, a);
+        err = launch_overlap(ov, k_gauge_staples<T>, pairs, dim3(kPlaqBlock), 0, st, a);
+        if (err == cudaSuccess) err = launch_overlap(ov, k_gauge_bent<T>, pairs, dim3(kPlaqBlock), 0, st, a);
+        if (err == cudaSuccess) err = launch_overlap(ov, k_gauge_gather<T>, dim3(nb, 4), dim3(kPlaqBlock), 0, st, a);
     }
     const cudaError_t f = cudaFreeAsync(ws, st);
     if (err == cudaSuccess) err = f;

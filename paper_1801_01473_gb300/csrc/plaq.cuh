@@ -11,7 +11,8 @@
 // the number of 3x3 products decides their time and the extra memory traffic does not show.
 #pragma once
 
-#include "dslash.cuh"  // launch_pdl
+#include "dslash.cuh"  // launch_overlap
+#include "stg_common.h"
 #include "su3.cuh"
 
 namespace stg {
@@ -96,11 +97,26 @@ __global__ void __launch_bounds__(kWsTile) k_links_to_ws(const typename C2<T>::t
         for (int k = 0; k < 9; ++k) dst[((long long)mu * 9 + k) * V + i0 + threadIdx.x] = tile[threadIdx.x * 9 + k];
 }
 
+// Whether the launches of a link operation may overlap (programmatic launch).  The blocks of the next kernel are
+// then placed while the running one holds its SMs: they gather on the SMs that it leaves idle, or are
+// stacked unevenly on top of it, and stay there.  That costs nothing while both kernels' warps find a quarter SM
+// each (`pair` warps per 32 sites for two consecutive launches, `fits` per SM) and little from `large` sites
+// up, where most blocks start later; between, plain launches are faster although each costs 2 to 3 us:
+//   FP64, overlapping -> plain, back to back calls: chain rule 576 sites 264 -> 250 us, 1296 426 -> 250, 3072 552 -> 264,
+//   6400 600 -> 473, 10000 731 -> 751; gauge force 256 sites 77 -> 83, 3072 169 -> 103, 6400 184 -> 162, 10000 275 ->
+//   280; smearing 256 89 -> 97, 3072 189 -> 101, 10000 306 -> 289, 20736 500 -> 483, 38416 789 -> 800.
+//   FP32 chain rule: 3072 44 -> 52, 4096 55 -> 50, 10000 78 -> 69, 20736 86 -> 93.
+inline bool overlap(long long V, int pair, int fits, long long large)
+{
+    return pair * ((V + 31) / 32) <= (long long)fits * sm_count() || V >= large;
+}
+
 template <typename T>
-cudaError_t links_to_ws(const void *links, typename C2<T>::type *ws, int V, cudaStream_t st)
+cudaError_t links_to_ws(bool overlap, const void *links, typename C2<T>::type *ws, int V, cudaStream_t st)
 {
     const dim3 tiles((unsigned)((V + kWsTile - 1) / kWsTile), 4);
-    return launch_pdl(k_links_to_ws<T>, tiles, dim3(kWsTile), st, static_cast<const typename C2<T>::type *>(links), ws, V);
+    return launch_overlap(overlap, k_links_to_ws<T>, tiles, dim3(kWsTile), 0, st,
+                          static_cast<const typename C2<T>::type *>(links), ws, V);
 }
 
 // acc += w a

@@ -60,6 +60,9 @@ stg_status f32_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge 
 // gauge): the operator of the mixed solver's FP64-accurate residuals, run on the FP32 pipes.
 stg_status ds_companion(const stg_gauge *g64, cudaStream_t st, const stg_gauge **out);
 
+// SMs of the current device (152 when it cannot be asked)
+int sm_count();
+
 // Workspace of a link operation (gauge force and action, smearing and its chain rule), freed with
 // cudaFreeAsync: from a pool of the library's own, one per device, which keeps at most 8 GiB mapped between
 // calls (with the default pool's threshold of 0 every call after a synchronisation maps its workspace again)

@@ -129,6 +129,14 @@ void count_lattice(int change)
     trim_link_pools();
 }
 
+int sm_count()
+{
+    int dev = 0, n = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        n = 152;
+    return n;
+}
+
 bool pdl_enabled()
 {
     static const bool on = [] {

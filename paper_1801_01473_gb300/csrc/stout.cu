@@ -456,9 +456,7 @@ template <typename T>
 bool use_plaq(long long V, size_t bytes)
 {
     if (sizeof(T) != 8 || V > INT_MAX || bytes > kStoutWorkspace) return false;
-    int dev = 0, nsm = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const long long warps = (V + 31) / 32;
+    const long long warps = (V + 31) / 32, nsm = sm_count();
     return 6 * warps <= 4 * nsm || 4 * warps > 4 * nsm;
 }
 
@@ -480,12 +478,13 @@ bool smear_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
     a.Lo = take<T>(w, a.g.V, 12);
     const size_t level = (size_t)4 * a.g.V * 9;
     const unsigned nb = (unsigned)((a.g.V + kStoutBlock - 1) / kStoutBlock);
+    const bool ov = overlap(a.g.V, 10, 4, 32768);
     err = cudaSuccess;
     for (int k = 0; k < nstep && err == cudaSuccess; ++k) {
         a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
         a.out = static_cast<C *>(levels) + (size_t)k * level;
-        err = launch_pdl(k_stout_loops<false, T>, dim3(nb, 6), dim3(kStoutBlock), st, a);
-        if (err == cudaSuccess) err = launch_pdl(k_stout_apply<T>, dim3(nb, 4), dim3(kStoutBlock), st, a);
+        err = launch_overlap(ov, k_stout_loops<false, T>, dim3(nb, 6), dim3(kStoutBlock), 0, st, a);
+        if (err == cudaSuccess) err = launch_overlap(ov, k_stout_apply<T>, dim3(nb, 4), dim3(kStoutBlock), 0, st, a);
     }
     const cudaError_t f = cudaFreeAsync(ws, st);
     if (err == cudaSuccess) err = f;
@@ -519,6 +518,7 @@ bool force_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
     C *out = static_cast<C *>(out_v);
     const unsigned nb = (unsigned)((a.g.V + kStoutBlock - 1) / kStoutBlock);
     const dim3 links4(nb, 4);
+    const bool ov = overlap(a.g.V, 16, 4, 8192);
     a.G = static_cast<const C *>(grad);
     err = cudaSuccess;
     for (int k = nstep - 1; k >= 0 && err == cudaSuccess; --k) {
@@ -526,10 +526,10 @@ bool force_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
         a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
         a.out = (k % 2 == 0) ? out : tmp;
         a.proj = k == 0 && kind == 0 ? static_cast<const C *>(links) : nullptr;
-        err = launch_pdl(k_stout_loops<true, T>, dim3(nb, 6), dim3(kStoutBlock), st, a);
-        if (err == cudaSuccess) err = launch_pdl(k_stout_grad_exp<T>, links4, dim3(kStoutBlock), st, a);
-        if (err == cudaSuccess) err = launch_pdl(k_stout_bent<T>, dim3(nb, 12), dim3(kStoutBlock), st, a);
-        if (err == cudaSuccess) err = launch_pdl(k_stout_gather<T>, links4, dim3(kStoutBlock), st, a);
+        err = launch_overlap(ov, k_stout_loops<true, T>, dim3(nb, 6), dim3(kStoutBlock), 0, st, a);
+        if (err == cudaSuccess) err = launch_overlap(ov, k_stout_grad_exp<T>, links4, dim3(kStoutBlock), 0, st, a);
+        if (err == cudaSuccess) err = launch_overlap(ov, k_stout_bent<T>, dim3(nb, 12), dim3(kStoutBlock), 0, st, a);
+        if (err == cudaSuccess) err = launch_overlap(ov, k_stout_gather<T>, links4, dim3(kStoutBlock), 0, st, a);
         a.G = a.out;
     }
     const cudaError_t f = cudaFreeAsync(ws, st);
@@ -552,10 +552,11 @@ cudaError_t smear_t(const LinkGeo &g, int nstep, double rho, const void *links, 
     a.rho = (T)rho;
     const size_t level = (size_t)4 * g.V * 9;  // complex numbers per level
     const dim3 grid((unsigned)((g.V + 31) / 32));  // 32 sites, one warp per direction
+    const bool ov = sizeof(T) == 4 || overlap(g.V, 8, 4, 32768);
     for (int k = 0; k < nstep; ++k) {
         a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
         a.out = static_cast<C *>(levels) + (size_t)k * level;
-        const cudaError_t e = launch_pdl(k_stout_fwd<T>, grid, dim3(kStoutBlock), st, a);
+        const cudaError_t e = launch_overlap(ov, k_stout_fwd<T>, grid, dim3(kStoutBlock), 0, st, a);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -579,6 +580,7 @@ cudaError_t force_t(const LinkGeo &g, int nstep, double rho, const void *links, 
     C *tmp = ws + level, *U = ws + 2 * level, *out = static_cast<C *>(out_v);
     a.Y = ws;
     const dim3 grid((unsigned)((g.V + 31) / 32)), block(kStoutBlock);  // 32 sites, one warp per direction
+    const bool ov = sizeof(T) == 4 ? overlap(g.V, 8, 6, 16384) : overlap(g.V, 8, 4, 8192);
     a.G = static_cast<const C *>(grad);
     a.g_canon = 1;
     for (int k = nstep - 1; k >= 0 && e == cudaSuccess; --k) {
@@ -588,13 +590,13 @@ cudaError_t force_t(const LinkGeo &g, int nstep, double rho, const void *links, 
         if constexpr (sizeof(T) == 4) {
             if (soa) {
                 // each link's G, own terms and result share one place of tmp; the last result goes to out
-                e = links_to_ws<T>(a.U, U, g.V, st);
+                e = links_to_ws<T>(ov, a.U, U, g.V, st);
                 a.Uws = U;
                 a.acc = tmp;
                 a.out = k == 0 ? out : tmp;
                 a.out_canon = k == 0;
-                if (e == cudaSuccess) e = launch_pdl(k_stout_back_link<true, T>, grid, block, st, a);
-                if (e == cudaSuccess) e = launch_pdl(k_stout_back_staples<true, T>, grid, block, st, a);
+                if (e == cudaSuccess) e = launch_overlap(ov, k_stout_back_link<true, T>, grid, block, 0, st, a);
+                if (e == cudaSuccess) e = launch_overlap(ov, k_stout_back_staples<true, T>, grid, block, 0, st, a);
                 a.g_canon = 0;
                 done = true;
             }
@@ -602,8 +604,8 @@ cudaError_t force_t(const LinkGeo &g, int nstep, double rho, const void *links, 
         if (!done) {
             // the last step (k = 0) lands in out; earlier ones alternate so that it does
             a.acc = a.out = (k % 2 == 0) ? out : tmp;
-            e = launch_pdl(k_stout_back_link<false, T>, grid, block, st, a);
-            if (e == cudaSuccess) e = launch_pdl(k_stout_back_staples<false, T>, grid, block, st, a);
+            e = launch_overlap(ov, k_stout_back_link<false, T>, grid, block, 0, st, a);
+            if (e == cudaSuccess) e = launch_overlap(ov, k_stout_back_staples<false, T>, grid, block, 0, st, a);
         }
         a.G = a.out;
     }
