@@ -19,7 +19,6 @@
 // Layout: canonical complex128 or complex64 [4][V][3][3] (site index x + Lx (y + Ly (z + Lz t))); one
 // thread per link.  FP64 steps mostly go by shared plaquettes (further down).
 #include <algorithm>
-#include <climits>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -446,18 +445,23 @@ E *take(char *&p, int V, int count)
     return r;
 }
 
-// Whether the steps go by shared plaquettes.  FP32 stays with the per-link kernels, which are not
-// bound by their products (32^4 chain rule: 2.8 ms against 5.1 ms shared).  In FP64 every warp has a
-// quarter SM's pipe to itself while a launch has no more warps than quarters; the one window where
-// the per-link kernels fit that once and the 6 planes of a site do not (3243 to 4864 sites on 152
-// SMs) is theirs: 8^4 smears in 191 us against 220 us, 6^4 (191 against 94) and 5120 sites (351
-// against 250) do not.
+// Whether the steps go by shared plaquettes: FP64 within the workspace.  FP32 stays with the per-link kernels,
+// which are not bound by their products (32^4 chain rule: 2.8 ms against 5.1 ms shared).
 template <typename T>
-bool use_plaq(long long V, size_t bytes)
+bool plaq_fits(size_t bytes)
 {
-    if (sizeof(T) != 8 || V > INT_MAX || bytes > kStoutWorkspace) return false;
-    const long long warps = (V + 31) / 32, nsm = sm_count();
-    return 6 * warps <= 4 * nsm || 4 * warps > 4 * nsm;
+    return sizeof(T) == 8 && bytes <= kStoutWorkspace;
+}
+
+// Smearing has one window of its own.  In FP64 every warp has a quarter SM's pipe to itself while a launch has
+// no more warps than quarters; where the per-link kernel fits that once and the 6 planes of a site do not
+// (3233 to 4864 sites on 152 SMs) it is faster: 8^4 130 us against 147 us, but 3072 sites 130 against 101, 5120
+// 238 against 171.  The chain rule has none, its per-link kernels do nearly twice the products: 8^4 437 us
+// against 329 us, 768 sites 426 against 250, 6400 812 against 472.
+inline bool smear_by_links(long long V)
+{
+    const long long warps = (V + 31) / 32, quarters = 4LL * sm_count();
+    return 6 * warps > quarters && 4 * warps <= quarters;
 }
 
 template <typename T>
@@ -466,7 +470,7 @@ bool smear_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
 {
     using C = typename C2<T>::type;
     const size_t bytes = (size_t)18 * 9 * lat->V * sizeof(T) + 4096;
-    if (!use_plaq<T>(lat->V, bytes)) return false;
+    if (!plaq_fits<T>(bytes) || smear_by_links(lat->V)) return false;
     char *ws = nullptr, *w;
     if (link_workspace((void **)&ws, bytes, st) != cudaSuccess) return false;
     StoutPlaqArgs<T> a;
@@ -499,7 +503,7 @@ bool force_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
     const size_t level = (size_t)4 * lat->V * 9;
     const size_t bytes = (size_t)(22 * 9 + (36 + 4) * 18) * lat->V * sizeof(T) +
                          (nstep > 1 ? level * sizeof(C) : 0) + 4096;
-    if (!use_plaq<T>(lat->V, bytes)) return false;
+    if (!plaq_fits<T>(bytes)) return false;
     char *ws = nullptr, *w;
     if (link_workspace((void **)&ws, bytes, st) != cudaSuccess) return false;
     StoutPlaqArgs<T> a;
