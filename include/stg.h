@@ -324,7 +324,7 @@ stg_status stg_mscg_solve_batched(int32_t ninst, const stg_instance *inst, const
  *           U -> exp(eps X) U, X in su(3)), or
  *   kind 1: W^dag = dS/dRe U + i dS/dIm U.
  * y_i is computed with a double-single (FP32-pair, 48-bit significand) copy of the links, which
- * the F64 gauge creates on first use and keeps; W and F are formed in double-single and widened.
+ * the F64 gauge creates on first use and keeps; W and U W are formed in double-single, TA(U W) in FP64.
  * x_c128_dev[nshift]: canonical complex128 even fields (device);
  * out_c128_dev: canonical complex128 [4][V][3][3] (device).  g_f64 must be an F64 gauge. */
 stg_status stg_fermion_force(const stg_gauge *g_f64, int32_t nshift, const double *residues,

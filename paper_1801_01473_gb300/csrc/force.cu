@@ -15,7 +15,7 @@
 // direction mu gathers its rank-nshift sum of outer products (no atomics: every link is owned by
 // exactly one thread) -- in double-single on the FP32 pipes (k_force_ds, the default: GB300 issues
 // FP64 at 1/64 of FP32, and the FP64 gather was FP64-pipe bound at ~94 %), or in FP64 (k_force,
-// with STG_FORCE_FP64=1).  F = TA(U W) is formed in double-single too, its 9 numbers then widened.
+// with STG_FORCE_FP64=1).  U W is formed in double-single too, its entries then widened for TA.
 #include <cstdlib>
 #include <cstring>
 #include <vector>
@@ -124,12 +124,14 @@ struct ForceArgsDS {
 
 // (double)(hi + lo), the widening on the integer pipes: one FP64 addition
 __device__ __forceinline__ double ds_to_f64(const dsf &v) { return f32_to_f64(v.hi) + f32_to_f64(v.lo); }
+__device__ __forceinline__ double half_to_f64(const dsf &v) { return ds_to_f64(dsf(0.5f * v.hi, 0.5f * v.lo)); }
 
-// Bound by the FP32 pipes (36 double-single multiply-adds of 15 operations per shift and link).  F by the
-// 9 numbers of its anti-Hermitian part, widened on the integer pipes, instead of the whole product
-// and TA in FP64: 9 FP64 operations per link instead of ~80, which had taken a third of the kernel.
-// Five blocks of 96 registers (128 without the bound: 3 % slower).  Force of 12 shifts, 24^3x32, kind 0:
-// 1196 -> 1049 us, kind 1 978 -> 970 us.
+// Bound by the FP32 pipes (36 double-single multiply-adds of 15 operations per shift and link).  F = TA(Z), Z = U W:
+// Z in double-single, where only the imaginary parts of its diagonal and its off-diagonal entries count,
+// widened on the integer pipes, and TA in FP64: ~35 FP64 operations per link (~80 when all of Z is converted).
+// The differences across Z and Z^dag in double-single too would take 9, but their rounding shows: 24^3x32,
+// 12 shifts, kind 0 1010 us instead of 1047 us, rms error 1.748e-14 instead of 1.740e-14.
+// Five blocks of 96 registers (128 without the bound: 3 % slower).  With all of Z converted 1196 us.
 template <typename LinkT>
 __global__ void __launch_bounds__(kForceBlock, 5) k_force_ds(const __grid_constant__ ForceArgsDS a)
 {
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(kForceBlock, 5) k_force_ds(const __grid_consta
                 for (int c = 0; c < 3; ++c) o[r * 3 + c] = make_double2((double)W[c][r].re, -(double)W[c][r].im);
             continue;
         }
-        // F = TA(U W), the SU(3) link in double-single: only the 9 numbers of the anti-Hermitian part
+        // F = TA(Z), Z = U W with the SU(3) link in double-single
         cx<dsf> U[3][3];
         LinkTraits<LinkT>::Base::load(blk, Vh, h, U);
         dsf d[3];
@@ -207,20 +209,13 @@ __global__ void __launch_bounds__(kForceBlock, 5) k_force_ds(const __grid_consta
 #pragma unroll
         for (int e = 0; e < 3; ++e) {  // (Z_rc - conj(Z_cr)) / 2
             const int r = e == 2 ? 1 : 0, c = e == 0 ? 1 : 2;
-            dsf re = dsf(0.f, 0.f), im = dsf(0.f, 0.f);
+            cx<dsf> z = cx<dsf>{dsf(0.f, 0.f), dsf(0.f, 0.f)}, w = z;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                re = fma(U[r][k].re, W[k][c].re, re);
-                re = fma(-U[r][k].im, W[k][c].im, re);
-                re = fma(-U[c][k].re, W[k][r].re, re);
-                re = fma(U[c][k].im, W[k][r].im, re);
-                im = fma(U[r][k].re, W[k][c].im, im);
-                im = fma(U[r][k].im, W[k][c].re, im);
-                im = fma(U[c][k].re, W[k][r].im, im);
-                im = fma(U[c][k].im, W[k][r].re, im);
-            }
+            for (int k = 0; k < 3; ++k) cmac(z, U[r][k], W[k][c]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) cmac(w, U[c][k], W[k][r]);
             // halving is exact
-            const double fr = ds_to_f64(dsf(0.5f * re.hi, 0.5f * re.lo)), fi = ds_to_f64(dsf(0.5f * im.hi, 0.5f * im.lo));
+            const double fr = half_to_f64(z.re) - half_to_f64(w.re), fi = half_to_f64(z.im) + half_to_f64(w.im);
             o[r * 3 + c] = make_double2(fr, fi);
             o[c * 3 + r] = make_double2(-fr, fi);
         }
