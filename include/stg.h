@@ -351,7 +351,8 @@ stg_status stg_fermion_force_prec(const stg_gauge *g_f64, stg_prec prec, int32_t
  * links_dev: canonical [4][V][3][3] U^(0) (device, read only);
  * levels_dev: nstep consecutive canonical arrays U^(1) .. U^(nstep) (device, written).
  * 1 <= nstep <= 16, |rho| <= 0.5 (larger rho is refused: the series would cancel digits);
- * no aliasing between the two buffers; both 16-byte aligned.  Async on `stream`.
+ * no aliasing between the two buffers; both 16-byte aligned.  Async on `stream`.  Smearing, its chain rule,
+ * the gauge action and the gauge force refuse a lattice of 2^31 sites (STG_ERR_SHAPE).
  *
  * Workspaces of smearing, its chain rule, the gauge action and the gauge force: for the time of the call, from a
  * memory pool of the library's own, which keeps up to 8 GiB mapped between calls and gives it back when

@@ -14,7 +14,6 @@
 // Canonical complex128 [4][V][3][3]; FP64 forces share their staples between links, FP32 ones are
 // one thread per link over its loops (84 complex 3x3 products).
 #include <algorithm>
-#include <climits>
 #include <cmath>
 #include <cstring>
 
@@ -342,7 +341,6 @@ constexpr size_t kGaugeWorkspace = (size_t)4 << 30;
 template <typename C>
 static bool plaq_workspace(long long V, int fields, cudaStream_t st, int &np, C *&ws)
 {
-    if (V > INT_MAX) return false;
     const size_t per_plane = (size_t)fields * 9 * V * sizeof(C);
     np = (int)std::min<size_t>(6, std::max<size_t>(1, kGaugeWorkspace / per_plane));
     cudaError_t e = link_workspace((void **)&ws, np * per_plane, st);
@@ -420,6 +418,7 @@ extern "C" stg_status stg_gauge_force(const stg_lattice *lat, stg_prec prec, dou
     if (lat && stg::geom_is_slab(lat->g))
         return stg::set_error(STG_ERR_SHAPE, "stg_gauge_force: not available on a slab lattice (stg_dslash* only)");
     if (!lat) return set_error(STG_ERR_ARG, "stg_gauge_force: null lattice");
+    if (lat->V > kMaxLinkSites) return set_error(STG_ERR_SHAPE, "stg_gauge_force: lattice of 2^31 sites");
     if (prec != STG_F64 && prec != STG_F32) return set_error(STG_ERR_ARG, "stg_gauge_force: prec must be F64 or F32");
     if (misaligned(links_dev) || misaligned(out_dev))
         return set_error(STG_ERR_ARG, "stg_gauge_force: buffers must be non-null and 16-byte aligned");
@@ -438,6 +437,7 @@ extern "C" stg_status stg_gauge_action(const stg_lattice *lat, double beta, cons
     if (lat && stg::geom_is_slab(lat->g))
         return stg::set_error(STG_ERR_SHAPE, "stg_gauge_action: not available on a slab lattice (stg_dslash* only)");
     if (!lat) return set_error(STG_ERR_ARG, "stg_gauge_action: null lattice");
+    if (lat->V > kMaxLinkSites) return set_error(STG_ERR_SHAPE, "stg_gauge_action: lattice of 2^31 sites");
     if (misaligned(links_c128_dev)) return set_error(STG_ERR_ARG, "stg_gauge_action: links must be non-null and 16-byte aligned");
     if (!out3_dev || (reinterpret_cast<uintptr_t>(out3_dev) & 7))
         return set_error(STG_ERR_ARG, "stg_gauge_action: out3 must be non-null and 8-byte aligned");

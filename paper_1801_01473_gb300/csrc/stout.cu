@@ -424,6 +424,7 @@ stg_status check_common(const stg_lattice *lat, int nstep, double rho, const cha
 {
     const std::string f(fn);
     if (!lat) return set_error(STG_ERR_ARG, f + ": null lattice");
+    if (lat->V > kMaxLinkSites) return set_error(STG_ERR_SHAPE, f + ": lattice of 2^31 sites");
     if (nstep < 1 || nstep > 16) return set_error(STG_ERR_ARG, f + ": nstep must be in 1..16");
     if (!(fabs(rho) <= 0.5)) return set_error(STG_ERR_ARG, f + ": |rho| must be <= 0.5");
     return STG_OK;

@@ -34,6 +34,10 @@ struct LinkGeo {
     FastDiv by_stride[4], by_L[4];
 };
 
+// Site numbers are 32 bits: 2^31 sites, which a lattice may have, are refused by the link operations (their
+// FP32 links alone would take 618 GB).
+constexpr long long kMaxLinkSites = 0x7fffffffLL;
+
 inline LinkGeo link_geo(const Geom &geo)
 {
     LinkGeo g;
