@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kWsTile) k_links_to_ws(const typename C2<T>::t
 // up, where most blocks start later; between, plain launches are faster although each costs 2 to 3 us:
 //   FP64, overlapping -> plain, back to back calls: chain rule 576 sites 264 -> 250 us, 1296 426 -> 250, 3072 552 -> 264,
 //   6400 600 -> 473, 10000 731 -> 751; gauge force 256 sites 77 -> 83, 3072 169 -> 103, 6400 184 -> 162, 10000 275 ->
-//   280; smearing 256 89 -> 97, 3072 189 -> 101, 10000 306 -> 289, 20736 500 -> 483, 38416 789 -> 800.
+//   280; smearing 256 89 -> 97, 3072 189 -> 101, 10000 306 -> 289, 20736 500 -> 483, 32256 664 -> 674.
 //   FP32 chain rule: 3072 44 -> 52, 4096 55 -> 50, 10000 78 -> 69, 20736 86 -> 93.
 inline bool overlap(long long V, int pair, int fits, long long large)
 {

@@ -483,7 +483,7 @@ bool smear_plaq(const stg_lattice *lat, int nstep, double rho, const void *links
     a.Lo = take<T>(w, a.g.V, 12);
     const size_t level = (size_t)4 * a.g.V * 9;
     const unsigned nb = (unsigned)((a.g.V + kStoutBlock - 1) / kStoutBlock);
-    const bool ov = overlap(a.g.V, 10, 4, 32768);
+    const bool ov = overlap(a.g.V, 10, 4, 26000);
     err = cudaSuccess;
     for (int k = 0; k < nstep && err == cudaSuccess; ++k) {
         a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
@@ -557,7 +557,7 @@ cudaError_t smear_t(const LinkGeo &g, int nstep, double rho, const void *links, 
     a.rho = (T)rho;
     const size_t level = (size_t)4 * g.V * 9;  // complex numbers per level
     const dim3 grid((unsigned)((g.V + 31) / 32));  // 32 sites, one warp per direction
-    const bool ov = sizeof(T) == 4 || overlap(g.V, 8, 4, 32768);
+    const bool ov = sizeof(T) == 4 || overlap(g.V, 8, 4, 26000);
     for (int k = 0; k < nstep; ++k) {
         a.U = k == 0 ? static_cast<const C *>(links) : static_cast<const C *>(levels) + (size_t)(k - 1) * level;
         a.out = static_cast<C *>(levels) + (size_t)k * level;
