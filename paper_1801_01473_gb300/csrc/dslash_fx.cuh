@@ -371,10 +371,10 @@ __global__ void __launch_bounds__(BS, (BS == 64 ? 512 : 640) / BS) k_dslash_fx(c
 // Small lattices (up to kFxSplitVh sites per parity): a block covers 64 output sites with four threads
 // each.  Thread (mu, site) does the two hops of one direction, so that every load of a site is in
 // flight at once and few sites fill the chip; the four partial sums meet in shared memory in the unit
-// of the largest neighbour.  One right-hand side, against one thread per site: 12^4 13.6 -> 9.2 us, 16^4
-// 22.5 -> 14.0 us, 20^4 34.7 -> 30.1 us, but 24^4 56.4 -> 57.3 us (normal operator 122 -> 128 us) and 32^4
-// 151 -> 168 us, where the exchange costs more than the parallelism gives.  The choice depends on
-// the lattice alone, so that results do not depend on what else a launch carries.
+// of the largest neighbour.  Back to back, one thread per site -> four: D 8^4 11.5 -> 6.0 us, 12^4 12.5 -> 10.3, 16^4 20.7
+// -> 14.0, 20^4 34.1 -> 30.1, but 24^4 57.5 -> 59.9 (normal operator 123 -> 130 us) and 32^4 155 -> 165, where the
+// exchange costs more than the parallelism gives.  The choice depends on the lattice alone, so that
+// results do not depend on what else a launch carries.
 constexpr int kFxSites = 64;
 constexpr int kFxSplitVh = 90000;
 

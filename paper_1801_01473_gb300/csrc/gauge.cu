@@ -154,7 +154,8 @@ __global__ void __launch_bounds__(kGaugeBlock, 2) k_gauge_force(const __grid_con
 // one by one take 84 (k_gauge_force), for 4 matrices of workspace per pair and site.
 // Bound by the FP64 pipe: 18x22x14x26 8.73 -> 3.02 ms (2970 multiply-adds per link at 0.57e12/s),
 // 24^4 20.0 -> 6.93 ms, 4^4 317 -> 77 us.  One warp per block: the pipe is per quarter SM and one warp
-// keeps it busy, so small lattices spread best in single warps (6^4: 98 us against 123 us with four).
+// keeps it busy, so small lattices spread best in single warps (6^4, overlapping launches: 98 us against 123 us
+// with four; launched plainly, as it is now, 86 us).
 constexpr int kPlaqBlock = 32;
 
 template <typename T>
