@@ -97,3 +97,16 @@ def test_sizes_over_many_decades(dims, kind):
     point = np.zeros_like(psi)
     point[3, 1] = 1.0
     _check(dims, u, point)
+
+
+@pytest.mark.parametrize("dims", [SMALL, LARGE])
+@pytest.mark.parametrize("part", [1.0, 1j, (1 + 1j) / 2])
+def test_largest_sums(dims, part):
+    """The largest links that have a fixed-point form (rows and columns of 2.49) and vectors of the largest numbers
+    below a power of two with random signs, so that at many sites all 48 products add up: nothing overflows."""
+    rng = np.random.default_rng(200)
+    u = np.full((4, int(np.prod(dims)), 3, 3), 2.49 / 3 * part, np.complex128)
+    u[:, 0] = S.gauge_links((2, 2, 2, 2), "haar", 200)[:, 0]  # the unit is the first link's
+    sign = rng.choice([-1.0, 1.0], size=(2, int(np.prod(dims)) // 2))
+    psi = (np.nextafter(2.0, 0.0) * (sign[0] + 1j * sign[1]))[:, None] * np.ones(3)
+    _check(dims, u, psi)

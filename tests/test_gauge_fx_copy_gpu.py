@@ -82,7 +82,8 @@ def test_batch_with_lattices_without_a_copy(others):
     insts = []
     for k, dims in enumerate([DIMS] + others):
         u = _gpu(S.gauge_links(dims, "expih", 211 + k))
-        insts.append((p.Gauge(p.Lattice(dims), u, "f64", 18), None, [_gpu(S.gaussian_field(dims, 215 + k + 3 * j)) for j in range(2)]))
+        bs = [_gpu(S.gaussian_field(dims, 215 + k + 3 * j)) for j in range(2)]
+        insts.append((p.Gauge(p.Lattice(dims), u, "f64", 18), None, bs))
     both = p.mscg_batched(insts, [0.01, 0.5], 0.3, tol=1e-10)
     for (g, _, bs), (x, _) in zip(insts, both):
         for b, xb in zip(bs, x):
